@@ -134,7 +134,7 @@ CLASS_NAMES = ["residual_fp64", "residual_fp32", "dht_rows_fp64", "dht_rows_fp32
 
 
 def algorithmic_bytes_per_cell(cls, order):
-    w = 8 if cls.endswith("fp64") or cls.endswith("_ff") else 4  # float-float passes keep FP64 storage
+    w = 8 if cls.endswith("fp64") or cls.endswith("_ff") else 4  # the outer passes are FP64
     fp32 = cls.endswith("fp32")
     table = {
         # inner (order 6): delta, d, ubase in; delta', r out.  FP64 plain: u, d, f in; u', r out

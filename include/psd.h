@@ -243,15 +243,15 @@ psd_status psd_spfc_steps(psd_handle h, double* u, double gamma1, int nsteps,
 psd_status psd_residual_fixed(psd_handle h, const double* u, const double* f,
                               double* r, int* scale);
 
-/* The float-float transform passes of the mixed sixth-order solver's outer
- * loop, for tests: theta += H[T_h x], with H the unnormalised separable
- * discrete Hartley transform (kernel prod_a cas(2 pi j_a k_a / n_a), which
+/* The FP64 transform passes of the mixed sixth-order solver's outer loop,
+ * for tests: theta += H[T_h x], with H the unnormalised separable discrete
+ * Hartley transform (kernel prod_a cas(2 pi j_a k_a / n_a), which
  * diagonalises the symbols of Sec. 5.1 like the DFT of Sec. 6 does) and
  * T_h = -Delta_h^{-1} on the mean-zero space (Sec. 5.1; the zero mode
- * gives 0), computed in double-word arithmetic (about 48 significant bits)
- * on FP64 storage.  x, theta: device, N doubles each, must not alias; the
- * handle's direction buffer is used as scratch.  Synchronises the stream.
- * Errors: PSD_ERR_INVALID for null pointers.                               */
+ * gives 0), computed in 64-bit block fixed point on FP64 storage.  x, theta:
+ * device, N doubles each, must not alias; the handle's direction buffer is
+ * used as scratch.  Synchronises the stream.  Errors: PSD_ERR_INVALID for
+ * null pointers.                                                           */
 psd_status psd_theta_ff(psd_handle h, const double* x, double* theta);
 
 /* Autotuner (not in the paper): choose the tile widths -- line pairs per
@@ -273,7 +273,7 @@ enum {
   PSD_PROF_MID_FP64 = 6,      PSD_PROF_MID_FP32 = 7,
   PSD_PROF_LINESEARCH_FP64 = 8, PSD_PROF_LINESEARCH_FP32 = 9,
   PSD_PROF_OTHER = 10,
-  PSD_PROF_DHT_ROWS_FF = 11,  PSD_PROF_DHT_COLS_FF = 12,  /* float-float passes */
+  PSD_PROF_DHT_ROWS_FF = 11,  PSD_PROF_DHT_COLS_FF = 12,  /* mixed solve: outer passes */
   PSD_PROF_CLASSES = 13
 };
 

@@ -282,7 +282,7 @@ def psd_residual_fixed(handle, u, f, r):
 
 
 def psd_theta_ff(handle, x, theta):
-    """theta += H[T_h x] by the float-float transform passes (see include/psd.h)."""
+    """theta += H[T_h x] by the FP64 transform passes (see include/psd.h)."""
     _check(load_library().psd_theta_ff(handle, _ptr(x), _ptr(theta)), handle)
 
 

@@ -3,8 +3,8 @@
 // pass that divides by the symbol of L_h (Sec. 5.3, 5.4) and forms the
 // Parseval sums the line search needs.
 //
-// Shared by the translation units k_dht_f32.cu, k_dht_f64.cu and
-// k_dht_ff.cu, each of which instantiates one arithmetic type.
+// FP32 passes (the mixed solver's inner iteration), and the bookkeeping and
+// spectral helpers they share with the FP64 passes of dht_fx.cuh.
 #pragma once
 
 #include <algorithm>
@@ -23,51 +23,6 @@ template <>
 struct Vec2<float> {
   using type = float2;
 };
-template <>
-struct Vec2<double> {
-  using type = double2;
-};
-struct __align__(16) ff2 {
-  ff x, y;
-};
-template <>
-struct Vec2<ff> {
-  using type = ff2;
-};
-
-// x * scale, skipping the (double-word) product when scale is 1
-template <typename T>
-__device__ __forceinline__ T scaled(T x, T scale) {
-  return x * scale;
-}
-template <>
-__device__ __forceinline__ ff scaled<ff>(ff x, ff scale) {
-  return (scale.hi == 1.0f && scale.lo == 0.0f) ? x : x * scale;
-}
-
-// Storage <-> compute element conversions (FP32, FP64, or float-float on
-// FP64 storage).
-template <typename C, typename S>
-__device__ __forceinline__ C to_compute(S v) {
-  return C(v);
-}
-template <typename S, typename C>
-__device__ __forceinline__ S to_storage(C v) {
-  return S(v);
-}
-template <>
-__device__ __forceinline__ ff to_compute<ff, double>(double v) {
-  return ff_from_double_bits(v);
-}
-template <>
-__device__ __forceinline__ ff to_compute<ff, float>(float v) {
-  return ff(v, 0.0f);
-}
-template <>
-__device__ __forceinline__ double to_storage<double, ff>(ff v) {
-  return ff_to_double_bits(v);
-}
-
 constexpr int kThreads = 256;
 
 // Elements between the real arrays of consecutive line pairs in shared
@@ -102,10 +57,9 @@ constexpr size_t kMaxSmemPre = 200 * 1024;   // with the prefetch buffers of the
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
 // -------------------------------------------------------------- x (rows)
-// S: element type in memory (SI of the source); T: arithmetic type.
-template <typename S, typename T, int N, int RM, typename SI = S>
+template <typename T, int N, int RM>
 __global__ void __launch_bounds__(kThreads)
-    k_dht_rows(const SI* src, S* dst, int nrows, T scale, const int* done, const T* __restrict__ twc,
+    k_dht_rows(const T* src, T* dst, int nrows, T scale, const int* done, const T* __restrict__ twc,
                const T* __restrict__ tws) {
   using F = LineFFT<T, N, RM>;
   if (done != nullptr && *done) return;
@@ -120,11 +74,11 @@ __global__ void __launch_bounds__(kThreads)
   T* sr = sm + (size_t)p * 2 * LS;
   T* si = sr + LS;
   T vr[F::R], vi[F::R];
-  const SI* s0 = src + (size_t)row0 * N;
+  const T* s0 = src + (size_t)row0 * N;
 #pragma unroll
   for (int q = 0; q < F::R; ++q) {
-    vr[q] = valid ? to_compute<T>(s0[j + q * F::TS]) : T(0);
-    vi[q] = valid ? to_compute<T>(s0[N + j + q * F::TS]) : T(0);
+    vr[q] = valid ? s0[j + q * F::TS] : T(0);
+    vi[q] = valid ? s0[N + j + q * F::TS] : T(0);
   }
   if constexpr (F::TS <= 32) {
     // a line's team is TS consecutive lanes: the last pass ends in registers
@@ -133,25 +87,25 @@ __global__ void __launch_bounds__(kThreads)
     T h1[F::R], h2[F::R];
     dht_split_regs<T, N, F::R, F::TS>(vr, vi, j, h1, h2);
     if (valid) {
-      S* d0 = dst + (size_t)row0 * N;
+      T* d0 = dst + (size_t)row0 * N;
 #pragma unroll
       for (int q = 0; q < F::R; ++q) {
         const int k = j + q * F::TS;
-        d0[k] = to_storage<S>(scaled(h1[q], scale));
-        d0[N + k] = to_storage<S>(scaled(h2[q], scale));
+        d0[k] = h1[q] * scale;
+        d0[N + k] = h2[q] * scale;
       }
     }
   } else {
     F::run(vr, vi, j, sr, si, twc, tws);
     if (valid) {
-      S* d0 = dst + (size_t)row0 * N;
+      T* d0 = dst + (size_t)row0 * N;
 #pragma unroll
       for (int q = 0; q < F::R; ++q) {
         const int k = j + q * F::TS;
         T h1, h2;
         dht_split(sr, si, k, N, h1, h2);
-        d0[k] = to_storage<S>(scaled(h1, scale));
-        d0[N + k] = to_storage<S>(scaled(h2, scale));
+        d0[k] = h1 * scale;
+        d0[N + k] = h2 * scale;
       }
     }
   }
@@ -161,12 +115,12 @@ __global__ void __launch_bounds__(kThreads)
 // Block: `pairs` pairs of adjacent x-columns (x, x+1) packed as re/im, lines
 // along the strided axis; thread (p, j) = (tid % pairs, tid / pairs) so that a
 // warp reads whole row segments.
-template <typename S, typename T, int N, int RM>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 || std::is_same<T, ff>::value ? 3 : 1)  // FP32 / float-float: 80 registers
-    k_dht_cols(S* data, size_t line_stride, size_t outer_stride, T scale, const int* done,
+template <typename T, int N, int RM>
+__global__ void __launch_bounds__(kThreads, 3)  // 80 registers
+    k_dht_cols(T* data, size_t line_stride, size_t outer_stride, T scale, const int* done,
                const T* __restrict__ twc, const T* __restrict__ tws) {
   using F = LineFFT<T, N, RM>;
-  using V = typename Vec2<S>::type;
+  using V = typename Vec2<T>::type;
   if (done != nullptr && *done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
@@ -181,8 +135,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 || std::is_same<T, ff
 #pragma unroll
   for (int q = 0; q < F::R; ++q) {
     const V v = *reinterpret_cast<const V*>(data + base + (size_t)(j + q * F::TS) * line_stride);
-    vr[q] = to_compute<T>(v.x);
-    vi[q] = to_compute<T>(v.y);
+    vr[q] = v.x;
+    vi[q] = v.y;
   }
   F::run(vr, vi, j, sr, si, twc, tws);
 #pragma unroll
@@ -191,102 +145,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 || std::is_same<T, ff
     T h1, h2;
     dht_split(sr, si, k, N, h1, h2);
     V o;
-    o.x = to_storage<S>(scaled(h1, scale));
-    o.y = to_storage<S>(scaled(h2, scale));
+    o.x = h1 * scale;
+    o.y = h2 * scale;
     *reinterpret_cast<V*>(data + base + (size_t)k * line_stride) = o;
-  }
-}
-
-// ------------------------------------ last axis, float-float, fused epilogue
-// The last 1D DHT (z in 3D, y in 2D) of FP64 lines in float-float
-// arithmetic; the transformed values h are not stored but consumed:
-//   EPI_THETA:  theta += h / mu            (theta = DHT(T_h v) accumulates)
-//   EPI_RESID:  out32 = h - theta (FP32), and sum of (h - theta)^2 into
-//               ctrl->res_l2 = (h^d / N sum)^{1/2} (Parseval)
-// with mu the symbol of -Delta_h at the element; the zero mode gives 0
-// (mean-zero projection).  Same thread mapping as k_dht_cols.
-enum { EPI_THETA = 0, EPI_RESID = 1 };
-template <int N, int RM, int EPI>
-__global__ void __launch_bounds__(kThreads, 3)  // 80 registers, 3 CTAs per SM
-    k_dht_last_ff(const ff* data, double* theta, float* out32, size_t line_stride, size_t outer_stride,
-                  KParams kp, Ctrl* ctrl, double* partials, const ff* __restrict__ twc,
-                  const ff* __restrict__ tws, const ff* __restrict__ symx, const ff* __restrict__ symo,
-                  const ff* __restrict__ syml, double* dc, const int* skip) {
-  using T = ff;
-  using F = LineFFT<T, N, RM>;
-  if (skip != nullptr && *skip) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sm = reinterpret_cast<T*>(smem_raw);
-  __shared__ float sred[32];
-  __shared__ int sflag;
-  const int tid = threadIdx.x;
-  const int pairs = blockDim.x / F::TS;
-  const int p = tid % pairs, j = tid / pairs;
-  const int x = blockIdx.x * 2 * pairs + 2 * p;
-  const size_t base = (size_t)blockIdx.y * outer_stride + x;
-  constexpr int LS = line_stride_words<T, N, RM, false>();
-  T* sr = sm + (size_t)p * 2 * LS;
-  T* si = sr + LS;
-  // theta of this thread's elements, copied asynchronously while the
-  // forward transform runs: [q][j][p] double2
-  double2* pre = reinterpret_cast<double2*>(smem_raw + align16((size_t)pairs * 2 * LS * sizeof(T)));
-  T vr[F::R], vi[F::R];
-#pragma unroll
-  for (int q = 0; q < F::R; ++q) {
-    const size_t idx = base + (size_t)(j + q * F::TS) * line_stride;
-    const ff2 v = *reinterpret_cast<const ff2*>(data + idx);
-    cp_async_16(pre + ((size_t)(q * F::TS + j) * pairs + p), theta + idx);
-    vr[q] = v.x;
-    vi[q] = v.y;
-  }
-  F::run(vr, vi, j, sr, si, twc, tws);
-  cp_async_wait_all();
-  const ff mo = symo != nullptr ? ld_tw(symo + blockIdx.y) : ff(0.0f, 0.0f);
-  const ff mx[2] = {ff_add(ld_tw(symx + x), mo), ff_add(ld_tw(symx + x + 1), mo)};
-  float acc = 0.0f;
-#pragma unroll
-  for (int q = 0; q < F::R; ++q) {
-    const int k = j + q * F::TS;
-    T h[2];
-    dht_split(sr, si, k, N, h[0], h[1]);
-    const ff ml = ld_tw(syml + k);
-    const size_t idx = base + (size_t)k * line_stride;
-    const double2 th = pre[(size_t)(q * F::TS + j) * pairs + p];
-    const double thv[2] = {th.x, th.y};
-    double outv[2];
-    float o32[2];
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const ff mu = ff_add(mx[c], ml);
-      const bool live = mu.hi > 0.0f;
-      if (EPI == EPI_THETA) {
-        if (dc != nullptr && c == 0 && x == 0 && blockIdx.y == 0 && k == 0) *dc = ff_to_double_bits(h[0]);
-        const ff t = live ? ff_mul(h[c], ff_recip(mu)) : ff(0.0f, 0.0f);
-        outv[c] = ff_to_double_bits(ff_add(ff_from_double_bits(thv[c]), t));
-      } else {
-        const ff w = live ? ff_sub(h[c], ff_from_double_bits(thv[c])) : ff(0.0f, 0.0f);
-        o32[c] = w.hi;
-        acc = fmaf(w.hi, w.hi, acc);
-      }
-    }
-    if (EPI == EPI_THETA) {
-      *reinterpret_cast<double2*>(theta + idx) = make_double2(outv[0], outv[1]);
-    } else {
-      *reinterpret_cast<float2*>(out32 + idx) = make_float2(o32[0], o32[1]);
-    }
-  }
-  if (EPI == EPI_RESID) {
-    float v[1] = {acc};
-    block_reduce<float, 1, false>(v, sred);
-    if (publish_and_check_last<float>(v, 1, reinterpret_cast<float*>(partials), &ctrl->counter[CS_MID], &sflag)) {
-      float tt[1];
-      gather_partials<float, 1, false>(tt, reinterpret_cast<const float*>(partials), sred);
-      if (tid == 0) {
-        ctrl->res_l2 = sqrt((double)tt[0] * kp.hd * kp.inv_ntot);
-        ctrl->res_linf = -1.0;
-        ctrl->counter[CS_MID] = 0;
-      }
-    }
   }
 }
 
@@ -377,15 +238,13 @@ __device__ __forceinline__ void mid_finish(T (&acc)[5], T* sred, double* partial
 
 // ------------------------------------------------------------- middle pass
 // Tiles of 2 * pairs x-columns at one outer index (y in 3D), lines along the
-// last axis.  PERSIST (the FP32 passes of the inner iteration): a grid of a
-// few CTAs per SM loops over the tiles, and every thread prefetches, with
-// cp.async into shared memory, its own elements of the next tile's data and
-// of the current tile's xi / dspec, so that loads stay in flight while the
-// transforms of the current tile run (no barrier is needed for the staged
-// data: each thread reads only what it copied).  Otherwise one tile per CTA
-// with direct loads.
-template <typename T, int N, int ORDER, int RM, bool PERSIST>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && ORDER == 4 && !PERSIST ? 3 : 2)
+// last axis.  A grid of a few CTAs per SM loops over the tiles, and every
+// thread prefetches, with cp.async into shared memory, its own elements of
+// the next tile's data and of the current tile's xi / dspec, so that loads
+// stay in flight while the transforms of the current tile run (no barrier is
+// needed for the staged data: each thread reads only what it copied).
+template <typename T, int N, int ORDER, int RM>
+__global__ void __launch_bounds__(kThreads, 2)
     k_mid(T* data, unsigned line_stride, unsigned outer_stride, int ntx, int ntiles, KParams kp, Ctrl* ctrl,
           double* partials, T* xi, T* dspec, const T* __restrict__ symx, const T* __restrict__ symo,
           const T* __restrict__ syml, const T* __restrict__ twc, const T* __restrict__ tws) {
@@ -403,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && ORDER == 4 && !PER
   T* sr = sm + (size_t)p * 2 * LS;
   T* si = sr + LS;
   // staging ([q][j][p] pairs of columns): order 6 xi and dspec of the
-  // current tile, then (PERSIST) two buffers of the data
+  // current tile, then two buffers of the data
   V* pre_x = reinterpret_cast<V*>(smem_raw + align16((size_t)pairs * 2 * LS * sizeof(T)));
   V* pre_d = pre_x + (size_t)N * pairs;
   V* pre_w = pre_x + (ORDER == 6 ? 2 : 0) * (size_t)N * pairs;
@@ -430,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && ORDER == 4 && !PER
   const T s = C.s, se2 = C.se2, sl = C.sl;
   const T alpha_prev = (ORDER == 6) ? (T)ctrl->alpha : T(0);
   T acc[5] = {T(0), T(0), T(0), T(0), T(0)};
-  if (PERSIST && (int)blockIdx.x < ntiles) {
+  if ((int)blockIdx.x < ntiles) {
     const unsigned b0 = tile_base(blockIdx.x);
 #pragma unroll
     for (int q = 0; q < F::R; ++q) copy_vec(pre_w + elem(q), data + (b0 + goff(q)));
@@ -452,41 +311,27 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && ORDER == 4 && !PER
       cp_async_commit();
     }
     T vr[F::R], vi[F::R];
-    if (PERSIST) {
-      const int tn = t + gridDim.x;
-      if (tn < ntiles) {
-        const unsigned bn = tile_base(tn);
-        V* wnx = pre_w + (unsigned)((it + 1) & 1) * N * pairs;
+    const int tn = t + gridDim.x;
+    if (tn < ntiles) {
+      const unsigned bn = tile_base(tn);
+      V* wnx = pre_w + (unsigned)((it + 1) & 1) * N * pairs;
 #pragma unroll
-        for (int q = 0; q < F::R; ++q) copy_vec(wnx + elem(q), data + (bn + goff(q)));
-      }
-      cp_async_commit();
-      // this tile's data is the oldest group in flight
-      if (ORDER == 6)
-        cp_async_wait_group<2>();
-      else
-        cp_async_wait_group<1>();
+      for (int q = 0; q < F::R; ++q) copy_vec(wnx + elem(q), data + (bn + goff(q)));
+    }
+    cp_async_commit();
+    // this tile's data is the oldest group in flight
+    if (ORDER == 6)
+      cp_async_wait_group<2>();
+    else
+      cp_async_wait_group<1>();
 #pragma unroll
-      for (int q = 0; q < F::R; ++q) {
-        const V v = wst[elem(q)];
-        vr[q] = v.x;
-        vi[q] = v.y;
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < F::R; ++q) {
-        const V v = *reinterpret_cast<const V*>(data + (base + (unsigned)(j + q * F::TS) * line_stride));
-        vr[q] = v.x;
-        vi[q] = v.y;
-      }
+    for (int q = 0; q < F::R; ++q) {
+      const V v = wst[elem(q)];
+      vr[q] = v.x;
+      vi[q] = v.y;
     }
     F::run(vr, vi, j, sr, si, twc, tws);
-    if (ORDER == 6) {
-      if (PERSIST)
-        cp_async_wait_group<1>();
-      else
-        cp_async_wait_all();
-    }
+    if (ORDER == 6) cp_async_wait_group<1>();
 
     const T mo = (symo != nullptr) ? symo[yo] : T(0);
     const T mxa = symx[x] + mo, mxb = symx[x + 1] + mo;
@@ -565,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && ORDER == 4 && !PER
     }
     __syncthreads();  // the line buffers are rewritten by the next tile
   }
-  if (PERSIST) cp_async_wait_all();
+  cp_async_wait_all();
   mid_finish<T, ORDER>(acc, sred, partials, ctrl, kp, &sflag);
 }
 
@@ -618,17 +463,10 @@ __global__ void k_spec_apply_T(T* a, T scale, KParams kp, const T* sx, const T* 
 }
 
 // ------------------------------------------------------------ launch helpers
-// Radix of the register passes: 16 for the FP32 row/column passes; 8 where
-// radix 16's register footprint would halve the occupancy (FP64, and the
-// middle pass, which also holds the symbol-division state).
-template <typename T>
-constexpr int radix_pass() {
-  return sizeof(T) == 8 ? 8 : 16;
-}
-template <typename T>
-constexpr int radix_mid() {
-  return 8;
-}
+// Radix of the register passes: 16 for the row and column passes; 8 where
+// radix 16's register footprint would halve the occupancy (the middle pass,
+// which also holds the symbol-division state).
+constexpr int kRadixPass = 16, kRadixMid = 8;
 template <typename T, int N, int RM, bool ROWS>
 size_t pair_smem() {
   return 2 * (size_t)line_stride_words<T, N, RM, ROWS>() * sizeof(T);
@@ -647,27 +485,27 @@ int pick_pairs(int avail_pairs, int cap = 0) {
   return pairs < 1 ? 1 : pairs;
 }
 
-template <typename S, typename T, int N, typename SI = S>
-cudaError_t rows_impl(const SI* src, S* dst, int nrows, T scale, const int* done, const T* twc,
+template <typename T, int N>
+cudaError_t rows_impl(const T* src, T* dst, int nrows, T scale, const int* done, const T* twc,
                       const T* tws, cudaStream_t st, int cap = 0) {
-  constexpr int RM = radix_pass<T>();
+  constexpr int RM = kRadixPass;
   using F = LineFFT<T, N, RM>;
   const int pairs = pick_pairs<T, N, RM, true>(1 << 30, cap);
   const int rows_per_block = 2 * pairs;
   const int grid = (nrows + rows_per_block - 1) / rows_per_block;
-  k_dht_rows<S, T, N, RM, SI><<<grid, pairs * F::TS, pairs * pair_smem<T, N, RM, true>(), st>>>(
+  k_dht_rows<T, N, RM><<<grid, pairs * F::TS, pairs * pair_smem<T, N, RM, true>(), st>>>(
       src, dst, nrows, scale, done, twc, tws);
   return cudaGetLastError();
 }
 
-template <typename S, typename T, int N>
-cudaError_t cols_impl(S* data, int nx, int nouter, size_t line_stride, size_t outer_stride, T scale,
+template <typename T, int N>
+cudaError_t cols_impl(T* data, int nx, int nouter, size_t line_stride, size_t outer_stride, T scale,
                       const int* done, const T* twc, const T* tws, cudaStream_t st, int cap = 0) {
-  constexpr int RM = radix_pass<T>();
+  constexpr int RM = kRadixPass;
   using F = LineFFT<T, N, RM>;
   const int pairs = pick_pairs<T, N, RM, false>(nx / 2, cap);
   dim3 grid(nx / (2 * pairs), nouter);
-  k_dht_cols<S, T, N, RM><<<grid, pairs * F::TS, pairs * pair_smem<T, N, RM, false>(), st>>>(
+  k_dht_cols<T, N, RM><<<grid, pairs * F::TS, pairs * pair_smem<T, N, RM, false>(), st>>>(
       data, line_stride, outer_stride, scale, done, twc, tws);
   return cudaGetLastError();
 }
@@ -675,8 +513,7 @@ cudaError_t cols_impl(S* data, int nx, int nouter, size_t line_stride, size_t ou
 template <typename T, int N>
 cudaError_t mid_impl(T* data, const KParams& kp, Ctrl* ctrl, double* partials, T* xi, T* dspec,
                      const AxisTables<T>& tb, cudaStream_t st) {
-  constexpr int RM = radix_mid<T>();
-  constexpr bool PERSIST = sizeof(T) == 4;
+  constexpr int RM = kRadixMid;
   using F = LineFFT<T, N, RM>;
   using V = typename Vec2<T>::type;
   const int nx = kp.nx;
@@ -708,16 +545,16 @@ cudaError_t mid_impl(T* data, const KParams& kp, Ctrl* ctrl, double* partials, T
   const int ntiles = ntx * nouter;
   // persistent: the CTAs that __launch_bounds__ keeps resident on every SM
   const int per_sm = 2;
-  const int grid = PERSIST ? std::min(ntiles, per_sm * kp.nsm) : ntiles;
+  const int grid = std::min(ntiles, per_sm * kp.nsm);
   const size_t sm = align16(pairs * pair_smem<T, N, RM, false>()) +
-                    ((kp.order == 6 ? 2 : 0) + (PERSIST ? 2 : 0)) * (size_t)N * pairs * sizeof(V);
+                    ((kp.order == 6 ? 2 : 0) + 2) * (size_t)N * pairs * sizeof(V);
   if (sm > kMaxSmemPre) return cudaErrorInvalidConfiguration;
   if (kp.order == 4)
-    k_mid<T, N, 4, RM, PERSIST><<<grid, pairs * F::TS, sm, st>>>(data, (unsigned)line_stride, (unsigned)outer_stride, ntx, ntiles, kp,
+    k_mid<T, N, 4, RM><<<grid, pairs * F::TS, sm, st>>>(data, (unsigned)line_stride, (unsigned)outer_stride, ntx, ntiles, kp,
                                                                  ctrl, partials, xi, dspec, tb.sym[0], symo, syml,
                                                                  twc, tws);
   else
-    k_mid<T, N, 6, RM, PERSIST><<<grid, pairs * F::TS, sm, st>>>(data, (unsigned)line_stride, (unsigned)outer_stride, ntx, ntiles, kp,
+    k_mid<T, N, 6, RM><<<grid, pairs * F::TS, sm, st>>>(data, (unsigned)line_stride, (unsigned)outer_stride, ntx, ntiles, kp,
                                                                  ctrl, partials, xi, dspec, tb.sym[0], symo, syml,
                                                                  twc, tws);
   return cudaGetLastError();
@@ -725,12 +562,11 @@ cudaError_t mid_impl(T* data, const KParams& kp, Ctrl* ctrl, double* partials, T
 
 template <typename T, int N>
 void set_attrs_T() {
-  constexpr int RP = radix_pass<T>(), RD = radix_mid<T>();
-  cudaFuncSetAttribute(k_dht_rows<T, T, N, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-  cudaFuncSetAttribute(k_dht_cols<T, T, N, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-  constexpr bool PST = sizeof(T) == 4;
-  cudaFuncSetAttribute(k_mid<T, N, 4, RD, PST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemPre);
-  cudaFuncSetAttribute(k_mid<T, N, 6, RD, PST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemPre);
+  constexpr int RP = kRadixPass, RD = kRadixMid;
+  cudaFuncSetAttribute(k_dht_rows<T, N, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+  cudaFuncSetAttribute(k_dht_cols<T, N, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+  cudaFuncSetAttribute(k_mid<T, N, 4, RD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemPre);
+  cudaFuncSetAttribute(k_mid<T, N, 6, RD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemPre);
 }
 
 #define PSD_DISPATCH_N(n, CALL)      \
@@ -748,38 +584,6 @@ void set_attrs_T() {
 
 
 }  // namespace
-
-template <typename T>
-cudaError_t launch_dht_rows(const T* src, T* dst, int nx, int nrows, T scale, const int* done,
-                            const AxisTables<T>& tb, cudaStream_t st) {
-  PSD_DISPATCH_N(nx, (rows_impl<T, T, NN>(src, dst, nrows, scale, done, tb.twc[0], tb.tws[0], st, tb.tile_cap[0])));
-}
-
-template <typename T>
-cudaError_t launch_dht_cols(T* data, const KParams& kp, int ax, T scale, const int* done,
-                            const AxisTables<T>& tb, cudaStream_t st) {
-  const int n = ax == 1 ? kp.ny : kp.nz;
-  size_t line_stride, outer_stride;
-  int nouter;
-  if (ax == 1) {
-    line_stride = kp.nx;
-    outer_stride = (size_t)kp.nx * kp.ny;
-    nouter = kp.nz;
-  } else {
-    line_stride = (size_t)kp.nx * kp.ny;
-    outer_stride = kp.nx;
-    nouter = kp.ny;
-  }
-  PSD_DISPATCH_N(n, (cols_impl<T, T, NN>(data, kp.nx, nouter, line_stride, outer_stride, scale, done,
-                                         tb.twc[ax], tb.tws[ax], st, tb.tile_cap[1])));
-}
-
-template <typename T>
-cudaError_t launch_mid(T* data, const KParams& kp, Ctrl* ctrl, double* partials, T* xi, T* dspec,
-                       const AxisTables<T>& tb, cudaStream_t st) {
-  const int n = kp.dim == 2 ? kp.ny : kp.nz;
-  PSD_DISPATCH_N(n, (mid_impl<T, NN>(data, kp, ctrl, partials, xi, dspec, tb, st)));
-}
 
 template <typename T>
 cudaError_t launch_spec6_combine(T* a, const T* b, const KParams& kp, const AxisTables<T>& tb,

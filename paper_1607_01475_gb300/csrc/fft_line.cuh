@@ -30,55 +30,43 @@ template <typename T>
 __device__ __forceinline__ T ld_tw(const T* p) {
   return __ldg(p);
 }
-template <>
-__device__ __forceinline__ ff ld_tw<ff>(const ff* p) {
-  const float2 v = __ldg(reinterpret_cast<const float2*>(p));
-  return ff(v.x, v.y);
-}
 template <typename T>
-__device__ __forceinline__ T half_of(T x) {
+__host__ __device__ __forceinline__ T half_of(T x) {
   return T(0.5) * x;
-}
-template <>
-__device__ __forceinline__ ff half_of<ff>(ff x) {
-  return ff_scale2(x, 0.5f);
 }
 
 // a * b + c and c - a * b with one rounding where the type allows it.
 template <typename T>
-__device__ __forceinline__ T mul_add(T a, T b, T c) {
+__host__ __device__ __forceinline__ T mul_add(T a, T b, T c) {
   return a * b + c;
 }
 template <>
-__device__ __forceinline__ float mul_add<float>(float a, float b, float c) {
+__host__ __device__ __forceinline__ float mul_add<float>(float a, float b, float c) {
   return fmaf(a, b, c);
 }
-template <>
-__device__ __forceinline__ double mul_add<double>(double a, double b, double c) {
-  return fma(a, b, c);
-}
 template <typename T>
-__device__ __forceinline__ T neg_mul_add(T a, T b, T c) {
+__host__ __device__ __forceinline__ T neg_mul_add(T a, T b, T c) {
   return c - a * b;
 }
 template <>
-__device__ __forceinline__ float neg_mul_add<float>(float a, float b, float c) {
+__host__ __device__ __forceinline__ float neg_mul_add<float>(float a, float b, float c) {
   return fmaf(-a, b, c);
-}
-template <>
-__device__ __forceinline__ double neg_mul_add<double>(double a, double b, double c) {
-  return fma(-a, b, c);
 }
 
 // Twiddle source: (cos, sin)(2 pi t / N) from two tables of the element type.
+// rotate: the product with W_N^t (odd: of an odd point of the butterfly); untwiddled: the points a pass does not
+// rotate (block fixed point scales them, see fx_line.cuh).
 template <typename T>
 struct TwPair {
   const T* __restrict__ c;
   const T* __restrict__ s;
-  __device__ __forceinline__ void get(int t, T& cv, T& sv) const {
-    cv = ld_tw(c + t);
-    sv = ld_tw(s + t);
+  __device__ __forceinline__ void rotate(int t, T& a, T& b, bool) const {
+    const T cv = ld_tw(c + t), sv = ld_tw(s + t);
+    const T a0 = a;
+    a = mul_add(b, sv, a * cv);
+    b = neg_mul_add(a0, sv, b * cv);
   }
+  __device__ __forceinline__ void untwiddled(T&, T&) const {}
 };
 
 // cos(2 pi m / 16), the 16th roots of unity (exact values of cos(pi/8),
@@ -103,12 +91,20 @@ __host__ __device__ constexpr double cos16(int m) {
 }
 __host__ __device__ constexpr double sin16(int m) { return cos16(m - 4); }
 
+// (tr, ti) = (a, b) W_16^m with W_16 = exp(-2 pi i / 16).
+template <typename T>
+__host__ __device__ __forceinline__ void rot16(int m, T a, T b, T& tr, T& ti) {
+  const T c = (T)cos16(m), sn = (T)sin16(m);
+  tr = mul_add(b, sn, a * c);
+  ti = neg_mul_add(a, sn, b * c);
+}
+
 // In-register DFT of size R (R | 16): radix-2 decimation in time, in-order
 // input and output.  X_k = sum_j x_j exp(-2 pi i j k / R).
 template <int R>
 struct DFT {
   template <typename T>
-  __device__ __forceinline__ static void run(T (&re)[R], T (&im)[R]) {
+  __host__ __device__ __forceinline__ static void run(T (&re)[R], T (&im)[R]) {
     T er[R / 2], ei[R / 2], orr[R / 2], oi[R / 2];
 #pragma unroll
     for (int j = 0; j < R / 2; ++j) {
@@ -133,9 +129,7 @@ struct DFT {
         tr = orr[k];
         ti = oi[k];
       } else {  // W = c - i sn
-        const T c = (T)cos16(k * 16 / R), sn = (T)sin16(k * 16 / R);
-        tr = mul_add(oi[k], sn, orr[k] * c);
-        ti = neg_mul_add(orr[k], sn, oi[k] * c);
+        rot16<T>(k * 16 / R, orr[k], oi[k], tr, ti);
       }
       re[k] = er[k] + tr;
       im[k] = ei[k] + ti;
@@ -147,7 +141,7 @@ struct DFT {
 template <>
 struct DFT<1> {
   template <typename T>
-  __device__ __forceinline__ static void run(T (&)[1], T (&)[1]) {}
+  __host__ __device__ __forceinline__ static void run(T (&)[1], T (&)[1]) {}
 };
 
 // Complex FFT of one line of N points by a team of TS threads (team index
@@ -181,15 +175,9 @@ struct LineFFT {
         xi[r] = vi[b + r * M];
       }
       if (NS > 1) {
+        tw.untwiddled(xr[0], xi[0]);
 #pragma unroll
-        for (int r = 1; r < RP; ++r) {
-          const int t = jm * r * (N / (NS * RP));
-          T c, sn;
-          tw.get(t, c, sn);
-          const T a = xr[r], bb = xi[r];
-          xr[r] = mul_add(bb, sn, a * c);
-          xi[r] = neg_mul_add(a, sn, bb * c);
-        }
+        for (int r = 1; r < RP; ++r) tw.rotate(jm * r * (N / (NS * RP)), xr[r], xi[r], r & 1);
       }
       DFT<RP>::run(xr, xi);
       const int base = (jp / NS) * NS * RP + jm;
@@ -237,14 +225,9 @@ struct LineFFT {
         xi[r] = vi[b + r * M];
       }
       if (NS > 1) {
+        tw.untwiddled(xr[0], xi[0]);
 #pragma unroll
-        for (int r = 1; r < RP; ++r) {
-          T c, sn;
-          tw.get(jp * r, c, sn);
-          const T a = xr[r], bb = xi[r];
-          xr[r] = mul_add(bb, sn, a * c);
-          xi[r] = neg_mul_add(a, sn, bb * c);
-        }
+        for (int r = 1; r < RP; ++r) tw.rotate(jp * r, xr[r], xi[r], r & 1);
       }
       DFT<RP>::run(xr, xi);
 #pragma unroll
@@ -303,15 +286,10 @@ struct LineFFT {
   }
 };
 
-// Value of lane src of the same warp (float, double, or float-float as two
-// shuffles of its words).
+// Value of lane src of the same warp.
 template <typename T>
 __device__ __forceinline__ T shfl_from(unsigned mask, T v, int src) {
   return __shfl_sync(mask, v, src);
-}
-template <>
-__device__ __forceinline__ ff shfl_from<ff>(unsigned mask, ff v, int src) {
-  return ff(__shfl_sync(mask, v.hi, src), __shfl_sync(mask, v.lo, src));
 }
 
 // Hartley outputs of the two real lines of a spectrum held in registers by

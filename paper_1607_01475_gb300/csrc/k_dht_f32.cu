@@ -1,20 +1,40 @@
-// FP32 instantiations of the Hartley transform passes and the middle pass
-// (the mixed solver's inner iteration).
+// FP32 Hartley transform passes and the middle pass (the mixed solver's
+// inner iteration).
 #include "dht_kernels.cuh"
 
 namespace psd {
 
-#define PSD_INST(T)                                                                                    \
-  template cudaError_t launch_dht_rows<T>(const T*, T*, int, int, T, const int*, const AxisTables<T>&, \
-                                          cudaStream_t);                                               \
-  template cudaError_t launch_dht_cols<T>(T*, const KParams&, int, T, const int*, const AxisTables<T>&, \
-                                          cudaStream_t);                                               \
-  template cudaError_t launch_mid<T>(T*, const KParams&, Ctrl*, double*, T*, T*, const AxisTables<T>&,  \
-                                     cudaStream_t);                                                    \
-  template cudaError_t launch_spec6_combine<T>(T*, const T*, const KParams&, const AxisTables<T>&,      \
-                                               cudaStream_t);                                          \
-  template cudaError_t launch_spec_apply_T<T>(T*, T, const KParams&, const AxisTables<T>&, cudaStream_t);
-PSD_INST(float)
+template <>
+cudaError_t launch_dht_rows<float>(const float* src, float* dst, int nx, int nrows, float scale, const int* done,
+                            const AxisTables<float>& tb, cudaStream_t st) {
+  PSD_DISPATCH_N(nx, (rows_impl<float, NN>(src, dst, nrows, scale, done, tb.twc[0], tb.tws[0], st, tb.tile_cap[0])));
+}
+
+template <>
+cudaError_t launch_dht_cols<float>(float* data, const KParams& kp, int ax, float scale, const int* done,
+                            const AxisTables<float>& tb, cudaStream_t st) {
+  const int n = ax == 1 ? kp.ny : kp.nz;
+  size_t line_stride, outer_stride;
+  int nouter;
+  if (ax == 1) {
+    line_stride = kp.nx;
+    outer_stride = (size_t)kp.nx * kp.ny;
+    nouter = kp.nz;
+  } else {
+    line_stride = (size_t)kp.nx * kp.ny;
+    outer_stride = kp.nx;
+    nouter = kp.ny;
+  }
+  PSD_DISPATCH_N(n, (cols_impl<float, NN>(data, kp.nx, nouter, line_stride, outer_stride, scale, done,
+                                         tb.twc[ax], tb.tws[ax], st, tb.tile_cap[1])));
+}
+
+template <>
+cudaError_t launch_mid<float>(float* data, const KParams& kp, Ctrl* ctrl, double* partials, float* xi, float* dspec,
+                       const AxisTables<float>& tb, cudaStream_t st) {
+  const int n = kp.dim == 2 ? kp.ny : kp.nz;
+  PSD_DISPATCH_N(n, (mid_impl<float, NN>(data, kp, ctrl, partials, xi, dspec, tb, st)));
+}
 
 void init_dht_attributes_f32() {
   set_attrs_T<float, 8>();

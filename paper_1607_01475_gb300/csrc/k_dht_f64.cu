@@ -1,33 +1,39 @@
-// FP64 instantiations of the Hartley transform passes, the middle pass and
-// the spectral helpers (the plain FP64 solver, the FP64 preconditioner and
-// residual entry points).
-#include "dht_kernels.cuh"
+// FP64 Hartley transform passes along x and along a strided axis (block
+// fixed point), and the spectral helpers.
+#include "dht_fx.cuh"
 
 namespace psd {
 
-#define PSD_INST(T)                                                                                    \
-  template cudaError_t launch_dht_rows<T>(const T*, T*, int, int, T, const int*, const AxisTables<T>&, \
-                                          cudaStream_t);                                               \
-  template cudaError_t launch_dht_cols<T>(T*, const KParams&, int, T, const int*, const AxisTables<T>&, \
-                                          cudaStream_t);                                               \
-  template cudaError_t launch_mid<T>(T*, const KParams&, Ctrl*, double*, T*, T*, const AxisTables<T>&,  \
-                                     cudaStream_t);                                                    \
+template <>
+cudaError_t launch_dht_rows<double>(const double* src, double* dst, int nx, int nrows, double scale, const int* done,
+                                    const AxisTables<double>& tb, cudaStream_t st) {
+  PSD_DISPATCH_N(nx, (rows_fx_impl<NN, double>(src, dst, nrows, scale, done, tb, st)));
+}
+
+cudaError_t launch_dht_rows_from_f32(const float* src, double* dst, int nx, int nrows, const AxisTables<double>& tb,
+                                     cudaStream_t st, const int* skip) {
+  PSD_DISPATCH_N(nx, (rows_fx_impl<NN, float>(src, dst, nrows, 1.0, skip, tb, st)));
+}
+
+template <>
+cudaError_t launch_dht_cols<double>(double* data, const KParams& kp, int ax, double scale, const int* done,
+                                    const AxisTables<double>& tb, cudaStream_t st) {
+  const int n = ax == 1 ? kp.ny : kp.nz;
+  const size_t plane = (size_t)kp.nx * kp.ny;
+  const size_t line_stride = ax == 1 ? (size_t)kp.nx : plane;
+  const size_t outer_stride = ax == 1 ? plane : (size_t)kp.nx;
+  const int nouter = ax == 1 ? kp.nz : kp.ny;
+  PSD_DISPATCH_N(n, (cols_fx_impl<NN>(data, kp.nx, nouter, line_stride, outer_stride, scale, done, tb.fxtw[ax], tb.nsm,
+                                      st)));
+}
+
+#define PSD_INST_SPEC(T)                                                                               \
   template cudaError_t launch_spec6_combine<T>(T*, const T*, const KParams&, const AxisTables<T>&,      \
                                                cudaStream_t);                                          \
   template cudaError_t launch_spec_apply_T<T>(T*, T, const KParams&, const AxisTables<T>&, cudaStream_t);
-PSD_INST(double)
+PSD_INST_SPEC(double)
+#undef PSD_INST_SPEC
 template cudaError_t launch_spec_quad<double>(const double*, const KParams&, Ctrl*, double*, const AxisTables<double>&,
                                               cudaStream_t);
-
-void init_dht_attributes_f64() {
-  set_attrs_T<double, 8>();
-  set_attrs_T<double, 16>();
-  set_attrs_T<double, 32>();
-  set_attrs_T<double, 64>();
-  set_attrs_T<double, 128>();
-  set_attrs_T<double, 256>();
-  set_attrs_T<double, 512>();
-  set_attrs_T<double, 1024>();
-}
 
 }  // namespace psd

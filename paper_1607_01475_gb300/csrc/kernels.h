@@ -8,7 +8,9 @@
 
 namespace psd {
 
-// Per-axis tables owned by a context, in FP64, FP32 and float-float.
+struct fx_tw;  // Q62 twiddle of the block fixed-point transforms (fx_line.cuh)
+
+// Per-axis tables owned by a context, in FP64 and FP32.
 template <typename T>
 struct AxisTables {
   const T* twc[3];  // cos(2 pi t / n_a), t < n_a
@@ -18,6 +20,8 @@ struct AxisTables {
   // block in the row, strided and middle passes (0: as many as fill 256
   // threads)
   int tile_cap[3];
+  const fx_tw* fxtw[3];  // FP64 passes: (cos, sin)(2 pi t / n_a) in Q62, t < n_a
+  int nsm;               // SMs of the device (tiles are narrowed while SMs would be idle)
 };
 
 // ----------------------------------------------------------------- DHT passes
@@ -32,25 +36,19 @@ template <typename T>
 cudaError_t launch_dht_cols(T* data, const KParams& kp, int ax, T scale, const int* done,
                             const AxisTables<T>& tb, cudaStream_t st);
 
-// Passes in float-float arithmetic (about 48 significant bits; tables of
-// double-word twiddles).  Between passes the data stays in float-float form
-// (hi, lo pairs in the 8 bytes of an FP64 element): the x pass reads FP64
-// (or FP32) and writes pairs; the strided pass transforms pairs in place.
-// skip (device, may be null): the pass returns at once when *skip != 0.
-cudaError_t launch_dht_rows_ff(const double* src, ff* dst, int nx, int nrows, const AxisTables<ff>& tb,
-                               cudaStream_t st, const int* skip = nullptr);
-cudaError_t launch_dht_rows_ff_from_f32(const float* src, ff* dst, int nx, int nrows, const AxisTables<ff>& tb,
-                                        cudaStream_t st, const int* skip = nullptr);
-cudaError_t launch_dht_cols_ff(ff* data, const KParams& kp, int ax, const AxisTables<ff>& tb, cudaStream_t st,
-                               const int* skip = nullptr);
-// The last pass (z in 3D, y in 2D) with a fused epilogue: out32 == nullptr:
-// theta += DHT(data) / mu, and (dc != null) *dc = the zero-frequency
+// (FP64 passes: block fixed point, see fx_line.cuh; their scale is a power of
+// two.)  The x pass from an FP32 field.  skip (device, may be null): the pass
+// returns at once when *skip != 0.
+cudaError_t launch_dht_rows_from_f32(const float* src, double* dst, int nx, int nrows, const AxisTables<double>& tb,
+                                     cudaStream_t st, const int* skip = nullptr);
+// The last FP64 pass (z in 3D, y in 2D) with a fused epilogue: out32 ==
+// nullptr: theta += DHT(data) / mu, and (dc != null) *dc = the zero-frequency
 // coefficient (the sum of the transformed field); else out32 = (float)(DHT(data)
 // - theta) and ctrl->res_l2 = its Parseval norm (h^d / N sum)^{1/2}.  mu = 0
 // gives 0.
-cudaError_t launch_dht_last_ff(const ff* data, double* theta, float* out32, const KParams& kp, Ctrl* ctrl,
-                               double* partials, const AxisTables<ff>& tb, cudaStream_t st, double* dc = nullptr,
-                               const int* skip = nullptr);
+cudaError_t launch_dht_last(const double* data, double* theta, float* out32, const KParams& kp, Ctrl* ctrl,
+                            double* partials, const AxisTables<double>& tb, cudaStream_t st, double* dc = nullptr,
+                            const int* skip = nullptr);
 
 // The middle pass along the slowest axis (y in 2D, z in 3D) of the
 // preconditioner: forward DHT, division by the symbol of L_h, Parseval sums
@@ -63,6 +61,16 @@ cudaError_t launch_dht_last_ff(const ff* data, double* theta, float* out32, cons
 template <typename T>
 cudaError_t launch_mid(T* data, const KParams& kp, Ctrl* ctrl, double* partials, T* xi, T* dspec,
                        const AxisTables<T>& tb, cudaStream_t st);
+#define PSD_DECL_PASSES(T)                                                                                      \
+  template <>                                                                                                   \
+  cudaError_t launch_dht_rows<T>(const T*, T*, int, int, T, const int*, const AxisTables<T>&, cudaStream_t);    \
+  template <>                                                                                                   \
+  cudaError_t launch_dht_cols<T>(T*, const KParams&, int, T, const int*, const AxisTables<T>&, cudaStream_t);   \
+  template <>                                                                                                   \
+  cudaError_t launch_mid<T>(T*, const KParams&, Ctrl*, double*, T*, T*, const AxisTables<T>&, cudaStream_t);
+PSD_DECL_PASSES(float)
+PSD_DECL_PASSES(double)
+#undef PSD_DECL_PASSES
 
 // Spectral helpers (order 6, off the hot loop).
 // spec6_combine: a <- (mu == 0) ? 0 : a - b / mu   (a, b full DHT spectra)

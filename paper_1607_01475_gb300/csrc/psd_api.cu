@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "../../include/psd.h"
+#include "fx_line.cuh"
 #include "kernels.h"
 
 using psd::AxisTables;
@@ -61,7 +62,6 @@ struct psd_context {
   void* tables = nullptr;
   AxisTables<double> tb64{};
   AxisTables<float> tb32{};
-  AxisTables<psd::ff> tbff{};
 
   // FP64 work arrays
   double* ub = nullptr;     // second iterate buffer (ping-pong with the caller's u)
@@ -239,34 +239,22 @@ psd_status build_tables(psd_context* c) {
     off += n[a];
   }
   for (size_t i = 0; i < tot; ++i) h32[i] = (float)h64[i];
-  // float-float twiddles: hi = the nearest float, lo = the nearest float to
-  // the remainder, both from the long-double value
-  std::vector<psd::ff> hff(tot);
+  // Q62 twiddles of the fixed-point transforms
+  std::vector<psd::fx_tw> hfx((size_t)n[0] + n[1] + n[2]);
+  size_t ofx[3] = {0, (size_t)n[0], (size_t)n[0] + n[1]};
   for (int a = 0; a < 3; ++a)
     for (int t = 0; t < n[a]; ++t)
-      for (int w = 0; w < 3; ++w) {
-        long double v;
-        if (w == 0)
-          v = cosl(2.0L * pi * t / n[a]);
-        else if (w == 1)
-          v = sinl(2.0L * pi * t / n[a]);
-        else {
-          const long double sn = (n[a] > 1) ? sinl(pi * t / n[a]) : 0.0L;
-          v = 4.0L / (h * h) * sn * sn;
-        }
-        const float hi = (float)v;
-        hff[offs[a][w] + t] = psd::ff(hi, (float)(v - (long double)hi));
-      }
+      hfx[ofx[a] + t] = psd::fx_make_tw(cosl(2.0L * pi * t / n[a]), sinl(2.0L * pi * t / n[a]));
   {
     unsigned char* t = nullptr;
-    TRY(alloc(c, &t, tot * (sizeof(double) + sizeof(float) + sizeof(psd::ff))));
+    TRY(alloc(c, &t, tot * (sizeof(double) + sizeof(float)) + hfx.size() * sizeof(psd::fx_tw)));
     c->tables = t;
   }
-  double* d64 = (double*)c->tables;
-  psd::ff* dff = (psd::ff*)(d64 + tot);
-  float* d32 = (float*)(dff + tot);
+  psd::fx_tw* dfx = (psd::fx_tw*)c->tables;  // 16-byte entries first
+  double* d64 = (double*)(dfx + hfx.size());
+  float* d32 = (float*)(d64 + tot);
   CK(cudaMemcpy(d64, h64.data(), tot * sizeof(double), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(dff, hff.data(), tot * sizeof(psd::ff), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(dfx, hfx.data(), hfx.size() * sizeof(psd::fx_tw), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(d32, h32.data(), tot * sizeof(float), cudaMemcpyHostToDevice));
   for (int a = 0; a < 3; ++a) {
     c->tb64.twc[a] = d64 + offs[a][0];
@@ -275,10 +263,9 @@ psd_status build_tables(psd_context* c) {
     c->tb32.twc[a] = d32 + offs[a][0];
     c->tb32.tws[a] = d32 + offs[a][1];
     c->tb32.sym[a] = d32 + offs[a][2];
-    c->tbff.twc[a] = dff + offs[a][0];
-    c->tbff.tws[a] = dff + offs[a][1];
-    c->tbff.sym[a] = dff + offs[a][2];
+    c->tb64.fxtw[a] = dfx + ofx[a];
   }
+  c->tb64.nsm = c->tb32.nsm = c->kp.nsm;
   return PSD_OK;
 }
 
@@ -418,20 +405,20 @@ psd_status full_dht(psd_context* c, T* x, T scale, const AxisTables<T>& tb) {
 // theta += DHT(v) / mu (order 6, mixed): v is src64 (FP64, transformed in
 // place) or src32 (FP32, transformed into D); theta lives in Z.  skip
 // (device, may be null): the passes return at once when *skip != 0.
-psd_status dht_theta_ff(psd_context* c, const double* src64, const float* src32, double* dc = nullptr,
+psd_status dht_theta(psd_context* c, const double* src64, const float* src32, double* dc = nullptr,
                         const int* skip = nullptr) {
   const KParams& kp = c->kp;
   const int nrows = kp.ny * kp.nz;
-  psd::ff* x = reinterpret_cast<psd::ff*>(c->D);  // float-float pairs between the passes
+  double* x = c->D;
   if (src32) {
     ProfScope p_(c, PSD_PROF_DHT_ROWS_FF);
-    CK(psd::launch_dht_rows_ff_from_f32(src32, x, kp.nx, nrows, c->tbff, c->st, skip));
+    CK(psd::launch_dht_rows_from_f32(src32, x, kp.nx, nrows, c->tb64, c->st, skip));
   } else {
     ProfScope p_(c, PSD_PROF_DHT_ROWS_FF);
-    CK(psd::launch_dht_rows_ff(src64, x, kp.nx, nrows, c->tbff, c->st, skip));
+    CK(psd::launch_dht_rows<double>(src64, x, kp.nx, nrows, 1.0, skip, c->tb64, c->st));
   }
-  if (kp.dim == 3) { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_cols_ff(x, kp, 1, c->tbff, c->st, skip)); }
-  { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_last_ff(x, c->Z, nullptr, kp, nullptr, c->partials, c->tbff, c->st, dc, skip)); }
+  if (kp.dim == 3) { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_cols<double>(x, kp, 1, 1.0, skip, c->tb64, c->st)); }
+  { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_last(x, c->Z, nullptr, kp, nullptr, c->partials, c->tb64, c->st, dc, skip)); }
   return PSD_OK;
 }
 
@@ -652,10 +639,10 @@ psd_status outer_residual6_spec(psd_context* c, const double* u, const double* f
   ResArgs<double> a{u, nullptr, nullptr, f, nullptr, c->W, 0, 0, fxs ? 1 : 0, fxs, fxs_dev};
   { ProfScope p_(c, PSD_PROF_RESIDUAL_FP64); CK(psd::launch_residual<double>(a, psd::RM_PLAIN, c->pk, kp, c->ctrl2, c->partials, c->st)); }
   const int nrows = kp.ny * kp.nz;
-  psd::ff* x = reinterpret_cast<psd::ff*>(c->W);  // transformed in place, float-float pairs after the x pass
-  { ProfScope p_(c, PSD_PROF_DHT_ROWS_FF); CK(psd::launch_dht_rows_ff(c->W, x, kp.nx, nrows, c->tbff, c->st)); }
-  if (kp.dim == 3) { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_cols_ff(x, kp, 1, c->tbff, c->st)); }
-  { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_last_ff(x, c->Z, c->R32, kp, c->ctrl2, c->partials, c->tbff, c->st)); }
+  double* x = c->W;  // transformed in place
+  { ProfScope p_(c, PSD_PROF_DHT_ROWS_FF); CK(psd::launch_dht_rows<double>(x, x, kp.nx, nrows, 1.0, nullptr, c->tb64, c->st)); }
+  if (kp.dim == 3) { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_cols<double>(x, kp, 1, 1.0, nullptr, c->tb64, c->st)); }
+  { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_last(x, c->Z, c->R32, kp, c->ctrl2, c->partials, c->tb64, c->st)); }
   return PSD_OK;
 }
 
@@ -857,7 +844,7 @@ psd_status mixed_start(psd_context* c, const double* g, double* u) {
   if (c->kp.order == 6) {
     CK(cudaMemsetAsync(c->Z, 0, c->N * sizeof(double), c->st));
     { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_axpby<double>(c->D, u, g, 1.0, -1.0, 0.0, c->N, c->st)); }
-    TRY(dht_theta_ff(c, c->D, nullptr));
+    TRY(dht_theta(c, c->D, nullptr));
   }
   return PSD_OK;
 }
@@ -901,7 +888,7 @@ psd_status mixed_graph_body(psd_context* c, const double* f, const double* g, do
     // (mean removed for order 6), u32 = fl32(u) -- skipped once the outer
     // loop is done
     double* dsum = six ? &c->ctrl2->c3 : nullptr;
-    if (six) TRY(dht_theta_ff(c, nullptr, c->da, dsum, &c->ctrl3->done));
+    if (six) TRY(dht_theta(c, nullptr, c->da, dsum, &c->ctrl3->done));
     { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_accumulate_f64(u, c->da, c->u32, c->N, dsum, c->st, &c->ctrl3->done)); }
     CK(psd::launch_loop_cond(ho, c->ctrl3, guard_outer, c->st));
     (void)inner_cap;
@@ -951,7 +938,7 @@ psd_status solve_mixed(psd_context* c, const double* f, const double* g, double*
       // removes the mean of delta, which is zero only up to FP32 rounding,
       // so that mean(u) = mean(g) holds throughout
       double* dsum = six ? &c->ctrl2->c3 : nullptr;
-      if (six) TRY(dht_theta_ff(c, nullptr, c->da, dsum));
+      if (six) TRY(dht_theta(c, nullptr, c->da, dsum));
       { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_accumulate_f64(u, c->da, c->u32, c->N, dsum, c->st)); }
     }
     int fxs = 0;
@@ -1491,10 +1478,10 @@ psd_status psd_theta_ff(psd_handle c, const double* x, double* theta) {
   TRY(ensure_fp64(c));
   const KParams& kp = c->kp;
   const int nrows = kp.ny * kp.nz;
-  psd::ff* w = reinterpret_cast<psd::ff*>(c->D);
-  { ProfScope p_(c, PSD_PROF_DHT_ROWS_FF); CK(psd::launch_dht_rows_ff(x, w, kp.nx, nrows, c->tbff, c->st)); }
-  if (kp.dim == 3) { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_cols_ff(w, kp, 1, c->tbff, c->st)); }
-  { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_last_ff(w, theta, nullptr, kp, nullptr, c->partials, c->tbff, c->st)); }
+  double* w = c->D;
+  { ProfScope p_(c, PSD_PROF_DHT_ROWS_FF); CK(psd::launch_dht_rows<double>(x, w, kp.nx, nrows, 1.0, nullptr, c->tb64, c->st)); }
+  if (kp.dim == 3) { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_cols<double>(w, kp, 1, 1.0, nullptr, c->tb64, c->st)); }
+  { ProfScope p_(c, PSD_PROF_DHT_COLS_FF); CK(psd::launch_dht_last(w, theta, nullptr, kp, nullptr, c->partials, c->tb64, c->st)); }
   CK(cudaStreamSynchronize(c->st));
   return PSD_OK;
 }
