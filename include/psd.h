@@ -230,16 +230,16 @@ psd_status psd_thinfilm_adjoint(psd_handle h, const double* u0, int nsteps,
 psd_status psd_spfc_steps(psd_handle h, double* u, double gamma1, int nsteps,
                           psd_info* info);
 
-/* FP64 residual by the kernel variant of the mixed solve's outer residual,
- * for tests: r = f - N_h[u] (order 6: the local part, without T_h) with the
- * linear part (z-pair sums, vertex gradients, both Laplacian passes of
- * Sec. 5.1) in exact 64-bit fixed point, q = round(u 2^S), and the p = 4
- * flux part in float-float; only the final combination is FP64.  S = 55 - e
- * for max|u| (1 + 2^-20) < 2^e, returned in *scale.  Applies to p = 4 on 3D
- * grids with nx >= 32 and ny >= 8, and max|u| in [2^-65, 2^40); otherwise
- * *scale = 0 and r is not written.  u, f, r: device, N doubles; scale: host.
- * The solver's bound on the float-float error of the flux part is not
- * checked here.  Errors: PSD_ERR_INVALID for null pointers.                */
+/* FP64 residual by the fixed-point kernel variant that the solvers take in
+ * 3D at p = 4, for tests: r = f - N_h[u] (order 6: the local part, without
+ * T_h) with the linear part (z-pair sums, vertex gradients, both Laplacian
+ * passes of Sec. 5.1) in exact 64-bit fixed point, q = round(u 2^S), and the
+ * flux part in 64-bit fixed point relative to the largest gradient; only the
+ * final combination is FP64.  S = 55 - e for max|u| (1 + 2^-20) < 2^e, returned
+ * in *scale.  Applies to p = 4 on 3D grids with nx >= 32 and ny >= 8, and
+ * max|u| in [2^-65, 2^40); otherwise *scale = 0 and r is not written.  u, f,
+ * r: device, N doubles; scale: host.  The solvers' rule on the error of the
+ * flux part is not checked here.  Errors: PSD_ERR_INVALID for null pointers. */
 psd_status psd_residual_fixed(psd_handle h, const double* u, const double* f,
                               double* r, int* scale);
 

@@ -274,7 +274,7 @@ def psd_thinfilm_adjoint(handle, u0, nsteps, grad_uN, grad_u0, checkpoints=0, to
 
 
 def psd_residual_fixed(handle, u, f, r):
-    """FP64 residual by the fixed-point / float-float kernel variant; returns
+    """FP64 residual by the fixed-point kernel variant; returns
     the fixed-point scale S (0: the variant does not apply, r untouched)."""
     scale = ctypes.c_int()
     _check(load_library().psd_residual_fixed(handle, _ptr(u), _ptr(f), _ptr(r), ctypes.byref(scale)), handle)

@@ -158,7 +158,8 @@ __device__ __forceinline__ double recip_pos(double x) {
 // -------------------------------------------------------------- x (rows)
 template <int N, typename SI>
 __global__ void __launch_bounds__(kFxThreads, 3)
-    k_rows_fx(const SI* src, double* dst, int nrows, int scale_e, const int* done, const fx_tw* __restrict__ tab) {
+    k_rows_fx(const SI* src, double* dst, int nrows, int scale_e, const int* done, const fx_tw* __restrict__ tab,
+              unsigned int* dmax_hi) {
   using F = LineFFT<fx, N, 8>;
   constexpr int R = F::R, TS = F::TS;
   if (done != nullptr && *done) return;
@@ -186,6 +187,13 @@ __global__ void __launch_bounds__(kFxThreads, 3)
   fx vr[R], vi[R];
   fx_enter<N>(xr, xi, ln, vr, vi);
   double* d0 = dst + (size_t)row0 * N;
+  unsigned top = 0u;  // largest magnitude written, high word
+  auto put = [&](int k, fx h1, fx h2) {
+    const double a = fx_leave<N>(h1, ln, scale_e), b = fx_leave<N>(h2, ln, scale_e);
+    d0[k] = a;
+    d0[N + k] = b;
+    top = max(top, max((unsigned)__double2hiint(a) & 0x7FFFFFFFu, (unsigned)__double2hiint(b) & 0x7FFFFFFFu));
+  };
   if constexpr (FxTeam<N, true>::kOneWarp) {
     // the last pass ends in registers, the split by shuffle
     F::run_tw_regs(vr, vi, j, sr, si, TwFx{tab});
@@ -193,22 +201,28 @@ __global__ void __launch_bounds__(kFxThreads, 3)
     dht_split_regs<fx, N, R, TS>(vr, vi, j, h1, h2);
     if (valid) {
 #pragma unroll
-      for (int q = 0; q < R; ++q) {
-        d0[j + q * TS] = fx_leave<N>(h1[q], ln, scale_e);
-        d0[N + j + q * TS] = fx_leave<N>(h2[q], ln, scale_e);
-      }
+      for (int q = 0; q < R; ++q) put(j + q * TS, h1[q], h2[q]);
     }
   } else {
     F::run_tw(vr, vi, j, sr, si, TwFx{tab});
     if (valid) {
 #pragma unroll
       for (int q = 0; q < R; ++q) {
-        const int k = j + q * TS;
         fx h1, h2;
-        dht_split(sr, si, k, N, h1, h2);
-        d0[k] = fx_leave<N>(h1, ln, scale_e);
-        d0[N + k] = fx_leave<N>(h2, ln, scale_e);
+        dht_split(sr, si, j + q * TS, N, h1, h2);
+        put(j + q * TS, h1, h2);
       }
+    }
+  }
+  if (dmax_hi != nullptr) {
+    const unsigned nthr = blockDim.x;
+    for (int o = 16; o > 0; o >>= 1)
+      if (o < (int)nthr) top = max(top, __shfl_xor_sync(nthr >= 32 ? 0xffffffffu : (1u << nthr) - 1u, top, o));
+    if ((tid & 31) == 0) scr[tid >> 5][0].x = top;
+    __syncthreads();
+    if (tid == 0) {
+      for (unsigned w = 1; w < (nthr + 31) / 32; ++w) top = max(top, scr[w][0].x);
+      atomicMax(dmax_hi, top + 1u);
     }
   }
 }
@@ -499,14 +513,14 @@ inline bool fx_scale_exp(double scale, int* e) {
 
 template <int N, typename SI>
 cudaError_t rows_fx_impl(const SI* src, double* dst, int nrows, double scale, const int* done,
-                         const AxisTables<double>& tb, cudaStream_t st) {
+                         const AxisTables<double>& tb, cudaStream_t st, unsigned int* dmax_hi) {
   constexpr int TS = LineFFT<fx, N, 8>::TS;
   int se;
   if (!fx_scale_exp(scale, &se)) return cudaErrorInvalidValue;
   const int np = (nrows + 1) / 2;
   const int pairs = fx_pairs<N, true>(np, 1 << 30, tb.nsm);
   k_rows_fx<N, SI><<<(np + pairs - 1) / pairs, pairs * TS, pairs * fx_pair_smem<N, true>(), st>>>(src, dst, nrows, se,
-                                                                                                 done, tb.fxtw[0]);
+                                                                                                 done, tb.fxtw[0], dmax_hi);
   return cudaGetLastError();
 }
 

@@ -231,6 +231,7 @@ __device__ __forceinline__ void mid_finish(T (&acc)[5], T* sred, double* partial
       ctrl->c3 = 0.0;
       ctrl->alpha = 0.0;
       ctrl->ls_pass = 0;
+      ctrl->dmax_hi = 0u;
       ctrl->counter[CS_MID] = 0;
     }
   }

@@ -87,6 +87,26 @@ __host__ __device__ __forceinline__ void fx_rotate(fx& a, fx& b, const fx_tw& w,
 // points would add up in the lowest frequencies.
 __host__ __device__ __forceinline__ fx fx_quarter(fx x) { return fx((x.v + 1 + ((x.v >> 2) & 1)) >> 2); }
 
+// The p = 4 flux F = |G|^2 G of a vertex gradient whose modulus is below 2^61, in
+// units of 2^125 of G^3: |G|^2 / 2^64, times 8, times G / 2^64, so |F| < 2^58.
+// Returns the high word of |G|^2 / 2^64.
+__host__ __device__ __forceinline__ unsigned fx_flux(long long g0, long long g1, long long g2, long long (&F)[3]) {
+  const fx_halves a = fx_split(g0), b = fx_split(g1), c = fx_split(g2);
+  const long long t = fx_wide(a.h, a.l) + (fx_wide(b.h, b.l) + (fx_wide(c.h, c.l) + (1LL << 30)));
+  const long long s = fx_wide(a.h, a.h) + (fx_wide(b.h, b.h) + (fx_wide(c.h, c.h) + (t >> 31)));
+  const fx_halves w = fx_split((long long)((unsigned long long)s << 3));
+  const long long half = 1LL << 31;
+  F[0] = fx_wide(w.h, a.h) + ((fx_wide(w.h, a.l) + (fx_wide(w.l, a.h) + half)) >> 32);
+  F[1] = fx_wide(w.h, b.h) + ((fx_wide(w.h, b.l) + (fx_wide(w.l, b.h) + half)) >> 32);
+  F[2] = fx_wide(w.h, c.h) + ((fx_wide(w.h, c.l) + (fx_wide(w.l, c.h) + half)) >> 32);
+  return (unsigned)((unsigned long long)s >> 32);
+}
+
+// The 64 bits of a value.
+__device__ __forceinline__ unsigned long long fx_bits(long long v) { return (unsigned long long)v; }
+__device__ __forceinline__ unsigned long long fx_bits(double v) { return (unsigned long long)__double_as_longlong(v); }
+__device__ __forceinline__ unsigned long long fx_bits(float v) { return (unsigned long long)__float_as_uint(v); }
+
 // x sqrt(1/2) = x + x (sqrt(1/2) - 1), the factor in units of 2^-64.
 __host__ __device__ __forceinline__ fx fx_mul_rsqrt2(fx x) {
   constexpr long long W = -5402926248376769404LL;  // (sqrt(1/2) - 1) 2^64

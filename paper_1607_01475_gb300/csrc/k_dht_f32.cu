@@ -6,7 +6,7 @@ namespace psd {
 
 template <>
 cudaError_t launch_dht_rows<float>(const float* src, float* dst, int nx, int nrows, float scale, const int* done,
-                            const AxisTables<float>& tb, cudaStream_t st) {
+                            const AxisTables<float>& tb, cudaStream_t st, unsigned int*) {
   PSD_DISPATCH_N(nx, (rows_impl<float, NN>(src, dst, nrows, scale, done, tb.twc[0], tb.tws[0], st, tb.tile_cap[0])));
 }
 

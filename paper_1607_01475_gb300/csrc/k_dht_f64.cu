@@ -6,13 +6,13 @@ namespace psd {
 
 template <>
 cudaError_t launch_dht_rows<double>(const double* src, double* dst, int nx, int nrows, double scale, const int* done,
-                                    const AxisTables<double>& tb, cudaStream_t st) {
-  PSD_DISPATCH_N(nx, (rows_fx_impl<NN, double>(src, dst, nrows, scale, done, tb, st)));
+                                    const AxisTables<double>& tb, cudaStream_t st, unsigned int* dmax_hi) {
+  PSD_DISPATCH_N(nx, (rows_fx_impl<NN, double>(src, dst, nrows, scale, done, tb, st, dmax_hi)));
 }
 
 cudaError_t launch_dht_rows_from_f32(const float* src, double* dst, int nx, int nrows, const AxisTables<double>& tb,
                                      cudaStream_t st, const int* skip) {
-  PSD_DISPATCH_N(nx, (rows_fx_impl<NN, float>(src, dst, nrows, 1.0, skip, tb, st)));
+  PSD_DISPATCH_N(nx, (rows_fx_impl<NN, float>(src, dst, nrows, 1.0, skip, tb, st, nullptr)));
 }
 
 template <>

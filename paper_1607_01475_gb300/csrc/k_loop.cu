@@ -84,23 +84,6 @@ __global__ void k_mixed_after(Ctrl* c3, const Ctrl* c) {
   }
 }
 
-// The host rule of the direct mixed solve: the fixed-point / float-float
-// residual applies when |Omega|^{1/2} 24 2^-47 cdiv (2 max|G|)^3 < tol / 20
-// and S = 55 - e (max|u| (1 + 2^-20) < 2^e) lies in [15, 120].
-__global__ void k_fluxff_decide(Ctrl* c3, const Ctrl* c2, double sqrt_vol, double cdiv, double tol) {
-  int fxs = 0;
-  const double gmax = 2.0 * sqrt(fmax(c2->res_linf, 0.0));
-  const double bound = sqrt_vol * 24.0 * ldexp(1.0, -47) * cdiv * gmax * gmax * gmax;
-  const double umax = c2->res_l2;
-  if (tol > 0.0 && isfinite(bound) && bound < 0.05 * tol && isfinite(umax)) {
-    int e = 0;
-    if (umax > 0.0) frexp(umax * (1.0 + ldexp(1.0, -20)), &e);
-    const int S = 55 - e;
-    if (S >= 15 && S <= 120) fxs = S;
-  }
-  c3->fxs = fxs;
-}
-
 __global__ void k_ctrl_reset(Ctrl* c) {
   Ctrl z;
   memset(&z, 0, sizeof(z));
@@ -108,6 +91,8 @@ __global__ void k_ctrl_reset(Ctrl* c) {
   z.max_iter = 1 << 30;
   z.res_linf = -1.0;
   z.c2 = -1.0;
+  z.umax = -1.0;
+  z.fx_s = kFxOff;
   *c = z;
 }
 
@@ -141,11 +126,6 @@ cudaError_t launch_mixed_check(Ctrl* c3, const Ctrl* c2, Ctrl* c, const Ctrl* tm
 }
 cudaError_t launch_mixed_after(Ctrl* c3, const Ctrl* c, cudaStream_t st) {
   k_mixed_after<<<1, 1, 0, st>>>(c3, c);
-  return cudaGetLastError();
-}
-cudaError_t launch_fluxff_decide(Ctrl* c3, const Ctrl* c2, double sqrt_vol, double cdiv, double tol,
-                                 cudaStream_t st) {
-  k_fluxff_decide<<<1, 1, 0, st>>>(c3, c2, sqrt_vol, cdiv, tol);
   return cudaGetLastError();
 }
 cudaError_t launch_ctrl_reset(Ctrl* c, cudaStream_t st) {

@@ -11,14 +11,37 @@
 namespace psd {
 namespace {
 
-// max |G|^2 over the vertices of an FP32 field (G from the 8 surrounding
-// cells) into ctrl->res_linf, and max |u| into ctrl->res_l2 (+inf if a
-// value is not finite).  Each thread takes four consecutive vertices of a
-// row (x fastest, nx a multiple of 4, the field 16-byte aligned): the four
-// cell rows around them are read as float4 plus one scalar each.
-__global__ void __launch_bounds__(NT) k_gradmax(const float* __restrict__ u, KParams kp, Ctrl* ctrl,
-                                                double* partials) {
-  __shared__ float sred[32 * 2];
+// Four consecutive values of a row (16-byte aligned, FP64 32-byte) as FP32,
+// rounded or truncated to 20 bits; FP64 values outside the FP32 range give 0 or
+// infinity.
+__device__ __forceinline__ float scan_f32(float v) { return v; }
+__device__ __forceinline__ float scan_f32(double v) {
+  const unsigned h = (unsigned)__double2hiint(v);
+  const int e = (int)((h >> 20) & 0x7FFu) - 896;
+  const unsigned b = e <= 0 ? 0u : (e >= 255 ? 0x7F800000u : ((unsigned)e << 23) | ((h & 0xFFFFFu) << 3));
+  return __uint_as_float(b | (h & 0x80000000u));
+}
+__device__ __forceinline__ void scan_load(const float* p, float (&v)[5]) {
+  const float4 a = *reinterpret_cast<const float4*>(p);
+  v[0] = a.x;
+  v[1] = a.y;
+  v[2] = a.z;
+  v[3] = a.w;
+}
+__device__ __forceinline__ void scan_load(const double* p, float (&v)[5]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v[k] = scan_f32(p[k]);
+}
+
+// Bounds on |u| and on the modulus of the vertex gradient sums G (G from the 8
+// surrounding cells) into ctrl->umax, gmax (infinity if a value is not finite),
+// and the scales of a fixed-point residual at u into ctrl->fx_s, fx_g.  The
+// maxima are taken in FP32 on values within 2^-20 of u, so G is within 2^-17
+// max|u| of the estimate.  Each thread takes four consecutive vertices of a row.
+template <typename T>
+__global__ void __launch_bounds__(NT) k_fx_scan(const T* __restrict__ u, KParams kp, double tol, int forced,
+                                                Ctrl* ctrl) {
+  __shared__ unsigned smax[2];
   __shared__ int sflag;
   const int nx = kp.nx, ny = kp.ny, nz = kp.nz;
   const int lq = __ffs(nx / 4) - 1, lqy = lq + __ffs(ny) - 1;  // sizes are powers of two
@@ -27,34 +50,44 @@ __global__ void __launch_bounds__(NT) k_gradmax(const float* __restrict__ u, KPa
   for (size_t i = blockIdx.x * (size_t)NT + threadIdx.x; i < nq; i += (size_t)gridDim.x * NT) {
     const int x = 4 * (int)(i & (nx / 4 - 1)), y = (int)((i >> lq) & (ny - 1)), z = (int)(i >> lqy);
     const int x4 = (x + 4) & (nx - 1), y1 = (y + 1) & (ny - 1), z1 = (z + 1) & (nz - 1);
-    const float* r00 = u + (size_t)z * plane + (size_t)y * nx;  // rows (z, y), (z, y1), (z1, y), (z1, y1)
-    const float* r01 = u + (size_t)z * plane + (size_t)y1 * nx;
-    const float* r10 = u + (size_t)z1 * plane + (size_t)y * nx;
-    const float* r11 = u + (size_t)z1 * plane + (size_t)y1 * nx;
-    const float4 a = *reinterpret_cast<const float4*>(r00 + x), b = *reinterpret_cast<const float4*>(r01 + x);
-    const float4 c = *reinterpret_cast<const float4*>(r10 + x), d = *reinterpret_cast<const float4*>(r11 + x);
-    const float av[5] = {a.x, a.y, a.z, a.w, r00[x4]}, bv[5] = {b.x, b.y, b.z, b.w, r01[x4]};
-    const float cv[5] = {c.x, c.y, c.z, c.w, r10[x4]}, dv[5] = {d.x, d.y, d.z, d.w, r11[x4]};
+    const T* r00 = u + (size_t)z * plane + (size_t)y * nx;  // rows (z, y), (z, y1), (z1, y), (z1, y1)
+    const T* r01 = u + (size_t)z * plane + (size_t)y1 * nx;
+    const T* r10 = u + (size_t)z1 * plane + (size_t)y * nx;
+    const T* r11 = u + (size_t)z1 * plane + (size_t)y1 * nx;
+    float av[5], bv[5], cv[5], dv[5];
+    scan_load(r00 + x, av);
+    scan_load(r01 + x, bv);
+    scan_load(r10 + x, cv);
+    scan_load(r11 + x, dv);
+    av[4] = scan_f32(r00[x4]);
+    bv[4] = scan_f32(r01[x4]);
+    cv[4] = scan_f32(r10[x4]);
+    dv[4] = scan_f32(r11[x4]);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       // u000 = av[k], u001 = av[k+1] (x), u010 = bv[k] (y), u100 = cv[k] (z)
       const float g0 = ((av[k + 1] - av[k]) + (bv[k + 1] - bv[k])) + ((cv[k + 1] - cv[k]) + (dv[k + 1] - dv[k]));
       const float g1 = ((bv[k] - av[k]) + (bv[k + 1] - av[k + 1])) + ((dv[k] - cv[k]) + (dv[k + 1] - cv[k + 1]));
       const float g2 = ((cv[k] - av[k]) + (cv[k + 1] - av[k + 1])) + ((dv[k] - bv[k]) + (dv[k + 1] - bv[k + 1]));
-      m = fmaxf(m, g0 * g0 + g1 * g1 + g2 * g2);
+      m = fmaxf(m, sqrtf(g0 * g0 + g1 * g1 + g2 * g2));
       const float au = fabsf(av[k]);
-      um = (au <= FLT_MAX) ? fmaxf(um, au) : INFINITY;  // NaN or infinity: +inf
+      um = (au <= FLT_MAX) ? fmaxf(um, au) : INFINITY;  // NaN or infinity: infinity
     }
   }
-  float v[2] = {m, um};
-  block_reduce<float, 2, true, true>(v, sred);
-  if (publish_and_check_last<float>(v, 2, reinterpret_cast<float*>(partials), &ctrl->counter[CS_MID], &sflag)) {
-    float tt[2];
-    gather_partials<float, 2, true, true>(tt, reinterpret_cast<const float*>(partials), sred);
-    if (threadIdx.x == 0) {
-      ctrl->res_linf = (double)tt[0];
-      ctrl->res_l2 = (double)tt[1];
-      ctrl->counter[CS_MID] = 0;
+  unsigned mb = __float_as_uint(m), ub = __float_as_uint(um);  // of non-negative floats: ordered as integers
+  block_max2(mb, ub, smax);
+  if (threadIdx.x == 0) {
+    atomicMax(&ctrl->gmax2_hi, mb);
+    atomicMax(&ctrl->umax_hi, ub);
+    __threadfence();
+    sflag = atomicAdd(&ctrl->counter[CS_MISC], 1u) == gridDim.x - 1;
+    if (sflag) {
+      const double g = (double)__uint_as_float(atomicExch(&ctrl->gmax2_hi, 0u));
+      const double um2 = (double)__uint_as_float(atomicExch(&ctrl->umax_hi, 0u)) * (1.0 + 0x1p-19);
+      ctrl->umax = um2;
+      ctrl->gmax = g * (1.0 + 0x1p-18) + 0x1p-16 * um2;
+      ctrl->counter[CS_MISC] = 0;
+      fx_decide(ctrl, kp, ctrl->umax, ctrl->gmax, forced ? INFINITY : tol);
     }
   }
 }
@@ -528,11 +561,15 @@ cudaError_t launch_dot(const double* x, const double* y, const double* z, size_t
   k_dot<<<std::min(grid1d(n), 1024), NT, 0, st>>>(x, y, z, n, c, partials);
   return cudaGetLastError();
 }
-cudaError_t launch_gradmax(const float* u, const KParams& kp, Ctrl* ctrl, double* partials, cudaStream_t st) {
+template <typename T>
+cudaError_t launch_fx_scan(const T* u, const KParams& kp, double tol, bool forced, Ctrl* ctrl, cudaStream_t st) {
   const size_t n = (size_t)kp.nx * kp.ny * kp.nz;
-  k_gradmax<<<std::min(grid1d(n / 4), 1024), NT, 0, st>>>(u, kp, ctrl, partials);  // 3D, nx % 4 == 0
+  k_fx_scan<T><<<std::min(grid1d(n / 4), 1024), NT, 0, st>>>(u, kp, tol, forced ? 1 : 0, ctrl);
   return cudaGetLastError();
 }
+template cudaError_t launch_fx_scan<float>(const float*, const KParams&, double, bool, Ctrl*, cudaStream_t);
+template cudaError_t launch_fx_scan<double>(const double*, const KParams&, double, bool, Ctrl*, cudaStream_t);
+bool fx_stencils(const KParams& kp, int pk) { return pk == PK_4 && residual_geometry(kp, false).kind == RK_COL; }
 cudaError_t launch_thinfilm_rhs(const double* u, double* f, const KParams& kp, cudaStream_t st) {
   const size_t n = (size_t)kp.nx * kp.ny * kp.nz;
   k_thinfilm_rhs<<<grid1d(n), NT, 0, st>>>(u, f, kp);

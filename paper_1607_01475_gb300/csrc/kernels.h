@@ -27,9 +27,11 @@ struct AxisTables {
 // ----------------------------------------------------------------- DHT passes
 // 1D DHT of every line along x (contiguous rows), src -> dst (may alias),
 // multiplied by `scale`.  Skipped when *done != 0 (done may be null).
+// dmax_hi (FP64 only, may be null): its maximum with the high word of a bound on
+// the outputs.
 template <typename T>
 cudaError_t launch_dht_rows(const T* src, T* dst, int nx, int nrows, T scale, const int* done,
-                            const AxisTables<T>& tb, cudaStream_t st);
+                            const AxisTables<T>& tb, cudaStream_t st, unsigned int* dmax_hi = nullptr);
 
 // 1D DHT of every line along axis `ax` (1 = y, 2 = z), in place.
 template <typename T>
@@ -63,7 +65,8 @@ cudaError_t launch_mid(T* data, const KParams& kp, Ctrl* ctrl, double* partials,
                        const AxisTables<T>& tb, cudaStream_t st);
 #define PSD_DECL_PASSES(T)                                                                                      \
   template <>                                                                                                   \
-  cudaError_t launch_dht_rows<T>(const T*, T*, int, int, T, const int*, const AxisTables<T>&, cudaStream_t);    \
+  cudaError_t launch_dht_rows<T>(const T*, T*, int, int, T, const int*, const AxisTables<T>&, cudaStream_t,      \
+                                 unsigned int*);                                                               \
   template <>                                                                                                   \
   cudaError_t launch_dht_cols<T>(T*, const KParams&, int, T, const int*, const AxisTables<T>&, cudaStream_t);   \
   template <>                                                                                                   \
@@ -97,12 +100,8 @@ struct ResArgs {
   T* r;            // residual (order 6: local part, without T_h)
   int norm;        // 1: reduce ||r|| into ctrl and decide convergence
   int update_iter; // 1: this call advances the iteration count
-  int fluxff;      // FP64 plain without d, p = 4, 3D: fixed-point linear part and
-                   // float-float flux (see k_res3d_col)
-  int fxs;         // with fluxff: the fixed-point scale S (u = q 2^-S), in [15, 120]
-  const int* fxs_dev;  // or (non-null) S read from device memory at launch: the fixed-point
-                       // variant and the plain FP64 kernel are both launched and the one that
-                       // does not apply (S outside [15, 120] / inside) returns at once
+  int fixed;       // FP64 plain, p = 4, 3D column kernel: take the fixed-point variant with the
+                   // scales in ctrl (fx_s, fx_g) unless they say not to
 };
 
 // r = f - N_h^{loc}[u_in + alpha d] (plain) or
@@ -119,10 +118,15 @@ template <typename T>
 cudaError_t launch_linesearch(const T* u, const T* ubase, const T* d, int pk, const KParams& kp,
                               Ctrl* ctrl, double* partials, cudaStream_t st);
 
-// max over vertices of |G|^2, G the unscaled vertex gradient sums of the
-// FP32 field u (g = q G), into ctrl->res_linf (an estimate for choosing the
-// float-float flux of the FP64 residual).  3D grids with nx >= 32, ny >= 8.
-cudaError_t launch_gradmax(const float* u, const KParams& kp, Ctrl* ctrl, double* partials, cudaStream_t st);
+// Bounds on |u| and on the unscaled vertex gradient sums |G| (g = q G) of u into
+// ctrl->umax, gmax, and the scales of a fixed-point residual at u (fx_decide;
+// forced: without its error rule) into ctrl->fx_s, fx_g.  T: FP64, or FP32 for
+// the FP64 field that u rounds.  3D grids with nx a multiple of 4.
+template <typename T>
+cudaError_t launch_fx_scan(const T* u, const KParams& kp, double tol, bool forced, Ctrl* ctrl, cudaStream_t st);
+// Whether the FP64 residual and line search of this problem have the
+// fixed-point variants (p = 4 and the 3D column kernel).
+bool fx_stencils(const KParams& kp, int pk);
 // Right-hand side of the thin-film convex-splitting step (Sec. 6.1):
 // f = u - s Delta_h^v u (FP64, 2D and 3D).
 cudaError_t launch_thinfilm_rhs(const double* u, double* f, const KParams& kp, cudaStream_t st);
@@ -168,10 +172,6 @@ cudaError_t launch_mixed_check(Ctrl* c3, const Ctrl* c2, Ctrl* c, const Ctrl* tm
 // Mixed solve, after the inner solve: inner_total += c->iter, last alpha,
 // non-finite inner residual -> c3 failed (done).
 cudaError_t launch_mixed_after(Ctrl* c3, const Ctrl* c, cudaStream_t st);
-// Mixed solve: the choice of the fixed-point / float-float FP64 residual
-// (the host rule of the direct solve, on device) from the max |G|^2 and
-// max|u| estimates in c2 (res_linf, res_l2) into c3->fxs.
-cudaError_t launch_fluxff_decide(Ctrl* c3, const Ctrl* c2, double sqrt_vol, double cdiv, double tol, cudaStream_t st);
 // c = a fresh control block (tol -1, no iteration limit), on device.
 cudaError_t launch_ctrl_reset(Ctrl* c, cudaStream_t st);
 

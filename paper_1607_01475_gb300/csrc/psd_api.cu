@@ -40,6 +40,7 @@ constexpr int kChunk = 8;          // iterations enqueued between host checks (d
 constexpr int kBody = 2;           // iterations per WHILE-loop body of a captured solve
 static_assert(kBody % 2 == 0, "a loop body must start and end on the same ping-pong parity");
 constexpr int kCapDepth = 3;       // nesting of WHILE loops: outer, inner, general-p line search
+constexpr size_t kFxScanCells = 1 << 18;  // grids from here on scan u for the fixed-point residual's scales
 constexpr int kSolveGraphs = 4;    // solve graphs cached per handle (by pointer set)
 static_assert(kChunk % 2 == 0, "a chunk must start and end on the same ping-pong parity");
 constexpr int kLsPassesGen = 16;   // Newton passes of the general-p line search
@@ -361,6 +362,8 @@ void init_ctrl(Ctrl& h, double tol, int max_iter) {
   h.max_iter = max_iter;
   h.res_linf = -1.0;
   h.c2 = -1.0;
+  h.umax = -1.0;
+  h.fx_s = psd::kFxOff;
 }
 
 psd_status upload_ctrl(psd_context* c, Ctrl* dst, const Ctrl& h) {
@@ -432,7 +435,7 @@ psd_status precond_passes(psd_context* c, T* W, T* D, Ctrl* ctrl, T* xi, T* dspe
   if (kp.dim == 3) { ProfScope p_(c, cls_of<T>(PSD_PROF_DHT_COLS_FP64)); CK(psd::launch_dht_cols<T>(W, kp, 1, T(1), done, tb, c->st)); }
   { ProfScope p_(c, cls_of<T>(PSD_PROF_MID_FP64)); CK(psd::launch_mid<T>(W, kp, ctrl, c->partials, xi, dspec, tb, c->st)); }
   if (kp.dim == 3) { ProfScope p_(c, cls_of<T>(PSD_PROF_DHT_COLS_FP64)); CK(psd::launch_dht_cols<T>(W, kp, 1, T(1), done, tb, c->st)); }
-  { ProfScope p_(c, cls_of<T>(PSD_PROF_DHT_ROWS_FP64)); CK(psd::launch_dht_rows<T>(W, D, kp.nx, nrows, T(1), done, tb, c->st)); }
+  { ProfScope p_(c, cls_of<T>(PSD_PROF_DHT_ROWS_FP64)); CK(psd::launch_dht_rows<T>(W, D, kp.nx, nrows, T(1), done, tb, c->st, &ctrl->dmax_hi)); }
   return PSD_OK;
 }
 
@@ -567,53 +570,31 @@ psd_status ensure_fp32(psd_context* c) {
   return PSD_OK;
 }
 
-// Whether the FP64 residual of the current iterate (its FP32 copy in u32)
-// may take the fixed-point linear part and the float-float flux part: p = 4,
-// 3D column kernel, and a worst-case error bound of the flux part,
-//   |Omega|^{1/2} * 24 * 2^-47 * s q^4 * (2 max|G|)^3
-// (24 flux values per cell in the divergence, 2^-47 the double-word
-// precision, a factor 2 of margin on the FP32 estimate of max|G|), below
-// tol / 20.  *fxs receives the fixed-point scale S (0: plain FP64): with
-// max|u| < 2^e (max|u32| (1 + 2^-20) bounds it, as u32 = fl32(u)),
-// S = 55 - e keeps |q| = |u| 2^S below 2^55; S must lie in [15, 120].
-psd_status use_fluxff(psd_context* c, int* fxs) {
-  *fxs = 0;
-  const KParams& kp = c->kp;
-  if (c->pk != psd::PK_4 || kp.dim != 3 || kp.nx < 32 || kp.ny < 8 || !(c->prm.tol > 0)) return PSD_OK;
-  Ctrl h;
-  init_ctrl(h, -1.0, 1 << 30);
-  TRY(upload_ctrl(c, c->ctrl2, h));
-  { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_gradmax(c->u32, kp, c->ctrl2, c->partials, c->st)); }
-  Ctrl h2;
-  TRY(read_ctrl(c, c->ctrl2, h2));
-  const double gmax = 2.0 * std::sqrt(std::max(h2.res_linf, 0.0));
-  const double bound = std::sqrt((double)c->N * kp.hd) * 24.0 * std::ldexp(1.0, -47) * kp.cdiv * gmax * gmax * gmax;
-  const double umax = h2.res_l2;
-  if (!(std::isfinite(bound) && bound < 0.05 * c->prm.tol) || !std::isfinite(umax)) return PSD_OK;
-  int e = 0;
-  if (umax > 0.0) std::frexp(umax * (1.0 + std::ldexp(1.0, -20)), &e);  // umax (1 + 2^-20) < 2^e
-  const int S = 55 - e;
-  if (S >= 15 && S <= 120) *fxs = S;
+// Whether a residual at a fresh iterate is worth a scan for the scales of its
+// fixed-point variant (a launch that reads u): the variant exists and the grid is
+// large enough for the FP64 variant to cost more.
+bool fx_scan_pays(const psd_context* c) { return psd::fx_stencils(c->kp, c->pk) && c->N >= kFxScanCells; }
+// Scales of the fixed-point residual at u into ctrl (without a scan: the FP64 variant).
+psd_status fx_scan(psd_context* c, const double* u, const float* u32, Ctrl* ctrl) {
+  if (!fx_scan_pays(c)) return PSD_OK;
+  ProfScope p_(c, PSD_PROF_OTHER);
+  if (u32)
+    CK(psd::launch_fx_scan<float>(u32, c->kp, c->prm.tol, false, ctrl, c->st));
+  else
+    CK(psd::launch_fx_scan<double>(u, c->kp, c->prm.tol, false, ctrl, c->st));
   return PSD_OK;
-}
-
-// Whether the FP64 outer residuals of this handle may take the fixed-point /
-// float-float variant at all (the per-iterate bound is checked on device in
-// graph mode, by use_fluxff in direct mode).
-bool fluxff_eligible(const psd_context* c) {
-  const KParams& kp = c->kp;
-  return c->pk == psd::PK_4 && kp.dim == 3 && kp.nx >= 32 && kp.ny >= 8 && c->prm.tol > 0;
 }
 
 // FP64 residual r = f - N_h[u] into r (order 6: P0[...] including T_h[u - g]),
 // norms into ctrl2 (res_l2, res_linf), all enqueued (ctrl2 reset on device).
-// fxs: fixed-point scale from the host (direct mode); fxs_dev: from device
-// memory (graph mode).  Uses W, Z as scratch (order 6).
-psd_status residual64(psd_context* c, const double* u, const double* f, const double* g, double* r, int fxs = 0,
-                      const int* fxs_dev = nullptr) {
+// u32: the FP32 copy of u where there is one (its scan reads half the bytes).
+// Uses W, Z as scratch (order 6).
+psd_status residual64(psd_context* c, const double* u, const double* f, const double* g, double* r,
+                      const float* u32 = nullptr) {
   const KParams& kp = c->kp;
   CK(psd::launch_ctrl_reset(c->ctrl2, c->st));
-  ResArgs<double> a{u, nullptr, nullptr, f, nullptr, r, kp.order == 4 ? 1 : 0, 0, fxs ? 1 : 0, fxs, fxs_dev};
+  TRY(fx_scan(c, u, u32, c->ctrl2));
+  ResArgs<double> a{u, nullptr, nullptr, f, nullptr, r, kp.order == 4 ? 1 : 0, 0, 1};
   { ProfScope p_(c, PSD_PROF_RESIDUAL_FP64); CK(psd::launch_residual<double>(a, psd::RM_PLAIN, c->pk, kp, c->ctrl2, c->partials, c->st)); }
   if (kp.order == 6) {
     // r <- P0[r_loc - T_h[u - g]] through the spectrum
@@ -632,11 +613,11 @@ psd_status residual64(psd_context* c, const double* u, const double* f, const do
 // with theta = DHT(T_h[u - g]) in Z (the subtraction, the rounding and the
 // Parseval norm fused into the last transform pass); ||R||_2 into
 // ctrl2->res_l2 (enqueued).
-psd_status outer_residual6_spec(psd_context* c, const double* u, const double* f, int fxs,
-                                const int* fxs_dev = nullptr) {
+psd_status outer_residual6_spec(psd_context* c, const double* u, const double* f) {
   const KParams& kp = c->kp;
   CK(psd::launch_ctrl_reset(c->ctrl2, c->st));
-  ResArgs<double> a{u, nullptr, nullptr, f, nullptr, c->W, 0, 0, fxs ? 1 : 0, fxs, fxs_dev};
+  TRY(fx_scan(c, u, c->u32, c->ctrl2));
+  ResArgs<double> a{u, nullptr, nullptr, f, nullptr, c->W, 0, 0, 1};
   { ProfScope p_(c, PSD_PROF_RESIDUAL_FP64); CK(psd::launch_residual<double>(a, psd::RM_PLAIN, c->pk, kp, c->ctrl2, c->partials, c->st)); }
   const int nrows = kp.ny * kp.nz;
   double* x = c->W;  // transformed in place
@@ -657,7 +638,8 @@ psd_status fp64_start(psd_context* c, const double* f, const double* g, double* 
     TRY(full_dht<double>(c, c->Z, 1.0, c->tb64));
     { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_spec_apply_T<double>(c->Z, -1.0, kp, c->tb64, c->st)); }
   }
-  ResArgs<double> a{u, nullptr, nullptr, f, nullptr, c->W, kp.order == 4 ? 1 : 0, 0};
+  TRY(fx_scan(c, u, nullptr, c->ctrl));
+  ResArgs<double> a{u, nullptr, nullptr, f, nullptr, c->W, kp.order == 4 ? 1 : 0, 0, 1};
   { ProfScope p_(c, PSD_PROF_RESIDUAL_FP64); CK(psd::launch_residual<double>(a, psd::RM_PLAIN, c->pk, kp, c->ctrl, c->partials, c->st)); }
   return PSD_OK;
 }
@@ -671,7 +653,7 @@ psd_status fp64_iterations(psd_context* c, const double* f, double* u, int count
     double* nxt = (i % 2 == 0) ? c->ub : u;
     TRY(precond_passes<double>(c, c->W, c->D, c->ctrl, c->Z, c->Dsp, c->tb64));
     TRY(linesearch<double>(c, cur, nullptr, c->D, c->ctrl));
-    ResArgs<double> a{cur, c->D, nxt, f, nullptr, c->W, kp.order == 4 ? 1 : 0, 1};
+    ResArgs<double> a{cur, c->D, nxt, f, nullptr, c->W, kp.order == 4 ? 1 : 0, 1, 1};
     { ProfScope p_(c, PSD_PROF_RESIDUAL_FP64); CK(psd::launch_residual<double>(a, psd::RM_PLAIN, c->pk, kp, c->ctrl, c->partials, c->st)); }
   }
   return PSD_OK;
@@ -855,23 +837,15 @@ psd_status mixed_start(psd_context* c, const double* g, double* u) {
 psd_status mixed_graph_body(psd_context* c, const double* f, const double* g, double* u) {
   const KParams& kp = c->kp;
   const bool six = kp.order == 6;
-  const bool elig = fluxff_eligible(c);
   TRY(mixed_start(c, g, u));
   const int guard_outer = std::max(c->prm.max_outer, 1) + 3;
   const int inner_cap = std::min(std::max(c->prm.max_iter, 1), kInnerMaxIter);
   const int guard_inner = inner_cap / kBody + 3;
   return capture_while(c, [&](cudaGraphConditionalHandle ho) -> psd_status {
-    const int* fxs_dev = nullptr;
-    if (elig) {
-      CK(psd::launch_ctrl_reset(c->ctrl2, c->st));
-      { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_gradmax(c->u32, kp, c->ctrl2, c->partials, c->st)); }
-      CK(psd::launch_fluxff_decide(c->ctrl3, c->ctrl2, std::sqrt((double)c->N * kp.hd), kp.cdiv, c->prm.tol, c->st));
-      fxs_dev = &c->ctrl3->fxs;
-    }
     if (six) {
-      TRY(outer_residual6_spec(c, u, f, 0, fxs_dev));
+      TRY(outer_residual6_spec(c, u, f));
     } else {
-      TRY(residual64(c, u, f, g, c->W, 0, fxs_dev));
+      TRY(residual64(c, u, f, g, c->W, c->u32));
       { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_round_f32(c->R32, c->W, c->N, c->st)); }
     }
     CK(psd::launch_mixed_check(c->ctrl3, c->ctrl2, c->ctrl, c->ctrl_tmpl, c->prm.tol, c->prm.max_iter,
@@ -941,14 +915,12 @@ psd_status solve_mixed(psd_context* c, const double* f, const double* g, double*
       if (six) TRY(dht_theta(c, nullptr, c->da, dsum));
       { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_accumulate_f64(u, c->da, c->u32, c->N, dsum, c->st)); }
     }
-    int fxs = 0;
-    TRY(use_fluxff(c, &fxs));
     if (six) {
       // the outer residual stays in the transform domain; the inner solve adds
       // it to its own transformed residual in the middle pass
-      TRY(outer_residual6_spec(c, u, f, fxs));
+      TRY(outer_residual6_spec(c, u, f));
     } else {
-      TRY(residual64(c, u, f, g, c->W, fxs));
+      TRY(residual64(c, u, f, g, c->W, c->u32));
     }
     Ctrl h2;
     TRY(read_ctrl(c, c->ctrl2, h2));
@@ -1456,16 +1428,19 @@ psd_status psd_residual_fixed(psd_handle c, const double* u, const double* f, do
   init_ctrl(h, -1.0, 1 << 30);
   TRY(upload_ctrl(c, c->ctrl2, h));
   { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_norms(u, c->N, kp.hd, c->ctrl2, c->partials, c->st)); }
+  { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_fx_scan<double>(u, kp, c->prm.tol, true, c->ctrl2, c->st)); }
   Ctrl h2;
   TRY(read_ctrl(c, c->ctrl2, h2));
   const double umax = h2.res_linf;
-  if (!std::isfinite(umax)) return PSD_OK;
+  if (!std::isfinite(umax) || h2.fx_s == psd::kFxOff) return PSD_OK;
   int e = 0;
   if (umax > 0.0) std::frexp(umax * (1.0 + std::ldexp(1.0, -20)), &e);
   const int S = 55 - e;
   if (S < 15 || S > 120) return PSD_OK;
-  TRY(upload_ctrl(c, c->ctrl2, h));
-  ResArgs<double> a{u, nullptr, nullptr, f, nullptr, r, 0, 0, 1, S};
+  h2.fx_g += h2.fx_s - S;  // the scan's bound on |u| may be the next power of two
+  h2.fx_s = S;
+  TRY(upload_ctrl(c, c->ctrl2, h2));
+  ResArgs<double> a{u, nullptr, nullptr, f, nullptr, r, 0, 0, 1};
   { ProfScope p_(c, PSD_PROF_RESIDUAL_FP64); CK(psd::launch_residual<double>(a, psd::RM_PLAIN, c->pk, kp, c->ctrl2, c->partials, c->st)); }
   CK(cudaStreamSynchronize(c->st));
   *scale = S;
@@ -1643,7 +1618,8 @@ psd_status psd_adjoint(psd_handle c, const double* u, const double* grad_u, doub
     Ctrl hz;
     init_ctrl(hz, -1.0, 1 << 30);
     TRY(upload_ctrl(c, c->ctrl2, hz));
-    ResArgs<double> a{u, nullptr, nullptr, nullptr, nullptr, c->W, 0, 0};
+    TRY(fx_scan(c, u, nullptr, c->ctrl2));
+    ResArgs<double> a{u, nullptr, nullptr, nullptr, nullptr, c->W, 0, 0, 1};
     { ProfScope p_(c, PSD_PROF_RESIDUAL_FP64); CK(psd::launch_residual<double>(a, psd::RM_PLAIN, c->pk, kp, c->ctrl2, c->partials, c->st)); }
     { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_dot(lam, c->W, u, c->N, c->ctrl2, c->partials, c->st)); }
     Ctrl o;

@@ -56,12 +56,19 @@ struct Ctrl {
   int ls_pass;      // general-p line search: Newton passes of this iteration
   int outer;        // mixed solve: FP64 outer residual evaluations
   int inner_total;  // mixed solve: inner iterations so far
-  int fxs;          // mixed solve: fixed-point scale of the next outer residual (0: plain FP64)
   int max_outer;
+  int cfg_pad_;
   double last_alpha;
   unsigned int counter[CS_COUNT];
+  // FP64 p = 4 stencils in 3D (fixed-point variants): bounds on |u| and on the
+  // vertex gradient sums |G| of the last residual's iterate (umax < 0: none),
+  // the high word of a bound on |d| (the x pass that ends the preconditioner),
+  // the scales of the next residual (fx_s = kFxOff: the FP64 variant), and
+  // running maxima (high words of bounds, zero between kernels)
+  double umax, gmax;
+  unsigned int dmax_hi, umax_hi, gmax2_hi;
+  int fx_s, fx_g;
   int hist_cap;
-  int pad_;
   double* hist_alpha;  // device arrays of length hist_cap (or null)
   double* hist_res;
 };
@@ -145,7 +152,64 @@ inline void finish_kparams(KParams& kp) {
   f.pm2 = (float)d.pm2;
 }
 
+// -------------------------------------------- scales of the fixed-point stencils
+constexpr int kFxOff = -10000;
+
+// The scale S with |v| 2^S < 2^55 for |v| <= vmax (1 + 2^-20); false when vmax
+// is not finite or S is outside [-200, 200].
+__device__ __forceinline__ bool fx_scale_of(double vmax, int* S) {
+  if (!isfinite(vmax)) return false;
+  int e = 0;
+  if (vmax > 0.0) frexp(vmax * (1.0 + 0x1p-20), &e);
+  *S = 55 - e;
+  return *S >= -200 && *S <= 200;
+}
+// The shift g of the gradient sums for |G| <= gmax (1 + 2^-20): |G| 2^(S+g) < 2^61.
+// (|G| < 16 max|u|, so g >= 2.)
+__device__ __forceinline__ int fx_shift_of(double gmax, int S, int* ge) {
+  int e = 0;
+  if (gmax > 0.0) frexp(gmax * (1.0 + 0x1p-20), &e);
+  const int g = gmax > 0.0 ? 61 - S - e : 60;
+  *ge = 61 - S - (g < 2 ? 2 : (g > 60 ? 60 : g));
+  return g < 2 ? 2 : (g > 60 ? 60 : g);
+}
+// Choose the scales of a fixed-point residual for |u| <= umax, |G| <= gmax into
+// c.  Its flux error is at most cdiv 2^-51 2^(3 ge) per cell (24 fluxes of a few
+// units of 2^-58 of the cube of 2^ge >= |G|); the variant runs when that is below
+// the FP64 rounding of the Laplacian sums, about 64 units 2^-53 of cbih max|u|,
+// or, in the 2-norm, below tol / 20.  Otherwise (gradients steeper than any
+// smooth field on the grid) the FP64 variant runs.
+template <class C, class K>
+__device__ __forceinline__ void fx_decide(C* c, const K& kp, double umax, double gmax, double tol) {
+  int S = kFxOff, g = 0, ge = 0;
+  if (!(umax >= 0.0) || !isfinite(gmax) || !fx_scale_of(umax, &S)) {
+    c->fx_s = kFxOff;
+    return;
+  }
+  g = fx_shift_of(gmax, S, &ge);
+  const double err = kp.cdiv * ldexp(1.0, 3 * ge - 51);
+  const bool ok = umax == 0.0 || err <= 64.0 * 0x1p-53 * kp.cbih * umax || err * sqrt(kp.hd / kp.inv_ntot) < 0.05 * tol;
+  c->fx_s = ok ? S : kFxOff;
+  c->fx_g = g;
+}
+
 // ------------------------------------------------------------------ reductions
+
+// Block maxima of two values, for every thread (one-dimensional blocks of
+// whole warps); sh: two words of shared memory.
+__device__ __forceinline__ void block_max2(unsigned& a, unsigned& b, unsigned* sh) {
+  if (threadIdx.x < 2) sh[threadIdx.x] = 0u;
+  __syncthreads();
+  a = __reduce_max_sync(0xffffffffu, a);
+  b = __reduce_max_sync(0xffffffffu, b);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&sh[0], a);
+    atomicMax(&sh[1], b);
+  }
+  __syncthreads();
+  a = sh[0];
+  b = sh[1];
+}
 
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {

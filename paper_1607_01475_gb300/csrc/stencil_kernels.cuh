@@ -21,6 +21,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "fx_line.cuh"
 #include "stencil_geom.h"
 
 namespace psd {
@@ -560,10 +561,11 @@ __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double 
 }
 
 // Block and grid reduction of a line-search pass (fixed order; the last
-// block runs the epilogue).  sred: 32 * ls_nsums<PK>() shared elements.
+// block runs the epilogue).  fx_tol >= 0: the scales of the residual that
+// follows are chosen from the bounds in ctrl (fx_decide).  sred: 32 * ls_nsums<PK>() shared elements.
 template <typename T, int PK>
 __device__ __forceinline__ void ls_finish(T (&acc)[ls_nsums<PK>()], T* sred, double* partials, Ctrl* ctrl,
-                                          const KParams& kp, int* sflag) {
+                                          const KParams& kp, int* sflag, double fx_tol = -1.0) {
   constexpr int M = ls_nsums<PK>();
   block_reduce<T, M, false>(acc, sred);
   if (publish_and_check_last<T>(acc, M, reinterpret_cast<T*>(partials), &ctrl->counter[CS_LS], sflag)) {
@@ -575,6 +577,11 @@ __device__ __forceinline__ void ls_finish(T (&acc)[ls_nsums<PK>()], T* sred, dou
 #pragma unroll
       for (int m = 0; m < M; ++m) tot[m] = (double)tt[m];
       linesearch_epilogue<PK>(ctrl, kp, tot);
+      if (fx_tol >= 0.0) {
+        // the next iterate u + alpha d: |u| and |G| are at most these
+        const double al = fabs(ctrl->alpha), gd = sqrt(__hiloint2double((int)atomicExch(&ctrl->gmax2_hi, 0u), 0));
+        fx_decide(ctrl, kp, ctrl->umax + al * __hiloint2double((int)ctrl->dmax_hi, 0), ctrl->gmax + al * gd, fx_tol);
+      }
     }
   }
 }
@@ -693,18 +700,6 @@ cudaError_t res_impl(const ResArgs<T>& a, const KParams& kp, Ctrl* ctrl, double*
       if constexpr (sizeof(T) == 4) k_res3d_rb<T, PK, MODE, 4><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials);
       break;
     case RK_COL:
-      if constexpr (sizeof(T) == 8 && MODE == RM_PLAIN && PK == PK_4) {
-        if (a.fxs_dev != nullptr && a.d == nullptr) {
-          // both variants; the one that does not apply returns at once
-          k_res3d_col<T, PK, MODE, true><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials);
-          k_res3d_col<T, PK, MODE><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials);
-          break;
-        }
-        if (a.fluxff && a.d == nullptr && a.fxs >= 15 && a.fxs <= 120) {
-          k_res3d_col<T, PK, MODE, true><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials);
-          break;
-        }
-      }
       k_res3d_col<T, PK, MODE><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials);
       break;
     case RK_SMALL3D:

@@ -3,7 +3,8 @@
 // kernels, run thread by thread for every length, against a long-double
 // transform.  For each kind of line its error (2-norm, relative) must not exceed
 // that of the same Stockham passes in FP64; and the conversions, the special
-// values and the extremes of the exponent range are checked.  Built and run by
+// values and the extremes of the exponent range are checked; so is the flux of
+// the fixed-point residual.  Built and run by
 // tests/test_fx_line.py (no GPU needed).  Exit status 0 = pass.
 #include <cmath>
 #include <cstdint>
@@ -257,6 +258,26 @@ int main() {
     const double r = psd::fx_result(w, e);
     const long double want = ldexpl((long double)w, e);
     if (fabsl(r - want) > fabsl(want) * 0x1p-53L) ++fails;
+  }
+  // p = 4 flux: moduli up to the bound 2^61, within 4 units of |G|^2 G 2^-125
+  for (int t = 0; t < 200000; ++t) {
+    const int sh = t < 1000 ? 0 : (int)(next_u64() % 40);
+    long double g[3], n = 0;
+    long long q[3], F[3];
+    for (auto& v : g) {
+      v = uni();
+      n += v * v;
+    }
+    if (t < 8) g[0] = (t & 1) ? -1 : 1, g[1] = (t & 2) ? 1e-9L : 0, g[2] = (t & 4) ? -1e-9L : 0, n = 1.0000000001L;
+    for (int c = 0; c < 3; ++c) q[c] = (long long)(g[c] / sqrtl(n) * ldexpl(1.0L, 61 - sh));
+    const unsigned top = psd::fx_flux(q[0], q[1], q[2], F);
+    long double m = 0;
+    for (int c = 0; c < 3; ++c) m += (long double)q[c] * q[c];
+    if (ldexpl((long double)top + 1, 96) < m) ++fails;
+    for (int c = 0; c < 3; ++c) {
+      const long double want = ldexpl(m * q[c], -125);
+      if (fabsl(F[c] - want) > 4.0L || fabsl((long double)F[c]) > 0x1p58L) ++fails;
+    }
   }
   check<8>();
   check<16>();

@@ -1,7 +1,10 @@
-"""FP64 transform passes in block fixed point on the GPU: every line length on
+"""Fixed-point FP64 kernels on the GPU.  Transform passes: every line length on
 every axis (one, several and part of a warp per line pair; full and narrowed
 tiles) against the oracle's preconditioner, and lines that are zero, tiny or
-not finite.
+not finite.  p = 4 stencils in 3D: residuals and PSD iterates on the smallest
+column tiles, on several and on grids large enough for the initial scan, with
+smooth data (the fixed-point variant), with gradients steeper than its rule
+allows (the FP64 variant) and with an offset much larger than the gradients.
 
 Tolerance 1e-12 relative L-infinity, as for every FP64 output of the parity
 tests (rounding of a few eps64 per pass, relative to the largest value).
@@ -16,7 +19,7 @@ pytestmark = pytest.mark.gpu
 if not torch.cuda.is_available():  # pragma: no cover - collected on CPU hosts
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
-from paper_1607_01475_gb300 import Solver  # noqa: E402
+from paper_1607_01475_gb300 import Solver, synthetic  # noqa: E402
 
 SHAPES = [(8, 8), (8, 1024), (1024, 8), (512, 16), (16, 512), (128, 32), (32, 128), (8, 8, 1024), (8, 1024, 8),
           (1024, 8, 8), (512, 8, 16), (16, 512, 8), (8, 16, 512), (64, 32, 16), (128, 64, 8), (8, 128, 256)]
@@ -53,3 +56,54 @@ def test_precond_zero_scaled_and_nonfinite_lines():
     r[1, 1, 1] = float("nan")
     S.precond_solve(r, d)
     assert torch.isnan(d).all()
+
+
+FIELDS = {"smooth": (1.0, 0.0, 0.0), "rough": (0.0, 0.3, 0.0), "steep": (0.0, 40.0, 0.0), "offset": (0.1, 0.0, 100.0)}
+
+
+def _field(shape, kind, seed):
+    smooth, noise, offset = FIELDS[kind]
+    u = np.full(shape, offset)
+    if smooth:
+        u += smooth * synthetic.fourier_field(shape, 2 * np.pi, 4, seed, nmodes=12)
+    if noise:
+        u += noise * np.random.default_rng(seed).standard_normal(shape)
+    return u
+
+
+@pytest.mark.parametrize("shape", [(8, 8, 32), (16, 8, 64), (64, 64, 64), (16, 128, 128)])
+@pytest.mark.parametrize("kind", sorted(FIELDS))
+@pytest.mark.parametrize("order", [4, 6])
+def test_residual_variants(oracle, shape, kind, order):
+    h = 2 * np.pi / shape[-1]
+    P = oracle.Problem(order, h, 4.0, 0.1, 0.1, 0.7)
+    u, f = _field(shape, kind, 3), _field(shape, "smooth", 4)
+    g = _field(shape, "smooth", 5) if order == 6 else None
+    if order == 6:
+        u += g.mean() - u.mean()
+    S = Solver(order, shape, h, 4.0, P.s, P.eps, P.lam)
+    r = torch.empty(shape, dtype=torch.float64, device="cuda")
+    S.residual(torch.from_numpy(u).cuda(), torch.from_numpy(f).cuda(), None if g is None else torch.from_numpy(g).cuda(), r)
+    ref = oracle.residual4(u, f, P) if order == 4 else oracle.residual6(u, f, g, P)
+    # the residual of a large offset cancels: its rounding is that of the terms
+    scale = max(np.max(np.abs(ref)), np.max(np.abs(u)) * (1.0 + 64.0 * P.s * P.eps ** 2 / h ** 4))
+    assert np.max(np.abs(r.cpu().numpy() - ref)) <= 1e-12 * np.max(np.abs(ref)) + 1e-15 * scale
+
+
+@pytest.mark.parametrize("shape", [(8, 8, 32), (16, 16, 64), (64, 64, 64)])
+@pytest.mark.parametrize("kind", ["smooth", "rough", "steep"])
+@pytest.mark.parametrize("order", [4, 6])
+def test_iterates_variants(oracle, shape, kind, order):
+    h = 2 * np.pi / shape[-1]
+    P = oracle.Problem(order, h, 4.0, 0.1, 0.1, 0.7)
+    u0, f = _field(shape, kind, 6), _field(shape, "smooth", 7)
+    g = _field(shape, "smooth", 8) if order == 6 else None
+    if order == 6:
+        u0 += g.mean() - u0.mean()
+    iters = 3
+    S = Solver(order, shape, h, 4.0, P.s, P.eps, P.lam, tol=0.0, max_iter=iters)
+    u = torch.from_numpy(u0).cuda()
+    S.solve(torch.from_numpy(f).cuda(), u, None if g is None else torch.from_numpy(g).cuda(), allow_noconv=True)
+    _, info = oracle.psd_solve(P, f, u0, g=g, tol=0.0, kmax=iters, record=True)
+    ref = info["u"][iters]
+    assert np.max(np.abs(u.cpu().numpy() - ref)) <= 1e-12 * np.max(np.abs(ref))
