@@ -144,17 +144,6 @@ __device__ __forceinline__ double fx_leave(fx w, const FxLine& ln, int scale_e) 
                           : fx_result(w.v, ln.E - ln.B + FxPlan<N>::kOut + scale_e);
 }
 
-// 1/x for finite x > 0 (the symbols): the hardware estimate (relative error
-// below 2^-20) with one cubic step r (1 + e + e^2), e = 1 - x r: within an
-// ulp of 1/x in three FP64 operations.
-__device__ __forceinline__ double recip_pos(double x) {
-  if ((unsigned)__double2hiint(x) >= 0x7FE00000u) return 1.0 / x;  // 2^1023 and above, infinity, NaN
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-
 // -------------------------------------------------------------- x (rows)
 template <int N, typename SI>
 __global__ void __launch_bounds__(kFxThreads, 3)
@@ -299,7 +288,7 @@ __global__ void __launch_bounds__(kFxThreads, 3)
   if (skip != nullptr && *skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint2 scr[kFxThreads / 32][32];
-  __shared__ float sred[32];
+  __shared__ float sred[red_size<float>(1)];
   __shared__ int sflag;
   const int tid = threadIdx.x;
   const int pairs = blockDim.x / TS;
@@ -386,7 +375,7 @@ __global__ void __launch_bounds__(kFxThreads, 2)
   if (ctrl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint2 scr[kFxThreads / 32][32];
-  __shared__ double sred[32 * 5];
+  __shared__ double sred[red_size<double>(3)];
   __shared__ int sflag;
   const int tid = threadIdx.x;
   const int pairs = blockDim.x / TS;
@@ -420,7 +409,7 @@ __global__ void __launch_bounds__(kFxThreads, 2)
   const double alpha_prev = ORDER == 6 ? ctrl->alpha : 0.0;
   const double mo = symo != nullptr ? symo[yo] : 0.0;
   const double mxa = symx[x] + mo, mxb = symx[x + 1] + mo;
-  double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  double acc[mid_nsums<double, ORDER>()] = {};
 #pragma unroll
   for (int q = 0; q < R; ++q) {
     const int kk = j + q * TS;
@@ -437,8 +426,7 @@ __global__ void __launch_bounds__(kFxThreads, 2)
         const double m = mu * d;
         dv[c] = d;
         acc[0] = fma(h, d, acc[0]);
-        acc[1] = fma(d, d, acc[1]);
-        acc[2] = fma(m, m, acc[2]);
+        acc[1] = fma(m, d, acc[1]);
       }
     } else {
       // xi advances with the previous step and is added to the transformed
@@ -464,10 +452,8 @@ __global__ void __launch_bounds__(kFxThreads, 2)
         tn[c] = td;
         dv[c] = d;
         acc[0] = fma(rt, d, acc[0]);
-        acc[1] = fma(d, d, acc[1]);
-        acc[2] = fma(m, m, acc[2]);
-        acc[3] = fma(d, td, acc[3]);
-        acc[4] = fma(rt, rt, acc[4]);
+        acc[1] = fma(m, d, acc[1]);
+        acc[mid_nsums<double, ORDER>() - 1] = fma(rt, rt, acc[mid_nsums<double, ORDER>() - 1]);
       }
       *reinterpret_cast<double2*>(xi_ + idx) = make_double2(xn[0], xn[1]);
       *reinterpret_cast<double2*>(dspec + idx) = make_double2(tn[0], tn[1]);

@@ -151,24 +151,32 @@ __global__ void __launch_bounds__(kThreads, 3)  // 80 registers
   }
 }
 
-// Block and grid reduction of the middle pass's five Parseval sums (fixed
-// order) and the last block's bookkeeping: the sums into ctrl, the inner
-// stopping rule on the preconditioned norm, the order-6 residual norm and
-// convergence test, and the reset of the line-search state.
+// Block and grid reduction of the middle pass's Parseval sums (fixed order) and
+// the last block's bookkeeping: the sums into ctrl, the inner stopping rule on
+// the preconditioned norm, the order-6 residual norm and convergence test, and
+// the reset of the line-search state.  FP32 sums: (r, d), (d, d), (Delta d,
+// Delta d), (T_h d, d), (r, r).  FP64, where every sum costs: (r, d), z = sum mu
+// d^2 and (order 6) (r, r); L_h r = d gives q's linear part as (r, d) - s z, a
+// difference whose terms are all positive sums of the same spectrum.
 template <typename T, int ORDER>
-__device__ __forceinline__ void mid_finish(T (&acc)[5], T* sred, double* partials, Ctrl* ctrl, const KParams& kp,
-                                           int* sflag_) {
+__host__ __device__ constexpr int mid_nsums() {
+  return sizeof(T) == 4 ? 5 : (ORDER == 6 ? 3 : 2);
+}
+template <typename T, int ORDER>
+__device__ __forceinline__ void mid_finish(T (&acc)[mid_nsums<T, ORDER>()], T* sred, double* partials, Ctrl* ctrl,
+                                           const KParams& kp, int* sflag_) {
+  constexpr int M = mid_nsums<T, ORDER>();
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
   int& sflag = *sflag_;
-  T v[5];
+  T v[M];
 #pragma unroll
-  for (int m = 0; m < 5; ++m) v[m] = acc[m];
-  block_reduce<T, 5, false>(v, sred);
-  if (publish_and_check_last<T>(v, 5, reinterpret_cast<T*>(partials), &ctrl->counter[CS_MID], &sflag)) {
-    T tt[5];
-    gather_partials<T, 5, false>(tt, reinterpret_cast<const T*>(partials), sred);
-    double tot[5];
-    for (int m_ = 0; m_ < 5; ++m_) tot[m_] = (double)tt[m_];
+  for (int m = 0; m < M; ++m) v[m] = acc[m];
+  block_reduce<T, M, false>(v, sred);
+  if (publish_and_check_last<T>(v, M, reinterpret_cast<T*>(partials), &ctrl->counter[CS_MID], &sflag)) {
+    T tt[M];
+    gather_partials<T, M, false>(tt, reinterpret_cast<const T*>(partials), sred);
+    double tot[M];
+    for (int m_ = 0; m_ < M; ++m_) tot[m_] = (double)tt[m_];
     if (tid == 0 && ctrl->cg) {
       // conjugate gradients: z = L_h^{-1} r was just formed; beta = (r, z) /
       // (r, z)_previous goes to alpha for the direction update p = z + beta p
@@ -185,9 +193,10 @@ __device__ __forceinline__ void mid_finish(T (&acc)[5], T* sred, double* partial
     } else if (tid == 0) {
       const double w = kp.hd * kp.inv_ntot;
       ctrl->rd = tot[0] * w;
-      ctrl->dd = tot[1] * w;
-      ctrl->lapdd = tot[2] * w;
-      ctrl->tdd = tot[3] * w;
+      if constexpr (sizeof(T) == 4)
+        ctrl->lin = (kp.cu * tot[1] + tot[3] + kp.s * kp.eps2 * tot[2]) * w;
+      else
+        ctrl->lin = (tot[0] - kp.s * tot[1]) * w;
       if (ctrl->pre_eta > 0.0) {
         // inner solve: stop when the preconditioned norm has dropped by
         // pre_eta, or when it has stopped halving (its rounding floor)
@@ -208,7 +217,7 @@ __device__ __forceinline__ void mid_finish(T (&acc)[5], T* sred, double* partial
         }
       }
       if (ORDER == 6) {
-        const double res = sqrt(tot[4] * w);
+        const double res = sqrt(tot[M - 1] * w);
         ctrl->res_l2 = res;
         ctrl->res_linf = -1.0;
         const int it = ctrl->iter;
@@ -254,7 +263,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   if (ctrl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
-  __shared__ T sred[32 * 5];
+  __shared__ T sred[red_size<T>(5)];
   __shared__ int sflag;
   const int tid = threadIdx.x;
   const int pairs = blockDim.x / F::TS;
@@ -436,7 +445,7 @@ __global__ void k_spec6_combine(T* a, const T* b, KParams kp, const T* sx, const
 template <typename T>
 __global__ void __launch_bounds__(256) k_spec_quad(const T* a, KParams kp, const T* sx, const T* sy, const T* sz,
                                                    size_t n, Ctrl* ctrl, double* partials) {
-  __shared__ double sred[32];
+  __shared__ double sred[red_size<double>(1)];
   __shared__ int sflag;
   double acc = 0.0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {

@@ -102,6 +102,10 @@ __host__ __device__ __forceinline__ unsigned fx_flux(long long g0, long long g1,
   return (unsigned)((unsigned long long)s >> 32);
 }
 
+__host__ __device__ __forceinline__ long long fx_shl(long long v, int k) {
+  return (long long)((unsigned long long)v << k);
+}
+
 // The 64 bits of a value.
 __device__ __forceinline__ unsigned long long fx_bits(long long v) { return (unsigned long long)v; }
 __device__ __forceinline__ unsigned long long fx_bits(double v) { return (unsigned long long)__double_as_longlong(v); }

@@ -57,6 +57,18 @@ __global__ void __launch_bounds__(NT) k_fx_scan(const T* __restrict__ u, KParams
     float av[5], bv[5], cv[5], dv[5];
     scan_load(r00 + x, av);
     scan_load(r01 + x, bv);
+    if (kp.dim == 2) {  // G_x = D(y) + D(y+1), G_y = A(y+1) - A(y)
+      av[4] = scan_f32(r00[x4]);
+      bv[4] = scan_f32(r01[x4]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float g0 = (av[k + 1] - av[k]) + (bv[k + 1] - bv[k]), g1 = (bv[k] - av[k]) + (bv[k + 1] - av[k + 1]);
+        m = fmaxf(m, sqrtf(g0 * g0 + g1 * g1));
+        const float au = fabsf(av[k]);
+        um = (au <= FLT_MAX) ? fmaxf(um, au) : INFINITY;
+      }
+      continue;
+    }
     scan_load(r10 + x, cv);
     scan_load(r11 + x, dv);
     av[4] = scan_f32(r00[x4]);
@@ -100,7 +112,7 @@ __global__ void __launch_bounds__(NT) k_fx_scan(const T* __restrict__ u, KParams
 // into ctrl->rd, dd, lapdd, tdd.
 __global__ void __launch_bounds__(NT) k_energy_terms(const double* __restrict__ u, const double* __restrict__ f,
                                                      double gbar, KParams kp, Ctrl* ctrl, double* partials) {
-  __shared__ double sred[32 * 4];
+  __shared__ double sred[red_size<double>(4)];
   __shared__ int sflag;
   const int nx = kp.nx, ny = kp.ny, nz = kp.nz;
   const int lx = __ffs(nx) - 1, lxy = lx + __ffs(ny) - 1;  // sizes are powers of two
@@ -174,7 +186,7 @@ __device__ __forceinline__ bool aligned16(const void* p) { return ((unsigned lon
 
 // sum x, sum x^2, max |x| over n values -> ctrl (rd, res_l2 = sqrt(hd sum x^2), res_linf)
 __global__ void __launch_bounds__(NT) k_norms(const double* x, size_t n, double hd, Ctrl* c, double* partials) {
-  __shared__ double sred[32 * 3];
+  __shared__ double sred[red_size<double>(3)];
   __shared__ int sflag;
   double v[3] = {0.0, 0.0, -1.0}, w[3] = {0.0, 0.0, -1.0};
   const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
@@ -221,7 +233,7 @@ __global__ void __launch_bounds__(NT) k_norms(const double* x, size_t n, double 
 // u += c->c2 (k_add_mean), with no host round trip.
 __global__ void __launch_bounds__(NT) k_mean_diff(const double* g, const double* u, size_t n, Ctrl* c,
                                                   double* partials) {
-  __shared__ double sred[32];
+  __shared__ double sred[red_size<double>(1)];
   __shared__ int sflag;
   double v[1] = {0.0}, w = 0.0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -291,7 +303,7 @@ __global__ void k_accumulate_f64(double* u, const float* delta, float* u32, size
 template <typename T>
 __global__ void __launch_bounds__(NT) k_cg_update(T* lam, const T* p, T* r, const T* q, T* w, size_t n, double hd,
                                                   Ctrl* ctrl, double* partials) {
-  __shared__ T sred[32];
+  __shared__ T sred[red_size<T>(1)];
   __shared__ int sflag;
   if (ctrl->done) return;
   const T al = (T)ctrl->alpha;
@@ -332,7 +344,7 @@ __global__ void __launch_bounds__(NT) k_cg_update(T* lam, const T* p, T* r, cons
 // (h^d sum (b - q)^2)^{1/2} into ctrl->res_l2 (FP64).
 __global__ void __launch_bounds__(NT) k_sub_round(const double* b, const double* q, float* out32, size_t n, double hd,
                                                   Ctrl* ctrl, double* partials) {
-  __shared__ double sred[32];
+  __shared__ double sred[red_size<double>(1)];
   __shared__ int sflag;
   double acc = 0.0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -421,7 +433,7 @@ __global__ void __launch_bounds__(NT) k_spfc_rhs(const double* __restrict__ u, d
 // sum x (y + z) (z may be null) -> c->rd
 __global__ void __launch_bounds__(NT) k_dot(const double* x, const double* y, const double* z, size_t n, Ctrl* c,
                                             double* partials) {
-  __shared__ double sred[32];
+  __shared__ double sred[red_size<double>(1)];
   __shared__ int sflag;
   double v[1] = {0.0};
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -439,6 +451,10 @@ __global__ void __launch_bounds__(NT) k_dot(const double* x, const double* y, co
 
 inline int grid1d(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 152 * 16); }
 
+#ifndef PSD_M2D
+#define PSD_M2D 8
+#endif
+constexpr int kMarchesPerSM = PSD_M2D;  // 2D kernels
 int pick_zc(int nz, int nblk_xy) {
   // z planes per CTA: enough CTAs to fill the GPU, long enough marches
   int zc = nz;
@@ -457,11 +473,22 @@ int pick_zc(int nz, int nblk_xy) {
 // of CTAs: the CTAs per SM times the SMs (cached in KParams at setup, so
 // captured and direct launches agree and the partial sums come in the same
 // order), at most one CTA per 16 (8) column-planes.
-ResGeom res_geometry(const KParams& kp, bool fp32, int ctas_per_sm) {
-  ResGeom g{RK_2D, dim3(1, 1, 1), 1};
+ResGeom res_geometry(const KParams& kp, bool fp32, int ctas_per_sm, bool linesearch, bool pairs) {
+  ResGeom g{RK_2D, dim3(1, 1, 1), 1, NT};
   if (kp.dim != 3) {
-    const int TX = kp.nx < BX ? kp.nx : BX, TY = kp.ny < BY2 ? kp.ny : BY2;
-    g.grid = dim3(kp.nx / TX, kp.ny / TY);
+    // marches of up to 32 rows, shorter while the SMs would have few; blocks of
+    // one warp while SMs would have no block
+    const int V = fp32 && pairs && kp.nx >= 256 ? 2 : 1;
+    const int strip = linesearch ? 31 * V : 32 * V - 4;
+    const int nstrip = (kp.nx + strip - 1) / strip;
+    int ty = std::min(32, kp.ny);
+    while (ty > 2 && (long long)nstrip * (kp.ny / ty) < kMarchesPerSM * kp.nsm) ty >>= 1;
+    const int tasks = nstrip * (kp.ny / ty);
+    int warps = kWarps2D;
+    while (warps > 1 && tasks / warps < kp.nsm) warps >>= 1;
+    g.grid = dim3((tasks + warps - 1) / warps);
+    g.threads = 32 * warps;
+    g.zc = V == 2 ? -ty : ty;
     return g;
   }
   const long long wave = (long long)ctas_per_sm * kp.nsm;
@@ -506,8 +533,8 @@ cudaError_t launch_residual(const ResArgs<T>& a, int mode, int pk, const KParams
 #undef PSD_RES_BY_PK
 }
 
-ResGeom residual_geometry(const KParams& kp, bool fp32) {
-  const ResGeom g = res_geometry(kp, fp32, 2);
+ResGeom residual_geometry(const KParams& kp, bool fp32, bool pairs) {
+  const ResGeom g = res_geometry(kp, fp32, 2, false, pairs);
   return g.kind == RK_COL ? res_geometry(kp, fp32, 3) : g;
 }
 
@@ -569,7 +596,10 @@ cudaError_t launch_fx_scan(const T* u, const KParams& kp, double tol, bool force
 }
 template cudaError_t launch_fx_scan<float>(const float*, const KParams&, double, bool, Ctrl*, cudaStream_t);
 template cudaError_t launch_fx_scan<double>(const double*, const KParams&, double, bool, Ctrl*, cudaStream_t);
-bool fx_stencils(const KParams& kp, int pk) { return pk == PK_4 && residual_geometry(kp, false).kind == RK_COL; }
+bool fx_stencils(const KParams& kp, int pk) {
+  const int kind = residual_geometry(kp, false).kind;
+  return pk == PK_4 && (kind == RK_COL || kind == RK_2D);
+}
 cudaError_t launch_thinfilm_rhs(const double* u, double* f, const KParams& kp, cudaStream_t st) {
   const size_t n = (size_t)kp.nx * kp.ny * kp.nz;
   k_thinfilm_rhs<<<grid1d(n), NT, 0, st>>>(u, f, kp);

@@ -100,7 +100,7 @@ struct ResArgs {
   T* r;            // residual (order 6: local part, without T_h)
   int norm;        // 1: reduce ||r|| into ctrl and decide convergence
   int update_iter; // 1: this call advances the iteration count
-  int fixed;       // FP64 plain, p = 4, 3D column kernel: take the fixed-point variant with the
+  int fixed;       // FP64 plain, p = 4, 2D or 3D column kernel: take the fixed-point variant with the
                    // scales in ctrl (fx_s, fx_g) unless they say not to
 };
 
@@ -121,11 +121,11 @@ cudaError_t launch_linesearch(const T* u, const T* ubase, const T* d, int pk, co
 // Bounds on |u| and on the unscaled vertex gradient sums |G| (g = q G) of u into
 // ctrl->umax, gmax, and the scales of a fixed-point residual at u (fx_decide;
 // forced: without its error rule) into ctrl->fx_s, fx_g.  T: FP64, or FP32 for
-// the FP64 field that u rounds.  3D grids with nx a multiple of 4.
+// the FP64 field that u rounds.
 template <typename T>
 cudaError_t launch_fx_scan(const T* u, const KParams& kp, double tol, bool forced, Ctrl* ctrl, cudaStream_t st);
 // Whether the FP64 residual and line search of this problem have the
-// fixed-point variants (p = 4 and the 3D column kernel).
+// fixed-point variants (p = 4, 2D or the 3D column kernel).
 bool fx_stencils(const KParams& kp, int pk);
 // Right-hand side of the thin-film convex-splitting step (Sec. 6.1):
 // f = u - s Delta_h^v u (FP64, 2D and 3D).

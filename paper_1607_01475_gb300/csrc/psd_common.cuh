@@ -27,11 +27,9 @@ struct Ctrl {
   double tol;      // stop when res_l2 < tol
   double res_l2;   // ||r||_2 of the current iterate
   double res_linf; // max |r| of the current iterate (-1 if not formed)
-  // Parseval sums of the current direction (already weighted by h^d / N):
-  double rd;       // (r, d)_2
-  double dd;       // (d, d)_2
-  double lapdd;    // (Delta_h d, Delta_h d)_2
-  double tdd;      // (T_h d, d)_2 (order 6)
+  double rd;       // (r, d)_2 of the current direction, by Parseval
+  double dd, lapdd, tdd;  // sums of the discrete energies (psd_energy)
+  double lin;      // cu (d, d)_2 + (T_h d, d)_2 + s eps^2 (Delta_h d, Delta_h d)_2: q's linear part
   // line search: the first three polynomial coefficients of q (p = 4, 6;
   // weighted by h^d and s), or the general-p Newton state (c1, c2 = bracket,
   // c3 = converged flag)
@@ -96,6 +94,8 @@ struct KParams {
   double hd;            // h^d (cell volume)
   double inv_ntot;      // 1 / (nx ny nz)
   int order;
+  double fx_lin;        // 64 2^-53 cbih and |Omega|^{1/2}: the error rule of the fixed-point residual
+  double sqrt_vol;
   int nsm;              // SMs of the current device (finish_kparams; sizes one-wave grids)
   // derived constants (set by finish_kparams): the column kernels work with
   // unscaled vertex-gradient sums G = g / q and Laplacian sums h^2 Delta_h.
@@ -128,6 +128,8 @@ inline void finish_kparams(KParams& kp) {
   const double qp = (kp.p == 4.0) ? kp.q * kp.q * kp.q * kp.q : std::pow(kp.q, kp.p);
   kp.cdiv = kp.s * qp;
   kp.cbih = kp.s * kp.eps2 * kp.inv_h * kp.inv_h * kp.inv_h * kp.inv_h;
+  kp.fx_lin = 64.0 * std::ldexp(1.0, -53) * kp.cbih;
+  kp.sqrt_vol = std::sqrt(kp.hd / kp.inv_ntot);
   KConst<double>& d = kp.c64;
   d.s = kp.s;
   d.se2 = kp.s * kp.eps2;
@@ -155,42 +157,54 @@ inline void finish_kparams(KParams& kp) {
 // -------------------------------------------- scales of the fixed-point stencils
 constexpr int kFxOff = -10000;
 
-// The scale S with |v| 2^S < 2^55 for |v| <= vmax (1 + 2^-20); false when vmax
-// is not finite or S is outside [-200, 200].
+// These run in one thread at the end of a reduction, where a dependent FP64
+// operation takes 65 clocks: exponents are taken from the bits.
+//
+// e with v (1 + 2^-20) < 2^e, from the bits of a finite v >= 0 (zero: -1022).
+__device__ __forceinline__ int fx_exp_above(double v) {
+  const unsigned h = (unsigned)__double2hiint(v) + 2u;  // at least v (1 + 2^-20)
+  return (int)(h >> 20) - 1022;
+}
+__device__ __forceinline__ bool fx_finite(double v) { return ((unsigned)__double2hiint(v) & 0x7FFFFFFFu) < 0x7FE00000u; }
+// The scale S with |v| 2^S < 2^55 for |v| <= vmax (1 + 2^-20) (zero: 55); false
+// when vmax is not finite or S is outside [-200, 200].
 __device__ __forceinline__ bool fx_scale_of(double vmax, int* S) {
-  if (!isfinite(vmax)) return false;
-  int e = 0;
-  if (vmax > 0.0) frexp(vmax * (1.0 + 0x1p-20), &e);
-  *S = 55 - e;
+  if (!fx_finite(vmax)) return false;
+  *S = vmax > 0.0 ? 55 - fx_exp_above(vmax) : 55;
   return *S >= -200 && *S <= 200;
 }
-// The shift g of the gradient sums for |G| <= gmax (1 + 2^-20): |G| 2^(S+g) < 2^61.
-// (|G| < 16 max|u|, so g >= 2.)
-__device__ __forceinline__ int fx_shift_of(double gmax, int S, int* ge) {
-  int e = 0;
-  if (gmax > 0.0) frexp(gmax * (1.0 + 0x1p-20), &e);
-  const int g = gmax > 0.0 ? 61 - S - e : 60;
-  *ge = 61 - S - (g < 2 ? 2 : (g > 60 ? 60 : g));
-  return g < 2 ? 2 : (g > 60 ? 60 : g);
-}
 // Choose the scales of a fixed-point residual for |u| <= umax, |G| <= gmax into
-// c.  Its flux error is at most cdiv 2^-51 2^(3 ge) per cell (24 fluxes of a few
-// units of 2^-58 of the cube of 2^ge >= |G|); the variant runs when that is below
-// the FP64 rounding of the Laplacian sums, about 64 units 2^-53 of cbih max|u|,
-// or, in the 2-norm, below tol / 20.  Otherwise (gradients steeper than any
-// smooth field on the grid) the FP64 variant runs.
+// c: S, and the shift g of the gradient sums with |G| 2^(S+g) < 2^61 (|G| < 16
+// max|u|, so g >= 2).  With 2^ge = 2^(61-S-g) >= |G|, the flux error is at most cdiv
+// 2^-51 2^(3 ge) per cell (24 fluxes of a few units of 2^-58 of the cube of 2^ge);
+// the variant runs when that is below the FP64 rounding of the Laplacian sums,
+// about 64 units 2^-53 of cbih max|u|, or, in the 2-norm, below tol / 20.
+// Otherwise (gradients steeper than any smooth field on the grid) the FP64
+// variant runs.
 template <class C, class K>
 __device__ __forceinline__ void fx_decide(C* c, const K& kp, double umax, double gmax, double tol) {
-  int S = kFxOff, g = 0, ge = 0;
-  if (!(umax >= 0.0) || !isfinite(gmax) || !fx_scale_of(umax, &S)) {
+  int S = kFxOff, g = 60;
+  if (!(umax >= 0.0) || !fx_finite(gmax) || !fx_scale_of(umax, &S)) {
     c->fx_s = kFxOff;
     return;
   }
-  g = fx_shift_of(gmax, S, &ge);
-  const double err = kp.cdiv * ldexp(1.0, 3 * ge - 51);
-  const bool ok = umax == 0.0 || err <= 64.0 * 0x1p-53 * kp.cbih * umax || err * sqrt(kp.hd / kp.inv_ntot) < 0.05 * tol;
+  if (gmax > 0.0) g = 61 - S - fx_exp_above(gmax);
+  g = g < 2 ? 2 : (g > 60 ? 60 : g);
+  const int e3 = 3 * (61 - S - g) - 51;
+  const double err = kp.cdiv * __hiloint2double((e3 < -1000 ? 23 : e3 + 1023) << 20, 0);
+  const bool ok = umax == 0.0 || err <= kp.fx_lin * umax || err * kp.sqrt_vol < 0.05 * tol;
   c->fx_s = ok ? S : kFxOff;
   c->fx_g = g;
+}
+// An upper bound of sqrt(v) (within 2^-20) from the high word of v >= 0.
+__device__ __forceinline__ double fx_sqrt_above(unsigned hi) {
+  if (hi == 0u) return 0.0;
+  const int e = ((int)(hi >> 20) - 1023) & ~1;  // even exponent: v = m 2^e, m in [1, 4)
+  const float m = __uint_as_float((((hi >> 20) - 1023u - (unsigned)e + 127u) << 23) | ((hi & 0xFFFFFu) << 3));
+  const float r = sqrtf(m) * (1.0f + 0x1p-20f);  // in [1, 2]
+  const unsigned b = __float_as_uint(r);
+  return __hiloint2double((int)((((b >> 23) - 127u + (unsigned)(e / 2) + 1023u) << 20) | ((b >> 3) & 0xFFFFFu)),
+                          (int)(b << 29));
 }
 
 // ------------------------------------------------------------------ reductions
@@ -225,17 +239,28 @@ __device__ __forceinline__ T warp_max(T v) {
   return v;
 }
 
-// Reduce M values of type A over the block (fixed order: warp butterflies,
-// then warp 0 over the warp results); the result is valid in thread 0.  The
-// last value is reduced with max when LASTMAX is set, every value when
-// ALLMAX is.  FP32 kernels reduce
-// in float (GB300 issues FP64 at 1/64 of the FP32 rate), FP64 kernels in
-// double.  Requires blockDim to be a multiple of 32 (<= 1024) or smaller
-// than 32 (then thread 0 sums serially); uses a shared scratch of 32*M A's.
+// Shared words of block_reduce over m values of type A in a block of up to
+// 256 threads.
+template <typename A>
+__host__ __device__ constexpr int red_size(int m) {
+  return (sizeof(A) == 8 ? 256 : 32) * m;
+}
+
+// Reduce M values of type A over the block in a fixed order; the result is
+// valid in thread 0.  The last value is reduced with max when LASTMAX is set,
+// every value when ALLMAX is.  FP32 kernels reduce in float, by warp
+// butterflies and then warp 0 over the warp results.  FP64 kernels reduce in
+// double through shared memory, each value summed by a group of up to 32
+// lanes: an FP64 instruction occupies the pipe for 16 clocks and its warp for
+// 65 whatever the lanes it needs, so the butterflies' 5 (M + M nthr / 32) adds
+// (225 for 5 values of 256 threads) cost 2 us, the groups' 12 M adds a third.
+// Requires blockDim to be a power of two (below 32: thread 0 sums serially);
+// sh: red_size<A>(M).
 template <typename A, int M, bool LASTMAX, bool ALLMAX = false>
 __device__ __forceinline__ void block_reduce(A (&v)[M], A* sh) {
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
   const int nthr = blockDim.x * blockDim.y * blockDim.z;
+  auto op = [](int m, A x, A y) { return (ALLMAX || (LASTMAX && m == M - 1)) ? fmax(x, y) : x + y; };
   if (nthr < 32) {
     __syncthreads();
 #pragma unroll
@@ -245,30 +270,55 @@ __device__ __forceinline__ void block_reduce(A (&v)[M], A* sh) {
 #pragma unroll
       for (int m = 0; m < M; ++m) {
         A acc = sh[m];
-        for (int t = 1; t < nthr; ++t) acc = (ALLMAX || (LASTMAX && m == M - 1)) ? fmax(acc, sh[t * M + m]) : acc + sh[t * M + m];
+        for (int t = 1; t < nthr; ++t) acc = op(m, acc, sh[t * M + m]);
         v[m] = acc;
       }
     }
     __syncthreads();
     return;
   }
-  const int lane = tid & 31, wid = tid >> 5, nw = (nthr + 31) >> 5;
+  if constexpr (sizeof(A) == 8) {
+    int P = 32;  // lanes per value
+    while (P * M > nthr) P >>= 1;
+    __syncthreads();
 #pragma unroll
-  for (int m = 0; m < M; ++m) v[m] = (ALLMAX || (LASTMAX && m == M - 1)) ? warp_max(v[m]) : warp_sum(v[m]);
-  __syncthreads();
-  if (lane == 0) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) sh[wid * M + m] = v[m];
-  }
-  __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      A x = (lane < nw) ? sh[lane * M + m] : ((ALLMAX || (LASTMAX && m == M - 1)) ? A(-1) : A(0));
-      v[m] = (ALLMAX || (LASTMAX && m == M - 1)) ? warp_max(x) : warp_sum(x);
+    for (int m = 0; m < M; ++m) sh[m * nthr + tid] = v[m];
+    __syncthreads();
+    if ((tid & ~31) < P * M) {  // the warps that hold a group
+      const int m = tid / P, l = tid - m * P;
+      A x = A(0);
+      if (m < M) {
+        x = sh[m * nthr + l];
+        for (int t = l + P; t < nthr; t += P) x = op(m, x, sh[m * nthr + t]);
+      }
+      for (int o = P >> 1; o > 0; o >>= 1) x = op(m, x, __shfl_xor_sync(0xffffffffu, x, o));
+      if (m < M && l == 0) sh[m * nthr] = x;
     }
+    __syncthreads();
+    if (tid == 0) {
+#pragma unroll
+      for (int m = 0; m < M; ++m) v[m] = sh[m * nthr];
+    }
+    __syncthreads();
+  } else {
+    const int lane = tid & 31, wid = tid >> 5, nw = (nthr + 31) >> 5;
+#pragma unroll
+    for (int m = 0; m < M; ++m) v[m] = (ALLMAX || (LASTMAX && m == M - 1)) ? warp_max(v[m]) : warp_sum(v[m]);
+    __syncthreads();
+    if (lane == 0) {
+#pragma unroll
+      for (int m = 0; m < M; ++m) sh[wid * M + m] = v[m];
+    }
+    __syncthreads();
+    if (wid == 0) {
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        A x = (lane < nw) ? sh[lane * M + m] : ((ALLMAX || (LASTMAX && m == M - 1)) ? A(-1) : A(0));
+        v[m] = (ALLMAX || (LASTMAX && m == M - 1)) ? warp_max(x) : warp_sum(x);
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
 }
 
 // Write this block's partials, then return true in every thread of the
@@ -299,7 +349,11 @@ __device__ __forceinline__ void gather_partials(A (&out)[M], const A* partials, 
   const unsigned int nb = gridDim.x * gridDim.y * gridDim.z;
 #pragma unroll
   for (int m = 0; m < M; ++m) out[m] = (ALLMAX || (LASTMAX && m == M - 1)) ? A(-1) : A(0);
-  for (unsigned int b = tid; b < nb; b += nthr) {
+  if (tid < (int)nb) {
+#pragma unroll
+    for (int m = 0; m < M; ++m) out[m] = __ldcg(partials + (size_t)tid * M + m);
+  }
+  for (unsigned int b = tid + nthr; b < nb; b += nthr) {
 #pragma unroll
     for (int m = 0; m < M; ++m) {
       A x = __ldcg(partials + (size_t)b * M + m);
@@ -353,16 +407,24 @@ __device__ __forceinline__ void cp_async_wait_group() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-// 1/x for finite x >= 1 (the preconditioner symbols).  FP32: the hardware
+// 1/x for finite x >= 1 (the FP32 preconditioner symbols): the hardware
 // reciprocal estimate (rcp.approx) refined by one Newton-Raphson step
 // r <- r + r (1 - x r), which squares the estimate's relative error, so the
-// result is within an ulp or so of 1/x; x >= 1 keeps it clear of
-// denormals.  FP64: the IEEE quotient.
+// result is within an ulp or so of 1/x; x >= 1 keeps it clear of denormals.
 __device__ __forceinline__ float recip_ge1(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return fmaf(r, fmaf(-x, r, 1.0f), r);
 }
-__device__ __forceinline__ double recip_ge1(double x) { return 1.0 / x; }
+// 1/x for finite x > 0 in FP64 (the symbols): the hardware estimate (relative error
+// below 2^-20) with one cubic step r (1 + e + e^2), e = 1 - x r: within an
+// ulp of 1/x in three FP64 operations.
+__device__ __forceinline__ double recip_pos(double x) {
+  if ((unsigned)__double2hiint(x) >= 0x7FE00000u) return 1.0 / x;  // 2^1023 and above, infinity, NaN
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
 
 }  // namespace psd

@@ -46,7 +46,7 @@ struct ResColSmem {
   T sPb[BASE ? TY + 2 : 1][BASE ? TX + 2 : 1];
   T sMb[BASE ? TY + 2 : 1][BASE ? TX + 2 : 1];
   T sS[3][TY + 1][TX + 1];
-  T sred[32 * 2];
+  T sred[red_size<T>(2)];
   unsigned smax[2];
   int sflag;
 };
@@ -407,20 +407,7 @@ __device__ __forceinline__ void res3d_col(const ResArgs<T>& a, const KParams& kp
   }
 
   if constexpr (TRACK) {
-    block_max2(um, gm, sm.smax);
-    if (tid == 0) {
-      // upper bounds in FP64 (high words): |u|, and |G| = |G|^2's root
-      double ub, g2;
-      if constexpr (FX) {
-        ub = ((double)um + 1.0) * fx_unit(fxs - 32);
-        g2 = ((double)gm + 1.0) * fx_unit(2 * (fxs + fxg) - 96);
-      } else {
-        ub = __hiloint2double((int)um, -1);
-        g2 = __hiloint2double((int)gm, -1);
-      }
-      atomicMax(&ctrl->umax_hi, (unsigned)__double2hiint(ub) + 1u);
-      atomicMax(&ctrl->gmax2_hi, (unsigned)__double2hiint(g2) + 1u);
-    }
+    track_publish(um, gm, FX ? fxs : kFxOff, fxg, ctrl, sm.smax);
   }
   T v[2] = {acc2, accm};
   block_reduce<T, 2, true>(v, sm.sred);
@@ -429,8 +416,7 @@ __device__ __forceinline__ void res3d_col(const ResArgs<T>& a, const KParams& kp
     gather_partials<T, 2, true>(tt, reinterpret_cast<const T*>(partials), sm.sred);
     if (tid == 0) {
       if constexpr (TRACK) {
-        ctrl->umax = __hiloint2double((int)atomicExch(&ctrl->umax_hi, 0u), 0);
-        ctrl->gmax = sqrt(__hiloint2double((int)atomicExch(&ctrl->gmax2_hi, 0u), 0));
+        track_collect(ctrl);
       }
       residual_epilogue(ctrl, kp, (double)tt[0], (double)tt[1], a.norm, a.update_iter, HVP);
     }
@@ -458,9 +444,9 @@ __global__ void __launch_bounds__(256, 3)  // 80 registers, 3 CTAs per SM
 // sums use the unscaled gradients A = a/q, B = b/q; the epilogue applies q^p.
 //
 // FX (FP64, p = 4): u and d enter as 64-bit integers (scales from the bounds
-// on |u| and |d| in ctrl), so the gradients are exact sums; their products and
-// the sums stay FP64: 13 FP64 operations per vertex instead of about 40 (at
-// 256^3 0.45 ms instead of 1.28 ms).  TRACK: the bounds of the next iterate, from
+// on |u| and |d| in ctrl), so the gradients are exact sums; |a|^2, a.b and |b|^2
+// are integer products (fx_ls_accumulate), four FP64 operations per vertex
+// accumulate instead of about 40 in all.  TRACK: the bounds of the next iterate, from
 // alpha and the largest |grad d|, choose the residual's scales.
 template <typename T>
 struct LsColSmem {
@@ -539,23 +525,14 @@ __device__ __forceinline__ void ls3d_col(const T* __restrict__ u, const T* __res
         hdd[k] = dn;
       }
   };
-  auto grad = [&](LT (&P)[SY][SX], LT (&M)[SY][SX], T (&g)[3]) {
-    const LT g0 = (P[ty][tx + 1] - P[ty][tx]) + (P[ty + 1][tx + 1] - P[ty + 1][tx]);
-    const LT g1 = (P[ty + 1][tx] - P[ty][tx]) + (P[ty + 1][tx + 1] - P[ty][tx + 1]);
-    const LT g2 = (M[ty][tx] + M[ty][tx + 1]) + (M[ty + 1][tx] + M[ty + 1][tx + 1]);
-    if constexpr (FX) {
-      g[0] = fx_result(g0, 0);
-      g[1] = fx_result(g1, 0);
-      g[2] = fx_result(g2, 0);
-    } else {
-      g[0] = g0;
-      g[1] = g1;
-      g[2] = g2;
-    }
+  auto grad = [&](LT (&P)[SY][SX], LT (&M)[SY][SX], LT (&g)[3]) {
+    g[0] = (P[ty][tx + 1] - P[ty][tx]) + (P[ty + 1][tx + 1] - P[ty + 1][tx]);
+    g[1] = (P[ty + 1][tx] - P[ty][tx]) + (P[ty + 1][tx + 1] - P[ty][tx + 1]);
+    g[2] = (M[ty][tx] + M[ty][tx + 1]) + (M[ty + 1][tx] + M[ty + 1][tx + 1]);
   };
   T acc[ls_nsums<PK>()] = {};
-  T sbb = T(0);       // TRACK: sum (a.b)^2, kept apart from sum |a|^2 |b|^2
-  unsigned gm = 0u, gu = 0u;  // TRACK: largest |b|^2, high word
+  T sbb = T(0);      // TRACK: sum (a.b)^2, kept apart from sum |a|^2 |b|^2
+  unsigned gm = 0u;  // TRACK: largest |b|^2, high word
   for (int w = (int)((long long)wtot * blockIdx.x / gridDim.x); w < wend;) {
     const int col = w / nz, z0 = w - col * nz;
     const int zc = min(nz - z0, wend - w);
@@ -572,36 +549,20 @@ __device__ __forceinline__ void ls3d_col(const T* __restrict__ u, const T* __res
       store(buf, false);  // vertex plane z + 1/2
       __syncthreads();
       fetch(z + 2);
-      T av[3], bv[3];
+      LT av[3], bv[3];
       grad(sPu[buf], sMu[buf], av);
       grad(sPd[buf], sMd[buf], bv);
-      if constexpr (TRACK) {
-        // the coefficients' constant factors (2, 3) are applied to the sums
-        const T A = fma(av[2], av[2], fma(av[1], av[1], av[0] * av[0]));
-        const T B = fma(av[2], bv[2], fma(av[1], bv[1], av[0] * bv[0]));
-        const T C = fma(bv[2], bv[2], fma(bv[1], bv[1], bv[0] * bv[0]));
-        gm = max(gm, (unsigned)__double2hiint(C));
-        acc[0] = fma(A, C, acc[0]);
-        sbb = fma(B, B, sbb);
-        acc[1] = fma(B, C, acc[1]);
-        acc[2] = fma(C, C, acc[2]);
-      } else {
+      if constexpr (FX)
+        gm = max(gm, fx_ls_accumulate(av[0], av[1], av[2], bv[0], bv[1], bv[2], acc, sbb));
+      else if constexpr (TRACK)
+        gm = max(gm, ls_accumulate4(av, bv, acc, sbb));
+      else
         ls_accumulate<PK>(av, bv, trial, beta, pm2, acc);
-      }
     }
     __syncthreads();  // the next segment writes the shared buffers again
   }
   if constexpr (TRACK) {
-    // FX: the integers' units 2^-Su, 2^-Sd
-    const T uu = FX ? (T)fx_unit(Su) : T(1), ud = FX ? (T)fx_unit(Sd) : T(1);
-    acc[0] = (acc[0] + T(2) * sbb) * (uu * ud) * (uu * ud);
-    acc[1] = T(3) * acc[1] * (uu * ud) * (ud * ud);
-    acc[2] = acc[2] * (ud * ud) * (ud * ud);
-    block_max2(gm, gu, sm.smax);
-    if (tid == 0) {
-      const double g2 = __hiloint2double((int)gm, -1) * (FX ? fx_unit(2 * Sd) : 1.0);
-      atomicMax(&ctrl->gmax2_hi, (unsigned)__double2hiint(g2) + 1u);
-    }
+    ls_track(acc, sbb, gm, FX, Su, Sd, ctrl, sm.smax);
   }
   ls_finish<T, PK>(acc, sred, partials, ctrl, kp, &sm.sflag, TRACK ? tol : -1.0);
 }
@@ -613,11 +574,10 @@ __global__ void __launch_bounds__(256, 3)
   if (ctrl->done) return;
   if (!ls_closed_form<PK>() && ctrl->c3 != 0.0) return;  // Newton already converged
   __shared__ __align__(16) LsColSmem<T> sm;
-  __shared__ T sred[32 * ls_nsums<PK>()];
+  __shared__ T sred[red_size<T>(ls_nsums<PK>())];
   if constexpr (sizeof(T) == 8 && PK == PK_4 && !INNER) {
-    const double dmax = __hiloint2double((int)ctrl->dmax_hi, 0);
     int Su, Sd;
-    if (ctrl->umax >= 0.0 && fx_scale_of(ctrl->umax, &Su) && fx_scale_of(dmax, &Sd)) {
+    if (ls_scales(ctrl, &Su, &Sd)) {
       ls3d_col<T, PK, INNER, true>(u, ubase, d, kp, ctrl, partials, ctrl->tol, sm, sred, Su, Sd);
       return;
     }

@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256, 2)
   __shared__ T sPb[BASE ? LY : 1][BASE ? LX : 1];
   __shared__ T sMb[BASE ? LY : 1][BASE ? LX : 1];
   __shared__ T sS[3][VY][VX];
-  __shared__ T sred[32 * 2];
+  __shared__ T sred[red_size<T>(2)];
   __shared__ int sflag;
 
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(256, 3)
   constexpr int SX = TX + 1, SY = TYT + 1;  // cells x0 .. x0+TX, y0 .. y0+TYT
   constexpr int NH = SY + TX;               // halo cells: column TX (SY) and row TYT (TX)
   __shared__ T sPu[2][SY][SX], sMu[2][SY][SX], sPd[2][SY][SX], sMd[2][SY][SX];
-  __shared__ T sred[32 * ls_nsums<PK>()];
+  __shared__ T sred[red_size<T>(ls_nsums<PK>())];
   __shared__ int sflag;
   const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
   const int nx = kp.nx, ny = kp.ny, nz = kp.nz;

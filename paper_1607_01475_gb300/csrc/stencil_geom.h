@@ -9,20 +9,22 @@ namespace psd {
 
 constexpr int BX = 32;   // tile width (x)
 constexpr int BY3 = 8;   // tile height (y), 3D
-constexpr int BY2 = 32;  // tile height (y), 2D
+constexpr int kWarps2D = 4;  // most marches (warps) per block, 2D
 constexpr int NT = 256;  // threads per block
 
 enum ResKind { RK_2D, RK_SMALL3D, RK_COL, RK_RB4 };
 struct ResGeom {
   int kind;
   dim3 grid;
-  int zc;
+  int zc;  // general 3D kernel: planes per CTA; 2D: rows per march (negative: two cells per lane)
+  int threads;
 };
-// Geometry for a kernel whose __launch_bounds__ guarantee ctas_per_sm
+// linesearch: the strips of the 2D line search; pairs: 2D FP32 fields aligned to
+// 8 bytes (two cells per lane on wide grids).  Geometry for a kernel whose __launch_bounds__ guarantee ctas_per_sm
 // resident CTAs per SM (defined in k_stencil.cu).
-ResGeom res_geometry(const KParams& kp, bool fp32, int ctas_per_sm);
+ResGeom res_geometry(const KParams& kp, bool fp32, int ctas_per_sm, bool linesearch = false, bool pairs = true);
 // The residual launch: k_res3d_rb keeps 2 CTAs per SM resident, k_res3d_col 3.
-ResGeom residual_geometry(const KParams& kp, bool fp32);
+ResGeom residual_geometry(const KParams& kp, bool fp32, bool pairs = true);
 
 namespace detail {
 // Residual and line-search launchers for one vertex-factor kind PK (PK_4,

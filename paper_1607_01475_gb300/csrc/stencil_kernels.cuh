@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(NT)
   __shared__ T sb[NB][SYM][SXM];
   __shared__ T sl[3][BY3 + 2][BX + 2];
   __shared__ T sf[2][3][BY3 + 1][BX + 1];
-  __shared__ T sred[32 * 2];
+  __shared__ T sred[red_size<T>(2)];
   __shared__ int sflag;
 
   const int nx = kp.nx, ny = kp.ny, nz = kp.nz;
@@ -303,106 +303,24 @@ __global__ void __launch_bounds__(NT)
   }
 }
 
-// ------------------------------------------------------------- 2D residual
-template <typename T, int PK, int MODE>
-__global__ void __launch_bounds__(NT) k_res2d(ResArgs<T> a, KParams kp, Ctrl* ctrl, double* partials) {
-  if (ctrl->done) return;
-  constexpr int SXM = BX + 4, SYM = BY2 + 4;
-  constexpr int NB = (MODE == RM_INNER) ? 1 : 1;
-  __shared__ T su[SYM][SXM];
-  __shared__ T sb[(MODE != RM_PLAIN) ? SYM : 1][SXM];
-  __shared__ T sl[BY2 + 2][BX + 2];
-  __shared__ T sf[2][BY2 + 1][BX + 1];
-  __shared__ T sred[32 * 2];
-  __shared__ int sflag;
-  (void)NB;
-
-  const int nx = kp.nx, ny = kp.ny;
-  const int TX = nx < BX ? nx : BX, TY = ny < BY2 ? ny : BY2;
-  const int SX = TX + 4, SY = TY + 4;
-  const int tid = threadIdx.x;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  const bool upd = a.d != nullptr;
-  const T alpha = upd ? (T)ctrl->alpha : T(0);
-  const KConst<T>& C = kconst<T>(kp);
-  const T ih = C.inv_h, ih2 = ih * ih, q2 = T(0.5) * ih;
-  const T s = C.s, se2 = C.se2, cu = C.cu;
-  const T beta = C.beta;
-
-  for (int idx = tid; idx < SX * SY; idx += NT) {
-    const int ly = idx / SX, lx = idx - ly * SX;
-    const int gx = wrapi(x0 + lx - 2, nx), gy = wrapi(y0 + ly - 2, ny);
-    const size_t g = (size_t)gy * nx + gx;
-    T v = a.u_in[g];
-    if (upd) {
-      v = v + alpha * a.d[g];
-      if (lx >= 2 && lx < TX + 2 && ly >= 2 && ly < TY + 2) a.u_out[g] = v;
-    }
-    su[ly][lx] = v;
-    if (MODE != RM_PLAIN) sb[ly][lx] = a.ubase[g];
+// The fixed-point variants' bookkeeping (see fx_decide).  track_publish: the
+// block's bounds on |u| and |G|^2 (um, gm: largest high words, of integers in
+// units of 2^-fxs and of the flux's |G|^2 when fxs is a scale, of FP64 values
+// otherwise) into the running maxima of ctrl; track_collect, in the last block:
+// the maxima become the iterate's bounds.
+__device__ __forceinline__ void track_publish(unsigned um, unsigned gm, int fxs, int fxg, Ctrl* ctrl, unsigned* smax) {
+  block_max2(um, gm, smax);
+  if (threadIdx.x == 0) {
+    const bool fx = fxs != kFxOff;
+    const double ub = fx ? ((double)um + 1.0) * fx_unit(fxs - 32) : __hiloint2double((int)um, -1);
+    const double g2 = fx ? ((double)gm + 1.0) * fx_unit(2 * (fxs + fxg) - 96) : __hiloint2double((int)gm, -1);
+    atomicMax(&ctrl->umax_hi, (unsigned)__double2hiint(ub) + 1u);
+    atomicMax(&ctrl->gmax2_hi, (unsigned)__double2hiint(g2) + 1u);
   }
-  __syncthreads();
-  {
-    const int LX = TX + 2, LY = TY + 2;
-    for (int idx = tid; idx < LX * LY; idx += NT) {
-      const int ly = idx / LX, lx = idx - ly * LX;
-      const T sum = (su[ly + 1][lx] + su[ly + 1][lx + 2]) + (su[ly][lx + 1] + su[ly + 2][lx + 1]);
-      sl[ly][lx] = (sum - T(4) * su[ly + 1][lx + 1]) * ih2;
-    }
-    const int VX = TX + 1, VY = TY + 1;
-    for (int idx = tid; idx < VX * VY; idx += NT) {
-      const int vy = idx / VX, vx = idx - vy * VX;
-      T g[3], F[3];
-      {
-        const T u00 = su[vy + 1][vx + 1], u01 = su[vy + 1][vx + 2], u10 = su[vy + 2][vx + 1], u11 = su[vy + 2][vx + 2];
-        g[0] = q2 * ((u01 - u00) + (u11 - u10));
-        g[1] = q2 * ((u10 - u00) + (u11 - u01));
-        g[2] = T(0);
-      }
-      if (MODE != RM_PLAIN) {
-        const T u00 = sb[vy + 1][vx + 1], u01 = sb[vy + 1][vx + 2], u10 = sb[vy + 2][vx + 1], u11 = sb[vy + 2][vx + 2];
-        T ab[3] = {q2 * ((u01 - u00) + (u11 - u10)), q2 * ((u10 - u00) + (u11 - u01)), T(0)};
-        if (MODE == RM_INNER)
-          flux_diff<PK>(ab, g, beta, F);
-        else
-          flux_lin<PK>(ab, g, beta, F);
-      } else {
-        flux<PK>(g, beta, F);
-      }
-      sf[0][vy][vx] = F[0];
-      sf[1][vy][vx] = F[1];
-    }
-  }
-  __syncthreads();
-  T acc2 = T(0), accm = T(0);
-  for (int idx = tid; idx < TX * TY; idx += NT) {
-    const int ty = idx / TX, tx = idx - ty * TX;
-    const T bih = (((sl[ty + 1][tx] + sl[ty + 1][tx + 2]) + (sl[ty][tx + 1] + sl[ty + 2][tx + 1])) - T(4) * sl[ty + 1][tx + 1]) * ih2;
-    const T dx = q2 * ((sf[0][ty][tx + 1] - sf[0][ty][tx]) + (sf[0][ty + 1][tx + 1] - sf[0][ty + 1][tx]));
-    const T dy = q2 * ((sf[1][ty + 1][tx] - sf[1][ty][tx]) + (sf[1][ty + 1][tx + 1] - sf[1][ty][tx + 1]));
-    const T div = dx + dy;
-    const T uc = su[ty + 2][tx + 2];
-    const size_t g = (size_t)(y0 + ty) * nx + (x0 + tx);
-    T r;
-    if (MODE == RM_INNER)
-      r = (a.f ? a.f[g] : T(0)) - ((cu * uc + se2 * bih) - s * div);
-    else if (MODE == RM_HVP)
-      r = (cu * uc + se2 * bih) - s * div;
-    else
-      r = (a.f ? a.f[g] : T(0)) - cu * uc + s * div - se2 * bih;
-    a.r[g] = r;
-    acc2 += (MODE == RM_HVP) ? uc * r : r * r;
-    accm = fmax(accm, fabs(r));
-  }
-  T v[2] = {acc2, accm};
-  block_reduce<T, 2, true>(v, sred);
-  if (publish_and_check_last<T>(v, 2, reinterpret_cast<T*>(partials), &ctrl->counter[CS_RES], &sflag)) {
-    T tt[2];
-    gather_partials<T, 2, true>(tt, reinterpret_cast<const T*>(partials), sred);
-    double tot[2];
-    for (int m_ = 0; m_ < 2; ++m_) tot[m_] = (double)tt[m_];
-    if (tid == 0) residual_epilogue(ctrl, kp, tot[0], tot[1], a.norm, a.update_iter, MODE == RM_HVP);
-  }
+}
+__device__ __forceinline__ void track_collect(Ctrl* ctrl) {
+  ctrl->umax = __hiloint2double((int)atomicExch(&ctrl->umax_hi, 0u), 0);
+  ctrl->gmax = fx_sqrt_above(atomicExch(&ctrl->gmax2_hi, 0u));
 }
 
 // ------------------------------------------------------------ line search
@@ -411,6 +329,65 @@ __global__ void __launch_bounds__(NT) k_res2d(ResArgs<T> a, KParams kp, Ctrl* ct
 // cubic) and p = 6 (a quintic) of Sec. 6.1, with the s factor folded into
 // c_j.  q(0) = -rd < 0 and q is strictly increasing (Sec. 2.3), so the root
 // is unique; Newton's method with a bisection safeguard on a bracket.
+//
+// One thread runs this at the end of the line search, where every dependent
+// FP64 operation takes 65 clocks and a division about 1000 (the plain FP64 Newton
+// iteration took 7 us of the 1024^2 line search's 11).  So the iteration is done
+// in FP32 on x = alpha / alpha_0, alpha_0 = rd / q'(0), where Q(x) = q / rd = -1 + x
+// + e_1 x^2 + .. is of order one, and finished by two FP64 Newton steps with FP32
+// quotients: the first leaves about 1e-13, the second is below rounding.
+// newton_x: false when that does not settle (then the plain iteration decides).
+// K: the coefficients e_1 .. e_{K-1}.
+template <int K>
+__device__ __forceinline__ bool newton_x(const double (&e)[4], double* x_out) {
+  float f[K - 1];
+#pragma unroll
+  for (int j = 0; j < K - 1; ++j) f[j] = (float)e[j];
+  auto qf = [&](float x) {
+    float v = f[K - 2];
+#pragma unroll
+    for (int j = K - 3; j >= 0; --j) v = fmaf(x, v, f[j]);
+    return fmaf(x, fmaf(x, v, 1.0f), -1.0f);
+  };
+  auto df = [&](float x) {
+    float v = (float)K * f[K - 2];
+#pragma unroll
+    for (int j = K - 3; j >= 0; --j) v = fmaf(x, v, (float)(j + 2) * f[j]);
+    return fmaf(x, v, 1.0f);
+  };
+  float lo = 0.0f, hi = 1.0f;
+  for (int i = 0; i < 40 && !(qf(hi) > 0.0f); ++i) {
+    lo = hi;
+    hi *= 2.0f;
+  }
+  float xf = hi;
+  for (int it = 0; it < 40; ++it) {
+    const float q = qf(xf);
+    if (q < 0.0f)
+      lo = xf;
+    else
+      hi = xf;
+    float nx = xf - __fdividef(q, df(xf));
+    if (!(lo < nx && nx < hi)) nx = 0.5f * (lo + hi);
+    const bool settled = fabsf(nx - xf) <= 4e-7f * nx;
+    xf = nx;
+    if (settled) break;
+  }
+  double x = (double)xf;
+  float step = 0.0f;
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    double v = e[K - 2];
+#pragma unroll
+    for (int j = K - 3; j >= 0; --j) v = fma(x, v, e[j]);
+    step = __fdividef((float)fma(x, fma(x, v, 1.0), -1.0), df((float)x));
+    x -= (double)step;
+  }
+  *x_out = x;
+  return x > 0.0 && fabsf(step) <= 1e-9f * (float)x && df((float)x) > 0.0f;
+}
+// K: the degree of q.
+template <int K>
 __device__ double solve_poly_alpha(double rd, double lin, const double (&c)[5], int* status) {
   auto q = [&](double al) { return -rd + al * (lin + c[0] + al * (c[1] + al * (c[2] + al * (c[3] + al * c[4])))); };
   auto dq = [&](double al) {
@@ -420,6 +397,19 @@ __device__ double solve_poly_alpha(double rd, double lin, const double (&c)[5], 
   if (!(rd > 0.0) || !(d0 > 0.0) || !isfinite(rd) || !isfinite(d0)) {
     *status = (isfinite(rd) && isfinite(d0)) ? 0 : 7;
     return 0.0;
+  }
+  {
+    const double r0 = recip_pos(d0), a0 = rd * r0, a2 = a0 * a0;
+    double e[4] = {c[1] * (a0 * r0), c[2] * (a2 * r0), 0.0, 0.0};
+    if (K == 5) {
+      e[2] = c[3] * (a2 * a0 * r0);
+      e[3] = c[4] * (a2 * a2 * r0);
+    }
+    double x;
+    // FP32 range: |e| below 2^60
+    const unsigned top = max(max((unsigned)__double2hiint(e[0]) & 0x7FFFFFFFu, (unsigned)__double2hiint(e[1]) & 0x7FFFFFFFu),
+                             max((unsigned)__double2hiint(e[2]) & 0x7FFFFFFFu, (unsigned)__double2hiint(e[3]) & 0x7FFFFFFFu));
+    if (top < (1083u << 20) && newton_x<K>(e, &x)) return a0 * x;
   }
   double lo = 0.0, hi = -1.0;
   double alpha = rd / d0;
@@ -507,16 +497,81 @@ __device__ __forceinline__ void ls_accumulate(const T (&av)[3], const T (&bv)[3]
   }
 }
 
+// p = 4 with the coefficients' constant factors (2, 3) left to the sums: AC, BC,
+// C^2 into acc, B^2 into sbb.  Returns the high word of C.
+template <typename T, int M>
+__device__ __forceinline__ unsigned ls_accumulate4(const T (&av)[3], const T (&bv)[3], T (&acc)[M], T& sbb) {
+  const T A = fma(av[2], av[2], fma(av[1], av[1], av[0] * av[0]));
+  const T B = fma(av[2], bv[2], fma(av[1], bv[1], av[0] * bv[0]));
+  const T C = fma(bv[2], bv[2], fma(bv[1], bv[1], bv[0] * bv[0]));
+  acc[0] = fma(A, C, acc[0]);
+  sbb = fma(B, B, sbb);
+  acc[1] = fma(B, C, acc[1]);
+  acc[2] = fma(C, C, acc[2]);
+  return (unsigned)__double2hiint(C);
+}
+// The same from integer gradients a, b (moduli below 2^61): A, B and C are
+// integer products of the gradients shifted to full length, each within a few
+// 2^-57 of |a||a|, |a||b|, |b||b|; only the four accumulations are FP64.
+template <int M>
+__device__ __forceinline__ unsigned fx_ls_accumulate(long long a0, long long a1, long long a2, long long b0,
+                                                     long long b1, long long b2, double (&acc)[M], double& sbb) {
+  // leading zeros of the largest component, by the ones' complement magnitudes
+  auto shift = [](long long x, long long y, long long z) {
+    const unsigned long long m = (unsigned long long)((x ^ (x >> 63)) | (y ^ (y >> 63)) | (z ^ (z >> 63))) | 1ULL;
+    return __clzll((long long)m) - 4;  // components below 2^60, moduli below 2^61 after the shift
+  };
+  const int sa = shift(a0, a1, a2), sb = shift(b0, b1, b2);
+  const fx_halves x0 = fx_split(fx_shl(a0, sa)), x1 = fx_split(fx_shl(a1, sa)), x2 = fx_split(fx_shl(a2, sa));
+  const fx_halves y0 = fx_split(fx_shl(b0, sb)), y1 = fx_split(fx_shl(b1, sb)), y2 = fx_split(fx_shl(b2, sb));
+  auto square = [](const fx_halves& p, const fx_halves& q, const fx_halves& r) {
+    const long long t = fx_wide(p.h, p.l) + (fx_wide(q.h, q.l) + (fx_wide(r.h, r.l) + (1LL << 30)));
+    return fx_wide(p.h, p.h) + (fx_wide(q.h, q.h) + (fx_wide(r.h, r.h) + (t >> 31)));
+  };
+  const long long ia = square(x0, x1, x2), ic = square(y0, y1, y2);
+  const long long t0 = fx_wide(x0.h, y0.l) + (fx_wide(x1.h, y1.l) + (fx_wide(x2.h, y2.l) + (1LL << 31)));
+  const long long t1 = fx_wide(x0.l, y0.h) + (fx_wide(x1.l, y1.h) + fx_wide(x2.l, y2.h));
+  const long long ib = fx_wide(x0.h, y0.h) + (fx_wide(x1.h, y1.h) + (fx_wide(x2.h, y2.h) + ((t0 + t1) >> 32)));
+  const double A = fx_result(ia, 64 - 2 * sa), B = fx_result(ib, 64 - sa - sb), C = fx_result(ic, 64 - 2 * sb);
+  acc[0] = fma(A, C, acc[0]);
+  sbb = fma(B, B, sbb);
+  acc[1] = fma(B, C, acc[1]);
+  acc[2] = fma(C, C, acc[2]);
+  return (unsigned)__double2hiint(C);
+}
+// Scales of u and d for the fixed-point line search from the bounds in ctrl.
+__device__ __forceinline__ bool ls_scales(const Ctrl* ctrl, int* Su, int* Sd) {
+  return ctrl->umax >= 0.0 && fx_scale_of(ctrl->umax, Su) && fx_scale_of(__hiloint2double((int)ctrl->dmax_hi, 0), Sd);
+}
+// The p = 4 sums with their factors and units, and the block's bound on |grad d|^2.
+template <typename T, int M>
+__device__ __forceinline__ void ls_track(T (&acc)[M], T sbb, unsigned gm, bool fixed, int Su, int Sd, Ctrl* ctrl,
+                                         unsigned* smax) {
+  acc[0] = acc[0] + T(2) * sbb;
+  acc[1] = T(3) * acc[1];
+  if (fixed) {  // powers of two
+    acc[0] *= (T)fx_unit(2 * (Su + Sd));
+    acc[1] *= (T)fx_unit(Su + 3 * Sd);
+    acc[2] *= (T)fx_unit(4 * Sd);
+  }
+  unsigned none = 0u;
+  block_max2(gm, none, smax);
+  if (threadIdx.x == 0) {
+    const double g2 = __hiloint2double((int)gm, -1) * (fixed ? fx_unit(2 * Sd) : 1.0);
+    atomicMax(&ctrl->gmax2_hi, (unsigned)__double2hiint(g2) + 1u);
+  }
+}
+
 // Last-block logic of the line search.
 template <int PK>
 __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double (&tot)[ls_nsums<PK>()]) {
-  const double lin = kp.cu * ctrl->dd + ctrl->tdd + kp.s * kp.eps2 * ctrl->lapdd;
+  const double lin = ctrl->lin;
   if (ls_closed_form<PK>()) {
     int st = 0;
     // the kernels sum unscaled vertex gradients G = g / q: s g^p-terms = cdiv G^p-terms
     double c[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     for (int j = 0; j < ls_nsums<PK>(); ++j) c[j] = kp.cdiv * kp.hd * tot[j];
-    const double al = solve_poly_alpha(ctrl->rd, lin, c, &st);
+    const double al = solve_poly_alpha<ls_nsums<PK>()>(ctrl->rd, lin, c, &st);
     ctrl->c1 = c[0];
     ctrl->c2 = c[1];
     ctrl->c3 = c[2];
@@ -579,7 +634,7 @@ __device__ __forceinline__ void ls_finish(T (&acc)[ls_nsums<PK>()], T* sred, dou
       linesearch_epilogue<PK>(ctrl, kp, tot);
       if (fx_tol >= 0.0) {
         // the next iterate u + alpha d: |u| and |G| are at most these
-        const double al = fabs(ctrl->alpha), gd = sqrt(__hiloint2double((int)atomicExch(&ctrl->gmax2_hi, 0u), 0));
+        const double al = fabs(ctrl->alpha), gd = fx_sqrt_above(atomicExch(&ctrl->gmax2_hi, 0u));
         fx_decide(ctrl, kp, ctrl->umax + al * __hiloint2double((int)ctrl->dmax_hi, 0), ctrl->gmax + al * gd, fx_tol);
       }
     }
@@ -588,6 +643,7 @@ __device__ __forceinline__ void ls_finish(T (&acc)[ls_nsums<PK>()], T* sred, dou
 
 }  // namespace
 }  // namespace psd
+#include "stencil2d.cuh"
 #include "stencil3d_col.cuh"
 #include "stencil3d_rb.cuh"
 namespace psd {
@@ -602,7 +658,7 @@ __global__ void __launch_bounds__(NT)
   constexpr int SXM = BX + 1, SYM = BY3 + 1;
   __shared__ T su[2][SYM][SXM];
   __shared__ T sd[2][SYM][SXM];
-  __shared__ T sred[32 * ls_nsums<PK>()];
+  __shared__ T sred[red_size<T>(ls_nsums<PK>())];
   __shared__ int sflag;
   const int nx = kp.nx, ny = kp.ny, nz = kp.nz;
   const int TX = nx < BX ? nx : BX, TY = ny < BY3 ? ny : BY3;
@@ -649,52 +705,19 @@ __global__ void __launch_bounds__(NT)
   ls_finish<T, PK>(acc, sred, partials, ctrl, kp, &sflag);
 }
 
-template <typename T, int PK, bool INNER>
-__global__ void __launch_bounds__(NT)
-    k_ls2d(const T* __restrict__ u, const T* __restrict__ ubase, const T* __restrict__ d, KParams kp, Ctrl* ctrl,
-           double* partials) {
-  if (ctrl->done) return;
-  if (!ls_closed_form<PK>() && ctrl->c3 != 0.0) return;
-  constexpr int SXM = BX + 1, SYM = BY2 + 1;
-  __shared__ T su[SYM][SXM];
-  __shared__ T sd[SYM][SXM];
-  __shared__ T sred[32 * ls_nsums<PK>()];
-  __shared__ int sflag;
-  const int nx = kp.nx, ny = kp.ny;
-  const int TX = nx < BX ? nx : BX, TY = ny < BY2 ? ny : BY2;
-  const int SX = TX + 1, SY = TY + 1;
-  const int tid = threadIdx.x;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  const T beta = kconst<T>(kp).beta, pm2 = kconst<T>(kp).pm2;
-  const T trial = ls_closed_form<PK>() ? T(0) : (T)ctrl->alpha;
-  for (int idx = tid; idx < SX * SY; idx += NT) {
-    const int ly = idx / SX, lx = idx - ly * SX;
-    const size_t g = (size_t)wrapi(y0 + ly, ny) * nx + wrapi(x0 + lx, nx);
-    T v = u[g];
-    if (INNER) v += ubase[g];
-    su[ly][lx] = v;
-    sd[ly][lx] = d[g];
-  }
-  __syncthreads();
-  T acc[ls_nsums<PK>()] = {};
-  for (int idx = tid; idx < TX * TY; idx += NT) {
-    const int vy = idx / TX, vx = idx - vy * TX;
-    T av[3] = {(su[vy][vx + 1] - su[vy][vx]) + (su[vy + 1][vx + 1] - su[vy + 1][vx]),
-               (su[vy + 1][vx] - su[vy][vx]) + (su[vy + 1][vx + 1] - su[vy][vx + 1]), T(0)};
-    T bv[3] = {(sd[vy][vx + 1] - sd[vy][vx]) + (sd[vy + 1][vx + 1] - sd[vy + 1][vx]),
-               (sd[vy + 1][vx] - sd[vy][vx]) + (sd[vy + 1][vx + 1] - sd[vy][vx + 1]), T(0)};
-    ls_accumulate<PK>(av, bv, trial, beta, pm2, acc);
-  }
-  ls_finish<T, PK>(acc, sred, partials, ctrl, kp, &sflag);
-}
-
 }  // namespace
 
 namespace detail {
 
+// Whether every pointer is 8-byte aligned.
+template <typename... P>
+bool aligned8(const P*... p) {
+  return ((reinterpret_cast<unsigned long long>(p) | ...) & 7ull) == 0;
+}
+
 template <typename T, int PK, int MODE>
 cudaError_t res_impl(const ResArgs<T>& a, const KParams& kp, Ctrl* ctrl, double* partials, cudaStream_t st) {
-  const ResGeom g = residual_geometry(kp, sizeof(T) == 4);
+  const ResGeom g = residual_geometry(kp, sizeof(T) == 4, aligned8(a.u_in, a.d, a.u_out, a.f, a.ubase, a.r));
   switch (g.kind) {
     case RK_RB4:
       if constexpr (sizeof(T) == 4) k_res3d_rb<T, PK, MODE, 4><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials);
@@ -706,7 +729,13 @@ cudaError_t res_impl(const ResArgs<T>& a, const KParams& kp, Ctrl* ctrl, double*
       k_res3d<T, PK, MODE><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials, g.zc);
       break;
     default:
-      k_res2d<T, PK, MODE><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials);
+      if constexpr (sizeof(T) == 4) {
+        if (g.zc < 0) {  // two cells per lane
+          k_res2d<T, PK, MODE, 2><<<g.grid, g.threads, 0, st>>>(a, kp, ctrl, partials, -g.zc);
+          break;
+        }
+      }
+      k_res2d<T, PK, MODE, 1><<<g.grid, g.threads, 0, st>>>(a, kp, ctrl, partials, g.zc);
   }
   return cudaGetLastError();
 }
@@ -715,7 +744,7 @@ template <typename T, int PK, bool INNER>
 cudaError_t ls_impl(const T* u, const T* ubase, const T* d, const KParams& kp, Ctrl* ctrl, double* partials,
                     cudaStream_t st) {
   // the same tiles as the residual; __launch_bounds__(256, 3)
-  const ResGeom g = res_geometry(kp, sizeof(T) == 4, 3);
+  const ResGeom g = res_geometry(kp, sizeof(T) == 4, 3, true, aligned8(u, ubase, d));
   switch (g.kind) {
     case RK_RB4:
       if constexpr (sizeof(T) == 4) k_ls3d_rb<T, PK, INNER, 4><<<g.grid, NT, 0, st>>>(u, ubase, d, kp, ctrl, partials);
@@ -727,7 +756,13 @@ cudaError_t ls_impl(const T* u, const T* ubase, const T* d, const KParams& kp, C
       k_ls3d<T, PK, INNER><<<g.grid, NT, 0, st>>>(u, ubase, d, kp, ctrl, partials, g.zc);
       break;
     default:
-      k_ls2d<T, PK, INNER><<<g.grid, NT, 0, st>>>(u, ubase, d, kp, ctrl, partials);
+      if constexpr (sizeof(T) == 4) {
+        if (g.zc < 0) {
+          k_ls2d<T, PK, INNER, 2><<<g.grid, g.threads, 0, st>>>(u, ubase, d, kp, ctrl, partials, -g.zc);
+          break;
+        }
+      }
+      k_ls2d<T, PK, INNER, 1><<<g.grid, g.threads, 0, st>>>(u, ubase, d, kp, ctrl, partials, g.zc);
   }
   return cudaGetLastError();
 }
