@@ -524,6 +524,7 @@ cudaError_t launch_residual(const ResArgs<T>& a, int mode, int pk, const KParams
 #define PSD_RES_BY_PK(MODE_)                                                              \
   switch (pk) {                                                                           \
     case PK_4: return res_impl<T, PK_4, MODE_>(a, kp, ctrl, partials, st);                \
+    case PK_3: return res_impl<T, PK_3, MODE_>(a, kp, ctrl, partials, st);                \
     case PK_6: return res_impl<T, PK_6, MODE_>(a, kp, ctrl, partials, st);                \
     default: return res_impl<T, PK_GEN, MODE_>(a, kp, ctrl, partials, st);               \
   }
@@ -550,6 +551,7 @@ cudaError_t launch_linesearch(const T* u, const T* ubase, const T* d, int pk, co
 #define PSD_LS_BY_PK(INNER_)                                                              \
   switch (pk) {                                                                           \
     case PK_4: return ls_impl<T, PK_4, INNER_>(u, ubase, d, kp, ctrl, partials, st);      \
+    case PK_3: return ls_impl<T, PK_3, INNER_>(u, ubase, d, kp, ctrl, partials, st);      \
     case PK_6: return ls_impl<T, PK_6, INNER_>(u, ubase, d, kp, ctrl, partials, st);      \
     default: return ls_impl<T, PK_GEN, INNER_>(u, ubase, d, kp, ctrl, partials, st);     \
   }

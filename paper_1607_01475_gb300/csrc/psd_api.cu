@@ -529,7 +529,7 @@ psd_status capture_graph(psd_context* c, cudaGraphExec_t* exec, Enq&& enqueue) {
 // a WHILE loop that stops at convergence inside a captured graph.
 template <typename T>
 psd_status linesearch(psd_context* c, const T* u, const T* ubase, const T* D, Ctrl* ctrl) {
-  if (c->pk != psd::PK_GEN) {
+  if (c->pk == psd::PK_4 || c->pk == psd::PK_6) {
     ProfScope p_(c, cls_of<T>(PSD_PROF_LINESEARCH_FP64));
     CK(psd::launch_linesearch<T>(u, ubase, D, c->pk, c->kp, ctrl, c->partials, c->st));
     return PSD_OK;
@@ -1251,7 +1251,7 @@ psd_status psd_create(const psd_params* params, psd_handle* out) {
   c->N = (size_t)kp.nx * kp.ny * kp.nz;
   kp.inv_ntot = 1.0 / (double)c->N;
   psd::finish_kparams(kp);
-  c->pk = (params->p == 4.0) ? psd::PK_4 : (params->p == 6.0) ? psd::PK_6 : psd::PK_GEN;
+  c->pk = psd::pkind_of(params->p);
   static const bool attrs = (psd::init_dht_attributes(), true);  // once, thread-safe
   (void)attrs;
 

@@ -9,9 +9,10 @@
 
 namespace psd {
 
-// Kinds of the vertex factor |g|^{p-2}: specialised p = 4 (|g|^2) and
-// p = 6 (|g|^4 = (|g|^2)^2), and a general p (pow).
-enum PKind { PK_GEN = 0, PK_4 = 4, PK_6 = 6 };
+// Kinds of the vertex factor |g|^{p-2}: specialised p = 3 (|g|), p = 4 (|g|^2)
+// and p = 6 (|g|^4 = (|g|^2)^2), and a general p (pow).
+enum PKind { PK_GEN = 0, PK_3 = 3, PK_4 = 4, PK_6 = 6 };
+inline int pkind_of(double p) { return p == 3.0 ? PK_3 : p == 4.0 ? PK_4 : p == 6.0 ? PK_6 : PK_GEN; }
 
 // Slots of the "last block" counters in the control block.
 enum CounterSlot { CS_RES = 0, CS_MID = 1, CS_LS = 2, CS_MISC = 3, CS_COUNT = 8 };

@@ -28,7 +28,7 @@ ResGeom residual_geometry(const KParams& kp, bool fp32, bool pairs = true);
 
 namespace detail {
 // Residual and line-search launchers for one vertex-factor kind PK (PK_4,
-// PK_6 or PK_GEN), explicitly instantiated by k_res_p4.cu, k_res_p6.cu and
+// PK_3, PK_6 or PK_GEN), explicitly instantiated by k_res_p3.cu, k_res_p4.cu, k_res_p6.cu and
 // k_res_pgen.cu.
 template <typename T, int PK, int MODE>
 cudaError_t res_impl(const ResArgs<T>& a, const KParams& kp, Ctrl* ctrl, double* partials, cudaStream_t st);

@@ -1,6 +1,6 @@
 // Residual and line-search kernels of the PSD iteration (included by the
-// per-vertex-factor translation units k_res_p4.cu, k_res_p6.cu and
-// k_res_pgen.cu, each of which instantiates one kind):
+// per-vertex-factor translation units k_res_p3.cu, k_res_p4.cu, k_res_p6.cu
+// and k_res_pgen.cu, each of which instantiates one kind):
 //   r = f - N_h[u],  N_h[u] = cu u - s d.(|D u|^{p-2} D u) + s eps^2 Delta_h^2 u
 // (Eq. "discrete-4th-order", Sec. 5.3; the local part of the sixth-order
 // operator of Sec. 5.4 / 6.2 with cu = s lambda), fused with the deferred
@@ -27,11 +27,13 @@
 namespace psd {
 namespace {
 
-// |g|^{p-2} from g2 = |g|^2: g2 (p = 4), g2^2 (p = 6), else pow.
+// |g|^{p-2} from g2 = |g|^2: g2 (p = 4), g2^2 (p = 6), its root (p = 3), else
+// pow.
 template <int PK, typename T>
 __device__ __forceinline__ T vfactor(T g2, T beta) {
   if (PK == PK_4) return g2;
   if (PK == PK_6) return g2 * g2;
+  if (PK == PK_3) return sqrt(g2);
   return pow(g2, beta);  // beta = (p-2)/2; pow(0, 0) = 1, pow(0, b>0) = 0
 }
 
@@ -52,6 +54,12 @@ __device__ __forceinline__ void flux_diff(const T (&a)[3], const T (&e)[3], T be
     const T c4 = c2 * c2, w = dl * (c2 + a2);
 #pragma unroll
     for (int c = 0; c < 3; ++c) out[c] = c4 * e[c] + w * a[c];
+  } else if (PK == PK_3) {
+    // |a+e| e + (|a+e| - |a|) a, the difference of the roots from dl
+    const T na = sqrt(a2), nc = sqrt(c2 > T(0) ? c2 : T(0)), den = na + nc;
+    const T w = den > T(0) ? dl / den : T(0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) out[c] = nc * e[c] + w * a[c];
   } else {
     const T fc = pow(c2 > T(0) ? c2 : T(0), beta);
     T dfac;  // |a+e|^{p-2} - |a|^{p-2}
@@ -86,6 +94,11 @@ __device__ __forceinline__ void flux_lin(const T (&a)[3], const T (&e)[3], T bet
     const T a4 = a2 * a2, w = T(4) * a2 * ae;
 #pragma unroll
     for (int c = 0; c < 3; ++c) out[c] = a4 * e[c] + w * a[c];
+  } else if (PK == PK_3) {
+    // |a| e + (a.e) / |a| a
+    const T na = sqrt(a2), w = na > T(0) ? ae / na : T(0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) out[c] = na * e[c] + w * a[c];
   } else {
     const T f = pow(a2, beta);
     const T w = (a2 > T(0)) ? T(2) * beta * pow(a2, beta - T(1)) * ae : T(0);
@@ -454,7 +467,7 @@ __host__ __device__ constexpr bool ls_closed_form() {
 }
 template <int PK>
 __host__ __device__ constexpr int ls_nsums() {
-  return PK == PK_6 ? 5 : 3;
+  return PK == PK_6 ? 5 : (PK == PK_4 ? 3 : 2);
 }
 
 // Vertex sums for one vertex with a = grad u (+ grad ubase), b = grad d.
@@ -483,17 +496,27 @@ __device__ __forceinline__ void ls_accumulate(const T (&av)[3], const T (&bv)[3]
       acc[ls_nsums<PK>() - 1] += C * C2;
     }
   } else {
-    T e[3] = {trial * bv[0], trial * bv[1], trial * bv[2]};
-    T df[3];
-    flux_diff<PK>(av, e, beta, df);
-    acc[0] += df[0] * bv[0] + df[1] * bv[1] + df[2] * bv[2];
-    const T c[3] = {av[0] + e[0], av[1] + e[1], av[2] + e[2]};
+    // with e = trial b, c = a + e: (F(c) - F(a)).b = |c|^{p-2} trial C + (|c|^{p-2} -
+    // |a|^{p-2}) B, and its derivative |c|^{p-2} C + (p-2) |c|^{p-4} (c.b)^2
+    const T A = av[0] * av[0] + av[1] * av[1] + av[2] * av[2];
+    const T B = av[0] * bv[0] + av[1] * bv[1] + av[2] * bv[2];
+    const T C = bv[0] * bv[0] + bv[1] * bv[1] + bv[2] * bv[2];
+    const T c[3] = {av[0] + trial * bv[0], av[1] + trial * bv[1], av[2] + trial * bv[2]};
     const T c2 = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
-    const T cb = c[0] * bv[0] + c[1] * bv[1] + c[2] * bv[2];
-    const T b2 = bv[0] * bv[0] + bv[1] * bv[1] + bv[2] * bv[2];
-    T t = pow(c2, beta) * b2;
-    if (c2 > T(0)) t += pm2 * pow(c2, beta - T(1)) * cb * cb;
-    acc[1] += t;
+    const T cb = B + trial * C, dl = trial * (B + cb);  // |c|^2 - |a|^2
+    T fc, dfac, w;  // |c|^{p-2}, its difference from |a|^{p-2}, (p-2) |c|^{p-4}
+    if (PK == PK_3) {
+      const T na = sqrt(A);
+      fc = sqrt(c2);
+      dfac = na + fc > T(0) ? dl / (na + fc) : T(0);
+      w = fc > T(0) ? T(1) / fc : T(0);
+    } else {
+      fc = pow(c2, beta);
+      dfac = A > T(0) ? pow(A, beta) * expm1(beta * log1p(fmax(dl / A, T(-1)))) : fc;
+      w = c2 > T(0) ? pm2 * fc / c2 : T(0);
+    }
+    acc[0] += fc * trial * C + dfac * B;
+    acc[1] += fc * C + w * cb * cb;
   }
 }
 
@@ -562,9 +585,9 @@ __device__ __forceinline__ void ls_track(T (&acc)[M], T sbb, unsigned gm, bool f
   }
 }
 
-// Last-block logic of the line search.
+// Last-block logic of the line search (f32: the sums are FP32's).
 template <int PK>
-__device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double (&tot)[ls_nsums<PK>()]) {
+__device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double (&tot)[ls_nsums<PK>()], bool f32) {
   const double lin = ctrl->lin;
   if (ls_closed_form<PK>()) {
     int st = 0;
@@ -581,8 +604,11 @@ __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double 
       ctrl->done = 1;
     }
   } else {
-    // one safeguarded Newton step per launch; state in c1 (lo), c2 (hi), c3 (done flag)
-    const double trial = ctrl->alpha;
+    // one safeguarded Newton step per launch; state in c1 (lo), c2 (hi), c3 (done
+    // flag); the first trial is the previous iteration's step size.  A step below
+    // 1e-4 of alpha (FP32 sums, whose alpha is used rounded to FP32) or 5e-9 (FP64)
+    // is the last: what it leaves is of the order of its square.
+    const double trial = f32 ? (double)(float)ctrl->alpha : ctrl->alpha;
     const double qv = -ctrl->rd + trial * lin + kp.cdiv * kp.hd * tot[0];
     const double dqv = lin + kp.cdiv * kp.hd * tot[1];
     double lo = ctrl->c1, hi = ctrl->c2;
@@ -590,9 +616,9 @@ __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double 
       lo = trial;
     else if (qv > 0.0)
       hi = trial;
-    const double step = (dqv > 0.0) ? qv / dqv : 0.0;
+    const double step = (dqv > 0.0) ? qv * recip_pos(dqv) : 0.0;
     double nw = (dqv > 0.0) ? trial - step : 0.5 * (lo + hi);
-    const bool tiny = (dqv > 0.0) && fabs(step) <= 4e-16 * fabs(trial);  // Newton step below rounding
+    const bool tiny = (dqv > 0.0) && fabs(step) <= (f32 ? 1e-4 : 5e-9) * fabs(trial);
     if (!tiny) {
       if (hi > 0.0) {
         if (!(lo < nw && nw < hi)) nw = 0.5 * (lo + hi);
@@ -631,7 +657,7 @@ __device__ __forceinline__ void ls_finish(T (&acc)[ls_nsums<PK>()], T* sred, dou
       double tot[M];
 #pragma unroll
       for (int m = 0; m < M; ++m) tot[m] = (double)tt[m];
-      linesearch_epilogue<PK>(ctrl, kp, tot);
+      linesearch_epilogue<PK>(ctrl, kp, tot, sizeof(T) == 4);
       if (fx_tol >= 0.0) {
         // the next iterate u + alpha d: |u| and |G| are at most these
         const double al = fabs(ctrl->alpha), gd = fx_sqrt_above(atomicExch(&ctrl->gmax2_hi, 0u));
