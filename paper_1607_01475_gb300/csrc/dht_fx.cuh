@@ -28,9 +28,9 @@ constexpr int kFxThreads = 256;
 // pairs): r = m/2, M = m for m = TS/2 (odd LS when m < 2, free when m >= 32);
 // strided passes (a warp spans `pairs` pairs): r = 16/k, M = 32/k for k =
 // min(2 pairs, 16).
-template <int N, bool ROWS>
+template <int N, int RM, bool ROWS>
 __host__ __device__ constexpr int fx_line_stride() {
-  constexpr int L = LineFFT<fx, N, 8>::L, TS = LineFFT<fx, N, 8>::TS;
+  constexpr int L = LineFFT<fx, N, RM>::L, TS = LineFFT<fx, N, RM>::TS;
   int r = 0, M = 1;
   if (ROWS) {
     const int m = TS / 2;
@@ -44,9 +44,9 @@ __host__ __device__ constexpr int fx_line_stride() {
   }
   return L + (((r - L) % M) + M) % M;
 }
-template <int N, bool ROWS>
+template <int N, int RM, bool ROWS>
 constexpr size_t fx_pair_smem() {
-  return 2 * (size_t)fx_line_stride<N, ROWS>() * sizeof(fx);
+  return 2 * (size_t)fx_line_stride<N, RM, ROWS>() * sizeof(fx);
 }
 
 // The common exponent and scale of a line pair from its team's values.  ROWS:
@@ -57,9 +57,9 @@ constexpr size_t fx_pair_smem() {
 struct FxLine {
   int E, B;  // largest biased exponent, scale
 };
-template <int N, bool ROWS>
+template <int N, int RM, bool ROWS>
 struct FxTeam {
-  static constexpr int R = FxPlan<N>::R, TS = N / R;
+  static constexpr int R = FxPlan<N, RM>::R, TS = N / R;
   static constexpr bool kOneWarp = ROWS && TS <= 32;
   int p, pairs;
   int E;       // of this warp
@@ -86,7 +86,7 @@ struct FxTeam {
     if (!kOneWarp && (ROWS ? lane == 0 : lane < pairs)) scr[threadIdx.x >> 5][lane] = make_uint2((unsigned)E, l);
   }
   __device__ __forceinline__ FxLine line(const uint2 (*scr)[32]) const {
-    if (kOneWarp) return {E, fx_scale<N>(l)};
+    if (kOneWarp) return {E, fx_scale<FxPlan<N, RM>>(l)};
     // the team's warps: w0, w0 + step, ..
     const int nw = ROWS ? p * (TS / 32) + TS / 32 : ((int)blockDim.x + 31) >> 5;
     const int step = !ROWS && pairs > 32 ? pairs >> 5 : 1;
@@ -98,7 +98,7 @@ struct FxTeam {
       const uint2 v = scr[w][lane];
       lm += (v.y >> min(Em - (int)v.x, 31)) + 1u;
     }
-    return {Em, fx_scale<N>(lm)};
+    return {Em, fx_scale<FxPlan<N, RM>>(lm)};
   }
 };
 
@@ -127,29 +127,29 @@ __device__ __forceinline__ double fx_load(float x) {
 
 // A line pair's points as integers of the line's scale (0 where the line is
 // zero or not finite), and a Hartley output from the split sum w.
-template <int N>
-__device__ __forceinline__ void fx_enter(const double (&xr)[FxPlan<N>::R], const double (&xi)[FxPlan<N>::R],
-                                         const FxLine& ln, fx (&vr)[FxPlan<N>::R], fx (&vi)[FxPlan<N>::R]) {
+template <int N, int RM>
+__device__ __forceinline__ void fx_enter(const double (&xr)[FxPlan<N, RM>::R], const double (&xi)[FxPlan<N, RM>::R],
+                                         const FxLine& ln, fx (&vr)[FxPlan<N, RM>::R], fx (&vi)[FxPlan<N, RM>::R]) {
   const bool live = ln.E >= kFxMinExp && ln.E <= kFxMaxExp;
 #pragma unroll
-  for (int q = 0; q < FxPlan<N>::R; ++q) {
+  for (int q = 0; q < FxPlan<N, RM>::R; ++q) {
     vr[q] = fx_quantise((unsigned)__double2hiint(xr[q]), (unsigned)__double2loint(xr[q]), ln.E, ln.B);
     vi[q] = fx_quantise((unsigned)__double2hiint(xi[q]), (unsigned)__double2loint(xi[q]), ln.E, ln.B);
     if (!live) vr[q].v = vi[q].v = 0;
   }
 }
-template <int N>
+template <int N, int RM>
 __device__ __forceinline__ double fx_leave(fx w, const FxLine& ln, int scale_e) {
   return ln.E > kFxMaxExp ? __longlong_as_double(0x7FF8000000000000LL)
-                          : fx_result(w.v, ln.E - ln.B + FxPlan<N>::kOut + scale_e);
+                          : fx_result(w.v, ln.E - ln.B + FxPlan<N, RM>::kOut + scale_e);
 }
 
 // -------------------------------------------------------------- x (rows)
-template <int N, typename SI>
+template <int N, int RM, typename SI>
 __global__ void __launch_bounds__(kFxThreads, 3)
     k_rows_fx(const SI* src, double* dst, int nrows, int scale_e, const int* done, const fx_tw* __restrict__ tab,
               unsigned int* dmax_hi) {
-  using F = LineFFT<fx, N, 8>;
+  using F = LineFFT<fx, N, RM>;
   constexpr int R = F::R, TS = F::TS;
   if (done != nullptr && *done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -159,10 +159,10 @@ __global__ void __launch_bounds__(kFxThreads, 3)
   const int p = tid / TS, j = tid - p * TS;
   const int row0 = 2 * (blockIdx.x * pairs + p);
   const bool valid = row0 < nrows;
-  constexpr int LS = fx_line_stride<N, true>();
+  constexpr int LS = fx_line_stride<N, RM, true>();
   fx* sr = reinterpret_cast<fx*>(smem_raw) + (size_t)p * 2 * LS;
   fx* si = sr + LS;
-  FxTeam<N, true> team{p, pairs};
+  FxTeam<N, RM, true> team{p, pairs};
   double xr[R], xi[R];
   const SI* s0 = src + (size_t)row0 * N;
 #pragma unroll
@@ -174,16 +174,16 @@ __global__ void __launch_bounds__(kFxThreads, 3)
   if (!team.kOneWarp) __syncthreads();
   const FxLine ln = team.line(scr);
   fx vr[R], vi[R];
-  fx_enter<N>(xr, xi, ln, vr, vi);
+  fx_enter<N, RM>(xr, xi, ln, vr, vi);
   double* d0 = dst + (size_t)row0 * N;
   unsigned top = 0u;  // largest magnitude written, high word
   auto put = [&](int k, fx h1, fx h2) {
-    const double a = fx_leave<N>(h1, ln, scale_e), b = fx_leave<N>(h2, ln, scale_e);
+    const double a = fx_leave<N, RM>(h1, ln, scale_e), b = fx_leave<N, RM>(h2, ln, scale_e);
     d0[k] = a;
     d0[N + k] = b;
     top = max(top, max((unsigned)__double2hiint(a) & 0x7FFFFFFFu, (unsigned)__double2hiint(b) & 0x7FFFFFFFu));
   };
-  if constexpr (FxTeam<N, true>::kOneWarp) {
+  if constexpr (FxTeam<N, RM, true>::kOneWarp) {
     // the last pass ends in registers, the split by shuffle
     F::run_tw_regs(vr, vi, j, sr, si, TwFx{tab});
     fx h1[R], h2[R];
@@ -221,25 +221,25 @@ __global__ void __launch_bounds__(kFxThreads, 3)
 // the spectrum in sr / si.  Block: `pairs` pairs of adjacent x-columns packed
 // as re/im, thread (p, j) = (tid % pairs, tid / pairs), so that a warp reads
 // whole row segments.  The line buffers are written after the first barrier.
-template <int N>
-__device__ __forceinline__ FxLine fx_cols_transform(const double (&xr)[FxPlan<N>::R], const double (&xi)[FxPlan<N>::R],
+template <int N, int RM>
+__device__ __forceinline__ FxLine fx_cols_transform(const double (&xr)[FxPlan<N, RM>::R], const double (&xi)[FxPlan<N, RM>::R],
                                                     int p, int j, int pairs, fx* sr, fx* si, uint2 (*scr)[32],
                                                     const fx_tw* __restrict__ tab) {
-  FxTeam<N, false> team{p, pairs};
+  FxTeam<N, RM, false> team{p, pairs};
   team.share(xr, xi, scr);
   __syncthreads();
   const FxLine ln = team.line(scr);
-  fx vr[FxPlan<N>::R], vi[FxPlan<N>::R];
-  fx_enter<N>(xr, xi, ln, vr, vi);
-  LineFFT<fx, N, 8>::run_tw(vr, vi, j, sr, si, TwFx{tab});
+  fx vr[FxPlan<N, RM>::R], vi[FxPlan<N, RM>::R];
+  fx_enter<N, RM>(xr, xi, ln, vr, vi);
+  LineFFT<fx, N, RM>::run_tw(vr, vi, j, sr, si, TwFx{tab});
   return ln;
 }
 
-template <int N>
+template <int N, int RM>
 __global__ void __launch_bounds__(kFxThreads, 3)
     k_cols_fx(double* data, size_t line_stride, size_t outer_stride, int scale_e, const int* done,
               const fx_tw* __restrict__ tab) {
-  using F = LineFFT<fx, N, 8>;
+  using F = LineFFT<fx, N, RM>;
   constexpr int R = F::R, TS = F::TS;
   if (done != nullptr && *done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kFxThreads, 3)
   const int pairs = blockDim.x / TS;
   const int p = tid % pairs, j = tid / pairs;
   const size_t base = (size_t)blockIdx.y * outer_stride + (size_t)blockIdx.x * 2 * pairs + 2 * p;
-  constexpr int LS = fx_line_stride<N, false>();
+  constexpr int LS = fx_line_stride<N, RM, false>();
   fx* sr = reinterpret_cast<fx*>(smem_raw) + (size_t)p * 2 * LS;
   fx* si = sr + LS;
   double xr[R], xi[R];
@@ -258,14 +258,14 @@ __global__ void __launch_bounds__(kFxThreads, 3)
     xr[q] = v.x;
     xi[q] = v.y;
   }
-  const FxLine ln = fx_cols_transform<N>(xr, xi, p, j, pairs, sr, si, scr, tab);
+  const FxLine ln = fx_cols_transform<N, RM>(xr, xi, p, j, pairs, sr, si, scr, tab);
 #pragma unroll
   for (int q = 0; q < R; ++q) {
     const int kk = j + q * TS;
     fx h1, h2;
     dht_split(sr, si, kk, N, h1, h2);
     *reinterpret_cast<double2*>(data + base + (size_t)kk * line_stride) =
-        make_double2(fx_leave<N>(h1, ln, scale_e), fx_leave<N>(h2, ln, scale_e));
+        make_double2(fx_leave<N, RM>(h1, ln, scale_e), fx_leave<N, RM>(h2, ln, scale_e));
   }
 }
 
@@ -278,12 +278,12 @@ __global__ void __launch_bounds__(kFxThreads, 3)
 // with mu the symbol of -Delta_h at the element; the zero mode gives 0
 // (mean-zero projection).  Same thread mapping as k_cols_fx.
 enum { EPI_THETA = 0, EPI_RESID = 1 };
-template <int N, int EPI>
+template <int N, int RM, int EPI>
 __global__ void __launch_bounds__(kFxThreads, 3)
     k_last_fx(const double* data, double* theta, float* out32, size_t line_stride, size_t outer_stride, KParams kp,
               Ctrl* ctrl, double* partials, const fx_tw* __restrict__ tab, const double* __restrict__ symx,
               const double* __restrict__ symo, const double* __restrict__ syml, double* dc, const int* skip) {
-  using F = LineFFT<fx, N, 8>;
+  using F = LineFFT<fx, N, RM>;
   constexpr int R = F::R, TS = F::TS;
   if (skip != nullptr && *skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kFxThreads, 3)
   const int p = tid % pairs, j = tid / pairs;
   const int x = blockIdx.x * 2 * pairs + 2 * p;
   const size_t base = (size_t)blockIdx.y * outer_stride + x;
-  constexpr int LS = fx_line_stride<N, false>();
+  constexpr int LS = fx_line_stride<N, RM, false>();
   fx* sr = reinterpret_cast<fx*>(smem_raw) + (size_t)p * 2 * LS;
   fx* si = sr + LS;
   // theta of this thread's elements, copied asynchronously while the
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kFxThreads, 3)
     xr[q] = v.x;
     xi[q] = v.y;
   }
-  const FxLine ln = fx_cols_transform<N>(xr, xi, p, j, pairs, sr, si, scr, tab);
+  const FxLine ln = fx_cols_transform<N, RM>(xr, xi, p, j, pairs, sr, si, scr, tab);
   cp_async_wait_all();
   const double mo = symo != nullptr ? symo[blockIdx.y] : 0.0;
   const double mx[2] = {symx[x] + mo, symx[x + 1] + mo};
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kFxThreads, 3)
     float o32[2];
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const double h = fx_leave<N>(w[c], ln, 0);
+      const double h = fx_leave<N, RM>(w[c], ln, 0);
       const bool live = !(x + c == 0 && blockIdx.y == 0 && kk == 0);  // mu > 0: every mode but the zero one
       if (EPI == EPI_THETA) {
         if (!live && dc != nullptr) *dc = h;
@@ -364,13 +364,13 @@ __global__ void __launch_bounds__(kFxThreads, 3)
 // one outer index per CTA, lines along the last axis.  The symbol division
 // and the Parseval sums are FP64; both transforms are fixed point, each with
 // its own line exponents.
-template <int N, int ORDER>
+template <int N, int RM, int ORDER>
 __global__ void __launch_bounds__(kFxThreads, 2)
     k_mid_fx(double* data, unsigned line_stride, unsigned outer_stride, int ntx, KParams kp, Ctrl* ctrl,
              double* partials, double* xi_, double* dspec, const double* __restrict__ symx,
              const double* __restrict__ symo, const double* __restrict__ syml, const fx_tw* __restrict__ tab,
              int scale_e) {
-  using F = LineFFT<fx, N, 8>;
+  using F = LineFFT<fx, N, RM>;
   constexpr int R = F::R, TS = F::TS;
   if (ctrl->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(kFxThreads, 2)
   const int tid = threadIdx.x;
   const int pairs = blockDim.x / TS;
   const int p = tid % pairs, j = tid / pairs;
-  constexpr int LS = fx_line_stride<N, false>();
+  constexpr int LS = fx_line_stride<N, RM, false>();
   fx* sr = reinterpret_cast<fx*>(smem_raw) + (size_t)p * 2 * LS;
   fx* si = sr + LS;
   // order 6: xi and dspec of the tile, copied while the transform runs
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(kFxThreads, 2)
     xr[q] = v.x;
     xi[q] = v.y;
   }
-  FxLine ln = fx_cols_transform<N>(xr, xi, p, j, pairs, sr, si, scr, tab);
+  FxLine ln = fx_cols_transform<N, RM>(xr, xi, p, j, pairs, sr, si, scr, tab);
   if (ORDER == 6) cp_async_wait_all();
   const KConst<double>& C = kp.c64;
   const double s = C.s, se2 = C.se2, sl = C.sl;
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(kFxThreads, 2)
     if (ORDER == 4) {
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
-        const double h = fx_leave<N>(w[c], ln, 0);
+        const double h = fx_leave<N, RM>(w[c], ln, 0);
         const double mu = (c ? mxb : mxa) + ml;
         const double d = h * recip_pos(fma(mu, fma(se2, mu, s), 1.0));
         const double m = mu * d;
@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(kFxThreads, 2)
       double xn[2], tn[2];
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
-        const double h = fx_leave<N>(w[c], ln, 0);
+        const double h = fx_leave<N, RM>(w[c], ln, 0);
         const double mu = (c ? mxb : mxa) + ml;
         double rt = 0.0, d = 0.0, xc = 0.0, td = 0.0;
         if (!(x + c == 0 && yo == 0 && kk == 0)) {  // mu > 0: every mode but the zero one
@@ -463,14 +463,14 @@ __global__ void __launch_bounds__(kFxThreads, 2)
   }
   // the barrier inside, before the line buffers are written again, comes
   // after every thread has read the forward spectrum
-  ln = fx_cols_transform<N>(xr, xi, p, j, pairs, sr, si, scr, tab);
+  ln = fx_cols_transform<N, RM>(xr, xi, p, j, pairs, sr, si, scr, tab);
 #pragma unroll
   for (int q = 0; q < R; ++q) {
     const int kk = j + q * TS;
     fx h1, h2;
     dht_split(sr, si, kk, N, h1, h2);
     *reinterpret_cast<double2*>(data + (base + (unsigned)kk * line_stride)) =
-        make_double2(fx_leave<N>(h1, ln, scale_e), fx_leave<N>(h2, ln, scale_e));
+        make_double2(fx_leave<N, RM>(h1, ln, scale_e), fx_leave<N, RM>(h2, ln, scale_e));
   }
   mid_finish<double, ORDER>(acc, sred, partials, ctrl, kp, &sflag);
 }
@@ -482,14 +482,22 @@ __global__ void __launch_bounds__(kFxThreads, 2)
 // (eight blocks of one warp instead of one of 256 threads, on one SM) a row pass
 // takes 8.6 us instead of 21 and the middle pass 26 instead of 59, fixed point
 // and narrowing together.
-template <int N, bool ROWS>
+template <int N, int RM, bool ROWS>
 int fx_pairs(long long total, int avail, int nsm) {
-  constexpr int TS = LineFFT<fx, N, 8>::TS;
+  constexpr int TS = LineFFT<fx, N, RM>::TS;
   int pairs = kFxThreads / TS;
   while (pairs > 1 && pairs > avail) pairs >>= 1;
   while (pairs > (ROWS ? 1 : 2) && pairs * TS > 32 && total / pairs < nsm) pairs >>= 1;
   return pairs;
 }
+// Whether a pass over a field of `cells` takes radix 4 instead of 8: with 16
+// points per thread (8 of each line of the pair) the grid would have fewer than
+// eight warps per SM, and a thread's chain of integer and FP64 work is the time.
+// Lines of 512 and more keep radix 8: with two more passes dividing by 4, decaying
+// lines would lose more than FP64 does.
+template <int N>
+constexpr int kFxShort = N <= 256 ? 4 : 8;
+inline bool fx_short(long long cells, int nsm) { return cells / 16 < 256LL * nsm; }
 // The exponent of a power-of-two scale (every pass scales by 1 or 1/N).
 inline bool fx_scale_exp(double scale, int* e) {
   const double m = std::frexp(scale, e);
@@ -497,27 +505,27 @@ inline bool fx_scale_exp(double scale, int* e) {
   return m == 0.5;
 }
 
-template <int N, typename SI>
+template <int N, int RM, typename SI>
 cudaError_t rows_fx_impl(const SI* src, double* dst, int nrows, double scale, const int* done,
                          const AxisTables<double>& tb, cudaStream_t st, unsigned int* dmax_hi) {
-  constexpr int TS = LineFFT<fx, N, 8>::TS;
+  constexpr int TS = LineFFT<fx, N, RM>::TS;
   int se;
   if (!fx_scale_exp(scale, &se)) return cudaErrorInvalidValue;
   const int np = (nrows + 1) / 2;
-  const int pairs = fx_pairs<N, true>(np, 1 << 30, tb.nsm);
-  k_rows_fx<N, SI><<<(np + pairs - 1) / pairs, pairs * TS, pairs * fx_pair_smem<N, true>(), st>>>(src, dst, nrows, se,
+  const int pairs = fx_pairs<N, RM, true>(np, 1 << 30, tb.nsm);
+  k_rows_fx<N, RM, SI><<<(np + pairs - 1) / pairs, pairs * TS, pairs * fx_pair_smem<N, RM, true>(), st>>>(src, dst, nrows, se,
                                                                                                  done, tb.fxtw[0], dmax_hi);
   return cudaGetLastError();
 }
 
-template <int N>
+template <int N, int RM>
 cudaError_t cols_fx_impl(double* data, int nx, int nouter, size_t line_stride, size_t outer_stride, double scale,
                          const int* done, const fx_tw* tab, int nsm, cudaStream_t st) {
-  constexpr int TS = LineFFT<fx, N, 8>::TS;
+  constexpr int TS = LineFFT<fx, N, RM>::TS;
   int se;
   if (!fx_scale_exp(scale, &se)) return cudaErrorInvalidValue;
-  const int pairs = fx_pairs<N, false>((long long)(nx / 2) * nouter, nx / 2, nsm);
-  k_cols_fx<N><<<dim3(nx / (2 * pairs), nouter), pairs * TS, pairs * fx_pair_smem<N, false>(), st>>>(
+  const int pairs = fx_pairs<N, RM, false>((long long)(nx / 2) * nouter, nx / 2, nsm);
+  k_cols_fx<N, RM><<<dim3(nx / (2 * pairs), nouter), pairs * TS, pairs * fx_pair_smem<N, RM, false>(), st>>>(
       data, line_stride, outer_stride, se, done, tab);
   return cudaGetLastError();
 }
@@ -532,44 +540,44 @@ inline LastAxis last_axis(const KParams& kp) {
   return {(size_t)kp.nx * kp.ny, (size_t)kp.nx, kp.ny, 2};
 }
 
-template <int N>
+template <int N, int RM>
 cudaError_t mid_fx_impl(double* data, const KParams& kp, Ctrl* ctrl, double* partials, double* xi, double* dspec,
                         const AxisTables<double>& tb, cudaStream_t st) {
-  constexpr int TS = LineFFT<fx, N, 8>::TS;
+  constexpr int TS = LineFFT<fx, N, RM>::TS;
   const LastAxis a = last_axis(kp);
   int se;
   if (!fx_scale_exp(kp.inv_ntot, &se)) return cudaErrorInvalidValue;
-  const int pairs = fx_pairs<N, false>((long long)(kp.nx / 2) * a.nouter, kp.nx / 2, tb.nsm);
+  const int pairs = fx_pairs<N, RM, false>((long long)(kp.nx / 2) * a.nouter, kp.nx / 2, tb.nsm);
   const int ntx = kp.nx / (2 * pairs);
   const double* symo = kp.dim == 2 ? nullptr : tb.sym[1];
-  const size_t sm = pairs * fx_pair_smem<N, false>() + (kp.order == 6 ? 2 : 0) * (size_t)N * pairs * sizeof(double2);
+  const size_t sm = pairs * fx_pair_smem<N, RM, false>() + (kp.order == 6 ? 2 : 0) * (size_t)N * pairs * sizeof(double2);
   if (kp.order == 4)
-    k_mid_fx<N, 4><<<ntx * a.nouter, pairs * TS, sm, st>>>(data, (unsigned)a.line_stride, (unsigned)a.outer_stride, ntx,
+    k_mid_fx<N, RM, 4><<<ntx * a.nouter, pairs * TS, sm, st>>>(data, (unsigned)a.line_stride, (unsigned)a.outer_stride, ntx,
                                                           kp, ctrl, partials, xi, dspec, tb.sym[0], symo, tb.sym[a.ax],
                                                           tb.fxtw[a.ax], se);
   else
-    k_mid_fx<N, 6><<<ntx * a.nouter, pairs * TS, sm, st>>>(data, (unsigned)a.line_stride, (unsigned)a.outer_stride, ntx,
+    k_mid_fx<N, RM, 6><<<ntx * a.nouter, pairs * TS, sm, st>>>(data, (unsigned)a.line_stride, (unsigned)a.outer_stride, ntx,
                                                           kp, ctrl, partials, xi, dspec, tb.sym[0], symo, tb.sym[a.ax],
                                                           tb.fxtw[a.ax], se);
   return cudaGetLastError();
 }
 
-template <int N>
+template <int N, int RM>
 cudaError_t last_fx_impl(const double* data, double* theta, float* out32, const KParams& kp, Ctrl* ctrl,
                          double* partials, const AxisTables<double>& tb, cudaStream_t st, double* dc,
                          const int* skip) {
-  constexpr int TS = LineFFT<fx, N, 8>::TS;
+  constexpr int TS = LineFFT<fx, N, RM>::TS;
   const LastAxis a = last_axis(kp);
-  const int pairs = fx_pairs<N, false>((long long)(kp.nx / 2) * a.nouter, kp.nx / 2, tb.nsm);
+  const int pairs = fx_pairs<N, RM, false>((long long)(kp.nx / 2) * a.nouter, kp.nx / 2, tb.nsm);
   const dim3 grid(kp.nx / (2 * pairs), a.nouter);
-  const size_t sm = pairs * fx_pair_smem<N, false>() + (size_t)N * pairs * sizeof(double2);
+  const size_t sm = pairs * fx_pair_smem<N, RM, false>() + (size_t)N * pairs * sizeof(double2);
   const double* symo = kp.dim == 2 ? nullptr : tb.sym[1];
   if (out32 == nullptr)
-    k_last_fx<N, EPI_THETA><<<grid, pairs * TS, sm, st>>>(data, theta, out32, a.line_stride, a.outer_stride, kp, ctrl,
+    k_last_fx<N, RM, EPI_THETA><<<grid, pairs * TS, sm, st>>>(data, theta, out32, a.line_stride, a.outer_stride, kp, ctrl,
                                                           partials, tb.fxtw[a.ax], tb.sym[0], symo, tb.sym[a.ax], dc,
                                                           skip);
   else
-    k_last_fx<N, EPI_RESID><<<grid, pairs * TS, sm, st>>>(data, theta, out32, a.line_stride, a.outer_stride, kp, ctrl,
+    k_last_fx<N, RM, EPI_RESID><<<grid, pairs * TS, sm, st>>>(data, theta, out32, a.line_stride, a.outer_stride, kp, ctrl,
                                                           partials, tb.fxtw[a.ax], tb.sym[0], symo, tb.sym[a.ax],
                                                           nullptr, skip);
   return cudaGetLastError();

@@ -482,25 +482,27 @@ size_t pair_smem() {
   return 2 * (size_t)line_stride_words<T, N, RM, ROWS>() * sizeof(T);
 }
 
-// Number of column pairs per block: fill 256 threads, bounded by the shared
-// memory budget, by the available pairs and by the autotuner's cap (0: no
-// cap); a power of two.
+// Number of line pairs per block: fill 256 threads, bounded by the shared
+// memory budget, by the available pairs and by the autotuner's cap (0: no cap),
+// narrower while SMs would be without a block (to one warp; strided passes to
+// four pairs, whole 32-byte sectors); a power of two.  total: pairs of the pass.
 template <typename T, int N, int RM, bool ROWS>
-int pick_pairs(int avail_pairs, int cap = 0) {
+int pick_pairs(long long total, int avail_pairs, int nsm, int cap = 0) {
   using F = LineFFT<T, N, RM>;
   int pairs = kThreads / F::TS;
   while (pairs > 1 && (size_t)pairs * pair_smem<T, N, RM, ROWS>() > kMaxSmem) pairs >>= 1;
   while (pairs > 1 && pairs > avail_pairs) pairs >>= 1;
+  while (pairs > (ROWS ? 1 : 4) && pairs * F::TS > 32 && total / pairs < nsm) pairs >>= 1;
   while (cap > 0 && pairs > 1 && pairs > cap) pairs >>= 1;
   return pairs < 1 ? 1 : pairs;
 }
 
 template <typename T, int N>
 cudaError_t rows_impl(const T* src, T* dst, int nrows, T scale, const int* done, const T* twc,
-                      const T* tws, cudaStream_t st, int cap = 0) {
+                      const T* tws, cudaStream_t st, int nsm, int cap) {
   constexpr int RM = kRadixPass;
   using F = LineFFT<T, N, RM>;
-  const int pairs = pick_pairs<T, N, RM, true>(1 << 30, cap);
+  const int pairs = pick_pairs<T, N, RM, true>(nrows / 2, 1 << 30, nsm, cap);
   const int rows_per_block = 2 * pairs;
   const int grid = (nrows + rows_per_block - 1) / rows_per_block;
   k_dht_rows<T, N, RM><<<grid, pairs * F::TS, pairs * pair_smem<T, N, RM, true>(), st>>>(
@@ -510,10 +512,10 @@ cudaError_t rows_impl(const T* src, T* dst, int nrows, T scale, const int* done,
 
 template <typename T, int N>
 cudaError_t cols_impl(T* data, int nx, int nouter, size_t line_stride, size_t outer_stride, T scale,
-                      const int* done, const T* twc, const T* tws, cudaStream_t st, int cap = 0) {
+                      const int* done, const T* twc, const T* tws, cudaStream_t st, int nsm, int cap) {
   constexpr int RM = kRadixPass;
   using F = LineFFT<T, N, RM>;
-  const int pairs = pick_pairs<T, N, RM, false>(nx / 2, cap);
+  const int pairs = pick_pairs<T, N, RM, false>((long long)(nx / 2) * nouter, nx / 2, nsm, cap);
   dim3 grid(nx / (2 * pairs), nouter);
   k_dht_cols<T, N, RM><<<grid, pairs * F::TS, pairs * pair_smem<T, N, RM, false>(), st>>>(
       data, line_stride, outer_stride, scale, done, twc, tws);
@@ -527,7 +529,8 @@ cudaError_t mid_impl(T* data, const KParams& kp, Ctrl* ctrl, double* partials, T
   using F = LineFFT<T, N, RM>;
   using V = typename Vec2<T>::type;
   const int nx = kp.nx;
-  const int pairs = pick_pairs<T, N, RM, false>(nx / 2, tb.tile_cap[2]);
+  const int pairs = pick_pairs<T, N, RM, false>((long long)(nx / 2) * (kp.dim == 2 ? 1 : kp.ny), nx / 2, tb.nsm,
+                                                tb.tile_cap[2]);
   size_t line_stride, outer_stride;
   int nouter;
   const T* symo;

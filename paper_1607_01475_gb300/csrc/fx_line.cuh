@@ -27,8 +27,8 @@
 // largest value, against 2^-53 of the value in FP64, with two to three units
 // on the outputs, so that the transform's error relative to the norm of the
 // line stays below that of the FP64 butterflies (tests/fx_line_check.cu
-// measures both against long double, for n = 8 .. 1024, dense and decaying
-// lines).  Lines whose largest value is below 2^-958 give zero; a NaN or an
+// measures both against long double, for n = 8 .. 1024 with radix 8 and
+// n = 8 .. 256 with radix 4, dense and decaying lines).  Lines whose largest value is below 2^-958 give zero; a NaN or an
 // infinity makes every output of its line pair NaN, as the FP64 sums would.
 #pragma once
 
@@ -148,16 +148,16 @@ __device__ __forceinline__ fx shfl_from<fx>(unsigned mask, fx v, int src) {
 
 constexpr int fx_log2(int n) { return n <= 1 ? 0 : 1 + fx_log2(n / 2); }
 
-// Passes, headroom and scale of the N-point line FFT with radix 8.
-template <int N>
+// Passes, headroom and scale of the N-point line FFT with radix RM.
+template <int N, int RM>
 struct FxPlan {
-  static constexpr int R = N < 8 ? N : 8;
-  static constexpr int lg = fx_log2(N);
-  static constexpr int P = (lg + 2) / 3;
+  static constexpr int R = N < RM ? N : RM;
+  static constexpr int lg = fx_log2(N), lr = fx_log2(R);
+  static constexpr int P = (lg + lr - 1) / lr;
   static constexpr int headroom() {
     int h = 0;
     for (int p = 1; p <= P; ++p) {
-      const int g = 3 * p < lg ? 3 * p : lg;
+      const int g = lr * p < lg ? lr * p : lg;
       if (g - 2 * (p - 1) > h) h = g - 2 * (p - 1);
     }
     return h;
@@ -178,7 +178,7 @@ __host__ __device__ __forceinline__ unsigned fx_l1(unsigned hi, int E) {
   return ((((hi & 0xFFFFFu) | 0x100000u) >> 1) >> (d < 31 ? d : 31)) + 1u;
 }
 // The scale B of a line whose L1 norm is below l1 2^(E - 1042).
-template <int N>
+template <class Plan>
 __host__ __device__ __forceinline__ int fx_scale(unsigned l1) {
 #ifdef __CUDA_ARCH__
   const int bits = 32 - __clz((int)l1);
@@ -186,7 +186,7 @@ __host__ __device__ __forceinline__ int fx_scale(unsigned l1) {
   const int bits = l1 ? 32 - __builtin_clz(l1) : 0;
 #endif
   const int B = 81 - bits;
-  return B < FxPlan<N>::B ? FxPlan<N>::B : (B > 60 ? 60 : B);
+  return B < Plan::B ? Plan::B : (B > 60 ? 60 : B);
 }
 
 // x 2^(B - (E - 1022)) rounded to nearest, from the bits of x (hi, lo), for a

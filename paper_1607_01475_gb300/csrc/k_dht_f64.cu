@@ -7,12 +7,14 @@ namespace psd {
 template <>
 cudaError_t launch_dht_rows<double>(const double* src, double* dst, int nx, int nrows, double scale, const int* done,
                                     const AxisTables<double>& tb, cudaStream_t st, unsigned int* dmax_hi) {
-  PSD_DISPATCH_N(nx, (rows_fx_impl<NN, double>(src, dst, nrows, scale, done, tb, st, dmax_hi)));
+  PSD_DISPATCH_N(nx, (fx_short((long long)nx * nrows, tb.nsm) ? rows_fx_impl<NN, kFxShort<NN>, double>(src, dst, nrows, scale, done, tb, st, dmax_hi)
+                                                              : rows_fx_impl<NN, 8, double>(src, dst, nrows, scale, done, tb, st, dmax_hi)));
 }
 
 cudaError_t launch_dht_rows_from_f32(const float* src, double* dst, int nx, int nrows, const AxisTables<double>& tb,
                                      cudaStream_t st, const int* skip) {
-  PSD_DISPATCH_N(nx, (rows_fx_impl<NN, float>(src, dst, nrows, 1.0, skip, tb, st, nullptr)));
+  PSD_DISPATCH_N(nx, (fx_short((long long)nx * nrows, tb.nsm) ? rows_fx_impl<NN, kFxShort<NN>, float>(src, dst, nrows, 1.0, skip, tb, st, nullptr)
+                                                              : rows_fx_impl<NN, 8, float>(src, dst, nrows, 1.0, skip, tb, st, nullptr)));
 }
 
 template <>
@@ -23,8 +25,11 @@ cudaError_t launch_dht_cols<double>(double* data, const KParams& kp, int ax, dou
   const size_t line_stride = ax == 1 ? (size_t)kp.nx : plane;
   const size_t outer_stride = ax == 1 ? plane : (size_t)kp.nx;
   const int nouter = ax == 1 ? kp.nz : kp.ny;
-  PSD_DISPATCH_N(n, (cols_fx_impl<NN>(data, kp.nx, nouter, line_stride, outer_stride, scale, done, tb.fxtw[ax], tb.nsm,
-                                      st)));
+  const bool small = fx_short((long long)plane * kp.nz, tb.nsm);
+  PSD_DISPATCH_N(n, (small ? cols_fx_impl<NN, kFxShort<NN>>(data, kp.nx, nouter, line_stride, outer_stride, scale, done,
+                                                 tb.fxtw[ax], tb.nsm, st)
+                           : cols_fx_impl<NN, 8>(data, kp.nx, nouter, line_stride, outer_stride, scale, done,
+                                                 tb.fxtw[ax], tb.nsm, st)));
 }
 
 #define PSD_INST_SPEC(T)                                                                               \

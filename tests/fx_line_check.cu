@@ -37,9 +37,9 @@ static unsigned lo(double x) {
 }
 
 // Pass NS of the Stockham FFT over a whole line, thread by thread.
-template <int N, int NS, typename T, typename Rot, typename Unt>
+template <int N, int RM, int NS, typename T, typename Rot, typename Unt>
 void pass(std::vector<T>& re, std::vector<T>& im, Rot rot, Unt unt) {
-  constexpr int R = N < 8 ? N : 8, TS = N / R, RP = (N / NS >= R) ? R : N / NS, M = R / RP;
+  constexpr int R = N < RM ? N : RM, TS = N / R, RP = (N / NS >= R) ? R : N / NS, M = R / RP;
   std::vector<T> ore(N), oim(N);
   for (int j = 0; j < TS; ++j)
     for (int b = 0; b < M; ++b) {
@@ -64,21 +64,21 @@ void pass(std::vector<T>& re, std::vector<T>& im, Rot rot, Unt unt) {
   im = oim;
 }
 
-template <int N, int NS, typename T, typename Rot, typename Unt>
+template <int N, int RM, int NS, typename T, typename Rot, typename Unt>
 void passes(std::vector<T>& re, std::vector<T>& im, Rot rot, Unt unt) {
-  constexpr int R = N < 8 ? N : 8;
+  constexpr int R = N < RM ? N : RM;
   if constexpr (NS < N) {
     constexpr int RP = (N / NS >= R) ? R : N / NS;
-    pass<N, NS>(re, im, rot, unt);
-    passes<N, NS * RP>(re, im, rot, unt);
+    pass<N, RM, NS>(re, im, rot, unt);
+    passes<N, RM, NS * RP>(re, im, rot, unt);
   }
 }
 
 // Hartley outputs of the pair (x, y) in fixed point.
-template <int N>
+template <int N, int RM>
 void run_fx(const std::vector<double>& x, const std::vector<double>& y, std::vector<double>& h1,
             std::vector<double>& h2) {
-  using Plan = psd::FxPlan<N>;
+  using Plan = psd::FxPlan<N, RM>;
   std::vector<psd::fx_tw> tw(N);
   const long double pi = 3.141592653589793238462643383279502884L;
   for (int t = 0; t < N; ++t) tw[t] = psd::fx_make_tw(cosl(2 * pi * t / N), sinl(2 * pi * t / N));
@@ -92,13 +92,13 @@ void run_fx(const std::vector<double>& x, const std::vector<double>& y, std::vec
   std::vector<fx> re(N), im(N);
   unsigned l1 = 0;
   for (int i = 0; i < N; ++i) l1 += psd::fx_l1(hi(x[i]), E) + psd::fx_l1(hi(y[i]), E);
-  const int scale = psd::fx_scale<N>(l1);
+  const int scale = psd::fx_scale<Plan>(l1);
   for (int i = 0; i < N; ++i) {
     re[i] = psd::fx_quantise(hi(x[i]), lo(x[i]), E, scale);
     im[i] = psd::fx_quantise(hi(y[i]), lo(y[i]), E, scale);
     if (!live) re[i].v = im[i].v = 0;
   }
-  passes<N, 1>(
+  passes<N, RM, 1>(
       re, im, [&](int t, fx& a, fx& b, bool odd) { psd::fx_rotate(a, b, tw[t], odd); },
       [](fx& a, fx& b) {
         a = psd::fx_quarter(a);
@@ -116,7 +116,7 @@ void run_fx(const std::vector<double>& x, const std::vector<double>& y, std::vec
 }
 
 // The same passes in FP64.
-template <int N>
+template <int N, int RM>
 void run_f64(const std::vector<double>& x, const std::vector<double>& y, std::vector<double>& h1,
              std::vector<double>& h2) {
   const long double pi = 3.141592653589793238462643383279502884L;
@@ -125,7 +125,7 @@ void run_f64(const std::vector<double>& x, const std::vector<double>& y, std::ve
     c[t] = (double)cosl(2 * pi * t / N);
     s[t] = (double)sinl(2 * pi * t / N);
   }
-  passes<N, 1>(
+  passes<N, RM, 1>(
       re, im,
       [&](int t, double& a, double& b, bool) {
         const double a0 = a;
@@ -160,7 +160,7 @@ std::vector<long double> exact(const std::vector<double>& x) {
 
 static int fails = 0;
 
-template <int N>
+template <int N, int RM>
 void check() {
   // kinds of lines: dense, one large point, spectra decaying like k^-4 and
   // exp(-k^2 / 64), a constant, a smooth mode, values over 60 binades, tiny and
@@ -190,8 +190,8 @@ void check() {
           y[i] = std::sin(6.283185307179586 * 2 * i / N);
         }
       }
-      run_fx<N>(x, y, a, b);
-      run_f64<N>(x, y, c, d);
+      run_fx<N, RM>(x, y, a, b);
+      run_f64<N, RM>(x, y, c, d);
       const auto u = exact<N>(x), v = exact<N>(y);
       long double scale = 0;
       for (int i = 0; i < N; ++i) scale = std::max(scale, std::max(fabsl(u[i]), fabsl(v[i])));
@@ -208,25 +208,25 @@ void check() {
     // (unrelated magnitudes over 60 binades, which no field or spectrum here has,
     // may lose one bit at n = 1024)
     const double bound = std::fmax(kind == 6 && N == 1024 ? 2.0 * rd : rd, 0x1p-53);
-    std::printf("n %4d %-9s fixed %.2e  fp64 %.2e%s\n", N, names[kind], rx, rd, rx > bound ? "  LARGER" : "");
+    std::printf("n %4d radix %d %-9s fixed %.2e  fp64 %.2e%s\n", N, RM, names[kind], rx, rd, rx > bound ? "  LARGER" : "");
     if (!(rx <= bound)) ++fails;
   }
   // special values: NaN and infinity spoil the pair, zeros and values below the
   // range give zero, the largest values give infinity or finite values as sums do
   std::vector<double> x(N, 0.0), y(N, 0.0), a, b;
-  run_fx<N>(x, y, a, b);
+  run_fx<N, RM>(x, y, a, b);
   for (int i = 0; i < N; ++i)
     if (a[i] != 0.0 || b[i] != 0.0) ++fails;
   x[N / 2] = INFINITY;
-  run_fx<N>(x, y, a, b);
+  run_fx<N, RM>(x, y, a, b);
   for (int i = 0; i < N; ++i)
     if (!std::isnan(a[i]) || !std::isnan(b[i])) ++fails;
   x[N / 2] = 1e-300;
-  run_fx<N>(x, y, a, b);
+  run_fx<N, RM>(x, y, a, b);
   for (int i = 0; i < N; ++i)
     if (a[i] != 0.0) ++fails;
   x.assign(N, 1.5e308);
-  run_fx<N>(x, y, a, b);
+  run_fx<N, RM>(x, y, a, b);
   if (!std::isinf(a[0]) || a[0] < 0) ++fails;
   // extremes of the headroom: all points at the largest magnitude, with signs
   // that add up in some output
@@ -237,7 +237,7 @@ void check() {
       y[i] = std::sin(th) >= 0 ? std::nextafter(1.0, 0.0) : -std::nextafter(1.0, 0.0);
     }
     if (N > 64 && k % (N / 32)) continue;
-    run_fx<N>(x, y, a, b);
+    run_fx<N, RM>(x, y, a, b);
     const auto u = exact<N>(x), v = exact<N>(y);
     for (int i = 0; i < N; ++i)
       if (fabsl(a[i] - u[i]) > N * 0x1p-52 || fabsl(b[i] - v[i]) > N * 0x1p-52) ++fails;
@@ -279,14 +279,20 @@ int main() {
       if (fabsl(F[c] - want) > 4.0L || fabsl((long double)F[c]) > 0x1p58L) ++fails;
     }
   }
-  check<8>();
-  check<16>();
-  check<32>();
-  check<64>();
-  check<128>();
-  check<256>();
-  check<512>();
-  check<1024>();
+  check<8, 8>();
+  check<8, 4>();
+  check<16, 8>();
+  check<16, 4>();
+  check<32, 8>();
+  check<32, 4>();
+  check<64, 8>();
+  check<64, 4>();
+  check<128, 8>();
+  check<128, 4>();
+  check<256, 8>();
+  check<256, 4>();
+  check<512, 8>();
+  check<1024, 8>();
   std::printf(fails ? "FAILED (%d)\n" : "OK\n", fails);
   return fails ? 1 : 0;
 }
