@@ -235,10 +235,12 @@ __device__ __forceinline__ void mid_finish(T (&acc)[mid_nsums<T, ORDER>()], T* s
       }
       // reset the line-search state for this iteration (general-p Newton:
       // bracket [c1, c2] with c2 < 0 meaning "no upper end yet", c3 = done; the
-      // previous step size stays in alpha as the first trial)
+      // previous step size is the first trial)
       ctrl->c1 = 0.0;
       ctrl->c2 = -1.0;
       ctrl->c3 = 0.0;
+      ctrl->trial = ctrl->alpha;
+      ctrl->alpha = 0.0;
       ctrl->ls_pass = 0;
       ctrl->dmax_hi = 0u;
       ctrl->counter[CS_MID] = 0;

@@ -451,10 +451,11 @@ __global__ void __launch_bounds__(NT) k_dot(const double* x, const double* y, co
 
 inline int grid1d(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 152 * 16); }
 
-#ifndef PSD_M2D
-#define PSD_M2D 8
-#endif
-constexpr int kMarchesPerSM = PSD_M2D;  // 2D kernels
+// 2D marches per SM: 1024^2 FP32 residual (event-timed) with 4, 8, 16, 32: 15.2,
+// 13.8, 16.7, 21.1 us.
+constexpr int kMarchesPerSM = 8;
+// Least planes per CTA of the 3D FP32 marches: 4, 8 and 16 measured alike at 128^3.
+constexpr int kMarchPlanes = 8;
 int pick_zc(int nz, int nblk_xy) {
   // z planes per CTA: enough CTAs to fill the GPU, long enough marches
   int zc = nz;
@@ -465,14 +466,13 @@ int pick_zc(int nz, int nblk_xy) {
 }  // namespace
 
 // Launch geometry of the residual and line-search kernels (ctas_per_sm =
-// the residency their __launch_bounds__ guarantee).  3D FP32 grids large
-// enough to fill the GPU with 32 x 32 tiles take the register-blocked
-// kernels (the FP32 residual is bound by instruction issue and shared-memory
-// traffic); FP64 and smaller grids the column kernels; tiles below 32 x 8
-// the general kernel.  The register-blocked and column kernels run one wave
-// of CTAs: the CTAs per SM times the SMs (cached in KParams at setup, so
-// captured and direct launches agree and the partial sums come in the same
-// order), at most one CTA per 16 (8) column-planes.
+// the residency their __launch_bounds__ guarantee).  2D: warp marches.  3D FP32:
+// the register-blocked tiles on grids that fill the GPU with 32 x 32 tiles,
+// warp marches on the others.  3D FP64: the column kernels; tiles below 32 x 8
+// the general kernel.  The 3D kernels but the general one run one wave of CTAs:
+// the CTAs per SM times the SMs (cached in KParams at setup, so captured and
+// direct launches agree and the partial sums come in the same order), with a
+// least number of column-planes per CTA.
 ResGeom res_geometry(const KParams& kp, bool fp32, int ctas_per_sm, bool linesearch, bool pairs) {
   ResGeom g{RK_2D, dim3(1, 1, 1), 1, NT};
   if (kp.dim != 3) {
@@ -499,6 +499,16 @@ ResGeom res_geometry(const KParams& kp, bool fp32, int ctas_per_sm, bool linesea
     g.kind = RK_RB4;
     g.grid = dim3((unsigned)std::min(wave, w / 16));
     g.zc = 0;
+    return g;
+  }
+  if (fp32) {
+    // at most one CTA per kMarchPlanes column-planes (a march starts with 4 planes more)
+    const int strip = linesearch ? 31 : 28, warps = std::min(kMarchWarps, kp.ny / 4);
+    const long long w = (long long)((kp.nx + strip - 1) / strip) * (kp.ny / (4 * warps)) * kp.nz;
+    const long long most = (long long)(linesearch ? kMarchLsCtas : kMarchResCtas) * kp.nsm;
+    g.kind = RK_MARCH;
+    g.grid = dim3((unsigned)std::max(1LL, std::min(most, w / kMarchPlanes)));
+    g.threads = 32 * warps;
     return g;
   }
   const int TX = kp.nx < BX ? kp.nx : BX, TY = kp.ny < BY3 ? kp.ny : BY3;

@@ -35,6 +35,7 @@ struct Ctrl {
   // weighted by h^d and s), or the general-p Newton state (c1, c2 = bracket,
   // c3 = converged flag)
   double c1, c2, c3;
+  double trial;    // general p: the step size at which the next Newton pass evaluates q
   // inner (mixed-precision) stop on the preconditioned residual norm
   // (r, L_h^{-1} r)^{1/2} = ||d||_L (Eq. "RRT-1"): done when it drops below
   // pre_eta times its first value pre_ref (pre_eta <= 0 disables).

@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kWarps2D * 32)
   __shared__ T sred[red_size<T>(ls_nsums<PK>())];
   __shared__ unsigned smax[2];
   __shared__ int sflag;
-  const T trial = ls_closed_form<PK>() ? T(0) : (T)ctrl->alpha;
+  const T trial = ls_closed_form<PK>() ? T(0) : (T)ctrl->trial;
   T acc[ls_nsums<PK>()] = {};
   T sbb = T(0);
   unsigned gm = 0u;

@@ -470,7 +470,7 @@ __device__ __forceinline__ void ls3d_col(const T* __restrict__ u, const T* __res
   const int nx = kp.nx, ny = kp.ny, nz = kp.nz;
   const size_t plane = (size_t)nx * ny;
   const T beta = kconst<T>(kp).beta, pm2 = kconst<T>(kp).pm2;
-  const T trial = ls_closed_form<PK>() ? T(0) : (T)ctrl->alpha;
+  const T trial = ls_closed_form<PK>() ? T(0) : (T)ctrl->trial;
   // one wave of CTAs, each marching an equal share of the column-planes (as
   // the residual column kernel)
   const int gx = nx / TX;

@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(256, 3)
   const int nx = kp.nx, ny = kp.ny, nz = kp.nz;
   const size_t plane = (size_t)nx * ny;
   const T beta = kconst<T>(kp).beta, pm2 = kconst<T>(kp).pm2;
-  const T trial = ls_closed_form<PK>() ? T(0) : (T)ctrl->alpha;
+  const T trial = ls_closed_form<PK>() ? T(0) : (T)ctrl->trial;
   const int cy0 = ty * NY;
   const bool hv = tid < NH;
   const int hly = tid < SY ? tid : TYT, hlx = tid < SY ? TX : tid - SY;

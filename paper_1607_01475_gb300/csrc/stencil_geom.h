@@ -11,8 +11,10 @@ constexpr int BX = 32;   // tile width (x)
 constexpr int BY3 = 8;   // tile height (y), 3D
 constexpr int kWarps2D = 4;  // most marches (warps) per block, 2D
 constexpr int NT = 256;  // threads per block
+// 3D FP32 marches: most warps (four rows each) per CTA, CTAs per SM
+constexpr int kMarchWarps = 4, kMarchResCtas = 2, kMarchLsCtas = 5;
 
-enum ResKind { RK_2D, RK_SMALL3D, RK_COL, RK_RB4 };
+enum ResKind { RK_2D, RK_SMALL3D, RK_COL, RK_RB4, RK_MARCH };
 struct ResGeom {
   int kind;
   dim3 grid;

@@ -608,7 +608,7 @@ __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double 
     // flag); the first trial is the previous iteration's step size.  A step below
     // 1e-4 of alpha (FP32 sums, whose alpha is used rounded to FP32) or 5e-9 (FP64)
     // is the last: what it leaves is of the order of its square.
-    const double trial = f32 ? (double)(float)ctrl->alpha : ctrl->alpha;
+    const double trial = f32 ? (double)(float)ctrl->trial : ctrl->trial;
     const double qv = -ctrl->rd + trial * lin + kp.cdiv * kp.hd * tot[0];
     const double dqv = lin + kp.cdiv * kp.hd * tot[1];
     double lo = ctrl->c1, hi = ctrl->c2;
@@ -633,6 +633,7 @@ __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double 
     ctrl->c1 = lo;
     ctrl->c2 = hi;
     ctrl->alpha = nw;
+    ctrl->trial = nw;
     if (!isfinite(nw) || !isfinite(qv)) {
       ctrl->status = 7;
       ctrl->done = 1;
@@ -671,6 +672,7 @@ __device__ __forceinline__ void ls_finish(T (&acc)[ls_nsums<PK>()], T* sred, dou
 }  // namespace psd
 #include "stencil2d.cuh"
 #include "stencil3d_col.cuh"
+#include "stencil3d_march.cuh"
 #include "stencil3d_rb.cuh"
 namespace psd {
 namespace {
@@ -693,7 +695,7 @@ __global__ void __launch_bounds__(NT)
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * zc;
   const size_t plane = (size_t)nx * ny;
   const T beta = kconst<T>(kp).beta, pm2 = kconst<T>(kp).pm2;
-  const T trial = ls_closed_form<PK>() ? T(0) : (T)ctrl->alpha;
+  const T trial = ls_closed_form<PK>() ? T(0) : (T)ctrl->trial;
   auto load = [&](int zz) {
     const int sl_ = (zz - z0) & 1;
     const size_t gz = (size_t)wrapi(zz, nz) * plane;
@@ -745,14 +747,17 @@ template <typename T, int PK, int MODE>
 cudaError_t res_impl(const ResArgs<T>& a, const KParams& kp, Ctrl* ctrl, double* partials, cudaStream_t st) {
   const ResGeom g = residual_geometry(kp, sizeof(T) == 4, aligned8(a.u_in, a.d, a.u_out, a.f, a.ubase, a.r));
   switch (g.kind) {
+    case RK_MARCH:
+      if constexpr (sizeof(T) == 4) k_res3d_march<T, PK, MODE><<<g.grid, g.threads, 0, st>>>(a, kp, ctrl, partials);
+      break;
     case RK_RB4:
       if constexpr (sizeof(T) == 4) k_res3d_rb<T, PK, MODE, 4><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials);
       break;
     case RK_COL:
-      k_res3d_col<T, PK, MODE><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials);
+      if constexpr (sizeof(T) == 8) k_res3d_col<T, PK, MODE><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials);
       break;
     case RK_SMALL3D:
-      k_res3d<T, PK, MODE><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials, g.zc);
+      if constexpr (sizeof(T) == 8) k_res3d<T, PK, MODE><<<g.grid, NT, 0, st>>>(a, kp, ctrl, partials, g.zc);
       break;
     default:
       if constexpr (sizeof(T) == 4) {
@@ -772,14 +777,18 @@ cudaError_t ls_impl(const T* u, const T* ubase, const T* d, const KParams& kp, C
   // the same tiles as the residual; __launch_bounds__(256, 3)
   const ResGeom g = res_geometry(kp, sizeof(T) == 4, 3, true, aligned8(u, ubase, d));
   switch (g.kind) {
+    case RK_MARCH:
+      if constexpr (sizeof(T) == 4)
+        k_ls3d_march<T, PK, INNER><<<g.grid, g.threads, 0, st>>>(u, ubase, d, kp, ctrl, partials);
+      break;
     case RK_RB4:
       if constexpr (sizeof(T) == 4) k_ls3d_rb<T, PK, INNER, 4><<<g.grid, NT, 0, st>>>(u, ubase, d, kp, ctrl, partials);
       break;
     case RK_COL:
-      k_ls3d_col<T, PK, INNER><<<g.grid, NT, 0, st>>>(u, ubase, d, kp, ctrl, partials);
+      if constexpr (sizeof(T) == 8) k_ls3d_col<T, PK, INNER><<<g.grid, NT, 0, st>>>(u, ubase, d, kp, ctrl, partials);
       break;
     case RK_SMALL3D:
-      k_ls3d<T, PK, INNER><<<g.grid, NT, 0, st>>>(u, ubase, d, kp, ctrl, partials, g.zc);
+      if constexpr (sizeof(T) == 8) k_ls3d<T, PK, INNER><<<g.grid, NT, 0, st>>>(u, ubase, d, kp, ctrl, partials, g.zc);
       break;
     default:
       if constexpr (sizeof(T) == 4) {
