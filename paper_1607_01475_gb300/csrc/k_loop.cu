@@ -96,6 +96,8 @@ __global__ void k_ctrl_reset(Ctrl* c) {
   *c = z;
 }
 
+__global__ void k_ctrl_set(Ctrl* c, const Ctrl h) { *c = h; }
+
 inline int grid1d(size_t n) { return (int)((n + 255) / 256 < 152 * 16 ? (n + 255) / 256 : 152 * 16); }
 
 }  // namespace
@@ -126,6 +128,10 @@ cudaError_t launch_mixed_check(Ctrl* c3, const Ctrl* c2, Ctrl* c, const Ctrl* tm
 }
 cudaError_t launch_mixed_after(Ctrl* c3, const Ctrl* c, cudaStream_t st) {
   k_mixed_after<<<1, 1, 0, st>>>(c3, c);
+  return cudaGetLastError();
+}
+cudaError_t launch_ctrl_set(Ctrl* c, const Ctrl& h, cudaStream_t st) {
+  k_ctrl_set<<<1, 1, 0, st>>>(c, h);
   return cudaGetLastError();
 }
 cudaError_t launch_ctrl_reset(Ctrl* c, cudaStream_t st) {

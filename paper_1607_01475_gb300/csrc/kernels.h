@@ -174,6 +174,8 @@ cudaError_t launch_mixed_check(Ctrl* c3, const Ctrl* c2, Ctrl* c, const Ctrl* tm
 cudaError_t launch_mixed_after(Ctrl* c3, const Ctrl* c, cudaStream_t st);
 // c = a fresh control block (tol -1, no iteration limit), on device.
 cudaError_t launch_ctrl_reset(Ctrl* c, cudaStream_t st);
+// *c = h, on the stream (h travels as the kernel's argument).
+cudaError_t launch_ctrl_set(Ctrl* c, const Ctrl& h, cudaStream_t st);
 
 // ------------------------------------------------------------ adjoint CG
 // lam += alpha p, r -= alpha q, w = r; ||r||_2, iteration count and stopping

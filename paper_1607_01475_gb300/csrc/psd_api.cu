@@ -90,8 +90,7 @@ struct psd_context {
   Ctrl* ctrl2 = nullptr;  // auxiliary reductions (outer residual, norms)
   Ctrl* ctrl3 = nullptr;  // mixed solve: outer-loop state of the captured solve
   Ctrl* ctrl_tmpl = nullptr;  // mixed solve: control block of a fresh inner solve
-  Ctrl* h_ctrl = nullptr; // pinned host mirror: [0] synchronous transfers, [1..3] staging of
-                          // asynchronous uploads (a batch's host part)
+  Ctrl* h_ctrl = nullptr; // pinned host mirror of a control block read back
 
   double* d_hist = nullptr;
   double* user_alpha = nullptr;
@@ -366,18 +365,11 @@ void init_ctrl(Ctrl& h, double tol, int max_iter) {
   h.fx_s = psd::kFxOff;
 }
 
+// A control block written on the stream by a kernel that carries it as its
+// argument: no staging buffer and no host wait (a copy from the pinned mirror had to
+// be waited for before the mirror was used again, about 10 us each).
 psd_status upload_ctrl(psd_context* c, Ctrl* dst, const Ctrl& h) {
-  *c->h_ctrl = h;
-  CK(cudaMemcpyAsync(dst, c->h_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, c->st));
-  CK(cudaStreamSynchronize(c->st));
-  return PSD_OK;
-}
-
-// Upload without waiting, from staging slot `slot` (1..3) of the pinned
-// mirror; the slot must not be reused before the copy has run.
-psd_status upload_ctrl_async(psd_context* c, Ctrl* dst, const Ctrl& h, int slot) {
-  c->h_ctrl[slot] = h;
-  CK(cudaMemcpyAsync(dst, c->h_ctrl + slot, sizeof(Ctrl), cudaMemcpyHostToDevice, c->st));
+  CK(psd::launch_ctrl_set(dst, h, c->st));
   return PSD_OK;
 }
 
@@ -1042,8 +1034,6 @@ psd_status autotune(psd_context* c) {
 // ------------------------------------------------ batch (internal hooks)
 // The host part of a solve before its graph work: control blocks uploaded
 // (and, order 6 mixed, the mean projection of u0).
-// The uploads are asynchronous on the handle's stream (work enqueued on that
-// stream after them sees them).
 psd_status solve_prepare(psd_context* c, const double* f, const double* g, double* u) {
   TRY(ensure_fp64(c));
   if (c->prm.precision == PSD_MIXED) {
@@ -1052,14 +1042,14 @@ psd_status solve_prepare(psd_context* c, const double* f, const double* g, doubl
     Ctrl h3;
     init_ctrl(h3, -1.0, 1 << 30);
     h3.status = PSD_ERR_NOCONV;
-    TRY(upload_ctrl_async(c, c->ctrl3, h3, 1));
+    TRY(upload_ctrl(c, c->ctrl3, h3));
     Ctrl ht;
     inner_ctrl(c, ht, 0);
-    TRY(upload_ctrl_async(c, c->ctrl_tmpl, ht, 2));
+    TRY(upload_ctrl(c, c->ctrl_tmpl, ht));
   } else {
     Ctrl h;
     init_ctrl(h, c->prm.tol, c->prm.max_iter);
-    TRY(upload_ctrl_async(c, c->ctrl, h, 1));
+    TRY(upload_ctrl(c, c->ctrl, h));
   }
   (void)f;
   return PSD_OK;
@@ -1272,7 +1262,7 @@ psd_status psd_create(const psd_params* params, psd_handle* out) {
     c->err = "cudaMemset failed";
     return bail(PSD_ERR_CUDA);
   }
-  if (cudaMallocHost((void**)&c->h_ctrl, 4 * sizeof(Ctrl)) != cudaSuccess) {
+  if (cudaMallocHost((void**)&c->h_ctrl, sizeof(Ctrl)) != cudaSuccess) {
     cudaGetLastError();
     c->err = "cudaMallocHost failed";
     return bail(PSD_ERR_NOMEM);
