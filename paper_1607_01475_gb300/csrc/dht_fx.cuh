@@ -3,11 +3,11 @@
 // the preconditioner and the last pass of the mixed solver's outer loop.
 // Data in memory is FP64 before and after every pass.
 //
-// At 256^3 a pass moves 268 MB (40 us at the measured copy rate) and takes 105
+// At 256^3 a pass moves 268 MB (40 us at the measured copy rate) and takes 92
 // us (rows, columns), bound by integer issue; with FP64 butterflies it took 547
-// us.  The sixth-order middle pass takes 723 us instead of 1711, bound by the
-// 17 FP64 operations per element of the symbol division and the Parseval sums
-// (545 us at 1.74 per clock and SM).
+// us.  The sixth-order middle pass takes 628 us instead of 1711, bound by the
+// 15 FP64 operations per element of the symbol division and the Parseval sums
+// (480 us at 1.74 per clock and SM).
 #pragma once
 
 #include <algorithm>
@@ -143,6 +143,18 @@ __device__ __forceinline__ double fx_leave(fx w, const FxLine& ln, int scale_e) 
   return ln.E > kFxMaxExp ? __longlong_as_double(0x7FF8000000000000LL)
                           : fx_result(w.v, ln.E - ln.B + FxPlan<N, RM>::kOut + scale_e);
 }
+// The same by the hardware conversion and an addition to the exponent, for the
+// passes whose FP64 pipe is otherwise idle (one FP64-rate operation instead of
+// about 20 integer ones; 256^3 row pass 107 -> 94 us, event-timed).  Lines whose outputs
+// could leave the normal range take fx_leave.
+template <int N, int RM>
+__device__ __forceinline__ double fx_leave_hw(fx w, const FxLine& ln, int scale_e) {
+  const int e = ln.E - ln.B + FxPlan<N, RM>::kOut + scale_e;
+  if (ln.E > kFxMaxExp || (unsigned)(e + 1000) >= 1900u) return fx_leave<N, RM>(w, ln, scale_e);
+  const double v = __ll2double_rn(w.v);
+  const int hi = __double2hiint(v);
+  return __hiloint2double(hi == 0 ? 0 : hi + (e << 20), __double2loint(v));
+}
 
 // -------------------------------------------------------------- x (rows)
 template <int N, int RM, typename SI>
@@ -178,7 +190,7 @@ __global__ void __launch_bounds__(kFxThreads, 3)
   double* d0 = dst + (size_t)row0 * N;
   unsigned top = 0u;  // largest magnitude written, high word
   auto put = [&](int k, fx h1, fx h2) {
-    const double a = fx_leave<N, RM>(h1, ln, scale_e), b = fx_leave<N, RM>(h2, ln, scale_e);
+    const double a = fx_leave_hw<N, RM>(h1, ln, scale_e), b = fx_leave_hw<N, RM>(h2, ln, scale_e);
     d0[k] = a;
     d0[N + k] = b;
     top = max(top, max((unsigned)__double2hiint(a) & 0x7FFFFFFFu, (unsigned)__double2hiint(b) & 0x7FFFFFFFu));
@@ -265,7 +277,7 @@ __global__ void __launch_bounds__(kFxThreads, 3)
     fx h1, h2;
     dht_split(sr, si, kk, N, h1, h2);
     *reinterpret_cast<double2*>(data + base + (size_t)kk * line_stride) =
-        make_double2(fx_leave<N, RM>(h1, ln, scale_e), fx_leave<N, RM>(h2, ln, scale_e));
+        make_double2(fx_leave_hw<N, RM>(h1, ln, scale_e), fx_leave_hw<N, RM>(h2, ln, scale_e));
   }
 }
 
