@@ -308,12 +308,23 @@ __global__ void __launch_bounds__(NT) k_cg_update(T* lam, const T* p, T* r, cons
   if (ctrl->done) return;
   const T al = (T)ctrl->alpha;
   T acc = T(0);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const T ri = r[i] - al * q[i];
-    lam[i] += al * p[i];
-    r[i] = ri;
-    w[i] = ri;
-    acc += ri * ri;
+  // 16-byte accesses (the arrays are the handle's, the grids multiples of 16)
+  constexpr int V = 16 / sizeof(T);
+  struct __align__(16) Vec {
+    T v[V];
+  };
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n / V; i += (size_t)gridDim.x * blockDim.x) {
+    Vec x = reinterpret_cast<Vec*>(lam)[i], ri = reinterpret_cast<Vec*>(r)[i];
+    const Vec pi = reinterpret_cast<const Vec*>(p)[i], qi = reinterpret_cast<const Vec*>(q)[i];
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      ri.v[k] -= al * qi.v[k];
+      x.v[k] += al * pi.v[k];
+      acc += ri.v[k] * ri.v[k];
+    }
+    reinterpret_cast<Vec*>(lam)[i] = x;
+    reinterpret_cast<Vec*>(r)[i] = ri;
+    reinterpret_cast<Vec*>(w)[i] = ri;
   }
   T v[1] = {acc};
   block_reduce<T, 1, false>(v, sred);
