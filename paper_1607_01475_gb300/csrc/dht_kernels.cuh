@@ -127,27 +127,30 @@ __global__ void __launch_bounds__(kThreads, 3)  // 80 registers
   const int tid = threadIdx.x;
   const int pairs = blockDim.x / F::TS;
   const int p = tid % pairs, j = tid / pairs;
-  const size_t base = (size_t)blockIdx.y * outer_stride + (size_t)blockIdx.x * 2 * pairs + 2 * p;
+  // byte offsets in 32 bits from the tile's (uniform) start: a line's extent is
+  // below 2^32 bytes
+  T* tile = data + ((size_t)blockIdx.y * outer_stride + (size_t)blockIdx.x * 2 * pairs);
+  const unsigned ls = (unsigned)line_stride * (unsigned)sizeof(T);
+  const unsigned off = (unsigned)j * ls + (unsigned)(2 * p) * (unsigned)sizeof(T), step = (unsigned)F::TS * ls;
   constexpr int LS = line_stride_words<T, N, RM, false>();
   T* sr = sm + (size_t)p * 2 * LS;
   T* si = sr + LS;
   T vr[F::R], vi[F::R];
 #pragma unroll
   for (int q = 0; q < F::R; ++q) {
-    const V v = *reinterpret_cast<const V*>(data + base + (size_t)(j + q * F::TS) * line_stride);
+    const V v = *reinterpret_cast<const V*>(reinterpret_cast<const char*>(tile) + (off + (unsigned)q * step));
     vr[q] = v.x;
     vi[q] = v.y;
   }
   F::run(vr, vi, j, sr, si, twc, tws);
 #pragma unroll
   for (int q = 0; q < F::R; ++q) {
-    const int k = j + q * F::TS;
     T h1, h2;
-    dht_split(sr, si, k, N, h1, h2);
+    dht_split(sr, si, j + q * F::TS, N, h1, h2);
     V o;
     o.x = h1 * scale;
     o.y = h2 * scale;
-    *reinterpret_cast<V*>(data + base + (size_t)k * line_stride) = o;
+    *reinterpret_cast<V*>(reinterpret_cast<char*>(tile) + (off + (unsigned)q * step)) = o;
   }
 }
 
