@@ -159,8 +159,8 @@ __device__ __forceinline__ double fx_leave_hw(fx w, const FxLine& ln, int scale_
 // -------------------------------------------------------------- x (rows)
 template <int N, int RM, typename SI>
 __global__ void __launch_bounds__(kFxThreads, 3)
-    k_rows_fx(const SI* src, double* dst, int nrows, int scale_e, const int* done, const fx_tw* __restrict__ tab,
-              unsigned int* dmax_hi) {
+    k_rows_fx(const SI* src, const SI* src_odd, const int* iter, double* dst, int nrows, int scale_e, const int* done,
+              const fx_tw* __restrict__ tab, unsigned int* dmax_hi) {
   using F = LineFFT<fx, N, RM>;
   constexpr int R = F::R, TS = F::TS;
   if (done != nullptr && *done) return;
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kFxThreads, 3)
   fx* si = sr + LS;
   FxTeam<N, RM, true> team{p, pairs};
   double xr[R], xi[R];
-  const SI* s0 = src + (size_t)row0 * N;
+  const SI* s0 = (iter != nullptr && (*iter & 1) ? src_odd : src) + (size_t)row0 * N;
 #pragma unroll
   for (int q = 0; q < R; ++q) {
     xr[q] = valid ? fx_load(s0[j + q * TS]) : 0.0;
@@ -518,14 +518,14 @@ inline bool fx_scale_exp(double scale, int* e) {
 }
 
 template <int N, int RM, typename SI>
-cudaError_t rows_fx_impl(const SI* src, double* dst, int nrows, double scale, const int* done,
+cudaError_t rows_fx_impl(const SI* src, const SI* src_odd, const int* iter, double* dst, int nrows, double scale, const int* done,
                          const AxisTables<double>& tb, cudaStream_t st, unsigned int* dmax_hi) {
   constexpr int TS = LineFFT<fx, N, RM>::TS;
   int se;
   if (!fx_scale_exp(scale, &se)) return cudaErrorInvalidValue;
   const int np = (nrows + 1) / 2;
   const int pairs = fx_pairs<N, RM, true>(np, 1 << 30, tb.nsm);
-  k_rows_fx<N, RM, SI><<<(np + pairs - 1) / pairs, pairs * TS, pairs * fx_pair_smem<N, RM, true>(), st>>>(src, dst, nrows, se,
+  k_rows_fx<N, RM, SI><<<(np + pairs - 1) / pairs, pairs * TS, pairs * fx_pair_smem<N, RM, true>(), st>>>(src, src_odd, iter, dst, nrows, se,
                                                                                                  done, tb.fxtw[0], dmax_hi);
   return cudaGetLastError();
 }

@@ -7,14 +7,14 @@ namespace psd {
 template <>
 cudaError_t launch_dht_rows<double>(const double* src, double* dst, int nx, int nrows, double scale, const int* done,
                                     const AxisTables<double>& tb, cudaStream_t st, unsigned int* dmax_hi) {
-  PSD_DISPATCH_N(nx, (fx_short((long long)nx * nrows, tb.nsm) ? rows_fx_impl<NN, kFxShort<NN>, double>(src, dst, nrows, scale, done, tb, st, dmax_hi)
-                                                              : rows_fx_impl<NN, 8, double>(src, dst, nrows, scale, done, tb, st, dmax_hi)));
+  PSD_DISPATCH_N(nx, (fx_short((long long)nx * nrows, tb.nsm) ? rows_fx_impl<NN, kFxShort<NN>, double>(src, src, nullptr, dst, nrows, scale, done, tb, st, dmax_hi)
+                                                              : rows_fx_impl<NN, 8, double>(src, src, nullptr, dst, nrows, scale, done, tb, st, dmax_hi)));
 }
 
-cudaError_t launch_dht_rows_from_f32(const float* src, double* dst, int nx, int nrows, const AxisTables<double>& tb,
-                                     cudaStream_t st, const int* skip) {
-  PSD_DISPATCH_N(nx, (fx_short((long long)nx * nrows, tb.nsm) ? rows_fx_impl<NN, kFxShort<NN>, float>(src, dst, nrows, 1.0, skip, tb, st, nullptr)
-                                                              : rows_fx_impl<NN, 8, float>(src, dst, nrows, 1.0, skip, tb, st, nullptr)));
+cudaError_t launch_dht_rows_from_f32(const float* src, const float* src_odd, const int* iter, double* dst, int nx,
+                                     int nrows, const AxisTables<double>& tb, cudaStream_t st, const int* skip) {
+  PSD_DISPATCH_N(nx, (fx_short((long long)nx * nrows, tb.nsm) ? rows_fx_impl<NN, kFxShort<NN>, float>(src, src_odd, iter, dst, nrows, 1.0, skip, tb, st, nullptr)
+                                                              : rows_fx_impl<NN, 8, float>(src, src_odd, iter, dst, nrows, 1.0, skip, tb, st, nullptr)));
 }
 
 template <>

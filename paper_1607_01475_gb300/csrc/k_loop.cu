@@ -28,8 +28,11 @@ __global__ void k_loop_cond(cudaGraphConditionalHandle h, Ctrl* c, int guard_max
 
 // Arm a WHILE node: its condition keeps the value of the loop's last exit
 // (0) when the enclosing body runs again, so a kernel placed just before the
-// node sets it to 1 (the body then runs at least once).
-__global__ void k_cond_arm(cudaGraphConditionalHandle h) { cudaGraphSetConditional(h, 1u); }
+// node sets it to 1 (the body then runs at least once), or to 0 when the run is
+// already done.
+__global__ void k_cond_arm(cudaGraphConditionalHandle h, const Ctrl* run) {
+  cudaGraphSetConditional(h, run != nullptr && run->done ? 0u : 1u);
+}
 
 __global__ void k_ls_cond(cudaGraphConditionalHandle h, Ctrl* c, int max_passes) {
   unsigned v = 0u;
@@ -44,7 +47,20 @@ __global__ void k_copy_if_odd(T* dst, const T* src, const Ctrl* c, size_t n) {
     dst[i] = src[i];
 }
 
-__global__ void k_mixed_check(Ctrl* c3, const Ctrl* c2, Ctrl* c, const Ctrl* tmpl, double tol, int max_iter,
+// A control block that stops nothing and knows no bounds of the fields.
+__device__ void reset_ctrl(Ctrl* c) {
+  Ctrl z;
+  memset(&z, 0, sizeof(z));
+  z.tol = -1.0;
+  z.max_iter = 1 << 30;
+  z.res_linf = -1.0;
+  z.c2 = -1.0;
+  z.umax = -1.0;
+  z.fx_s = kFxOff;
+  *c = z;
+}
+
+__global__ void k_mixed_check(Ctrl* c3, Ctrl* c2, Ctrl* c, const Ctrl* tmpl, double tol, int max_iter,
                               int max_outer, int inner_cap, int order6) {
   if (c3->done) {
     c->done = 1;
@@ -72,6 +88,7 @@ __global__ void k_mixed_check(Ctrl* c3, const Ctrl* c2, Ctrl* c, const Ctrl* tmp
   *c = *tmpl;
   const int left = max_iter - c3->inner_total;
   c->max_iter = left < inner_cap ? left : inner_cap;
+  reset_ctrl(c2);  // for the next outer residual
 }
 
 __global__ void k_mixed_after(Ctrl* c3, const Ctrl* c) {
@@ -84,17 +101,7 @@ __global__ void k_mixed_after(Ctrl* c3, const Ctrl* c) {
   }
 }
 
-__global__ void k_ctrl_reset(Ctrl* c) {
-  Ctrl z;
-  memset(&z, 0, sizeof(z));
-  z.tol = -1.0;
-  z.max_iter = 1 << 30;
-  z.res_linf = -1.0;
-  z.c2 = -1.0;
-  z.umax = -1.0;
-  z.fx_s = kFxOff;
-  *c = z;
-}
+__global__ void k_ctrl_reset(Ctrl* c) { reset_ctrl(c); }
 
 __global__ void k_ctrl_set(Ctrl* c, const Ctrl h) { *c = h; }
 
@@ -106,8 +113,8 @@ cudaError_t launch_loop_cond(cudaGraphConditionalHandle h, Ctrl* c, int guard_ma
   k_loop_cond<<<1, 1, 0, st>>>(h, c, guard_max);
   return cudaGetLastError();
 }
-cudaError_t launch_cond_arm(cudaGraphConditionalHandle h, cudaStream_t st) {
-  k_cond_arm<<<1, 1, 0, st>>>(h);
+cudaError_t launch_cond_arm(cudaGraphConditionalHandle h, const Ctrl* run, cudaStream_t st) {
+  k_cond_arm<<<1, 1, 0, st>>>(h, run);
   return cudaGetLastError();
 }
 cudaError_t launch_ls_cond(cudaGraphConditionalHandle h, Ctrl* c, int max_passes, cudaStream_t st) {
@@ -119,9 +126,8 @@ cudaError_t launch_copy_if_odd(T* dst, const T* src, const Ctrl* c, size_t n, cu
   k_copy_if_odd<T><<<grid1d(n), 256, 0, st>>>(dst, src, c, n);
   return cudaGetLastError();
 }
-template cudaError_t launch_copy_if_odd<float>(float*, const float*, const Ctrl*, size_t, cudaStream_t);
 template cudaError_t launch_copy_if_odd<double>(double*, const double*, const Ctrl*, size_t, cudaStream_t);
-cudaError_t launch_mixed_check(Ctrl* c3, const Ctrl* c2, Ctrl* c, const Ctrl* tmpl, double tol, int max_iter,
+cudaError_t launch_mixed_check(Ctrl* c3, Ctrl* c2, Ctrl* c, const Ctrl* tmpl, double tol, int max_iter,
                                int max_outer, int inner_cap, int order6, cudaStream_t st) {
   k_mixed_check<<<1, 1, 0, st>>>(c3, c2, c, tmpl, tol, max_iter, max_outer, inner_cap, order6);
   return cudaGetLastError();

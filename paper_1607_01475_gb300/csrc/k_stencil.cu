@@ -270,9 +270,10 @@ __global__ void k_round_f32(float* out, const double* in, size_t n) {
     for (size_t i = t0; i < n; i += stride) out[i] = (float)in[i];
   }
 }
-__global__ void k_accumulate_f64(double* u, const float* delta, float* u32, size_t n, const double* dsum,
-                                 const int* skip) {
+__global__ void k_accumulate_f64(double* u, const float* delta_even, const float* delta_odd, const int* iter,
+                                 float* u32, size_t n, const double* dsum, const int* skip) {
   if (skip != nullptr && *skip) return;
+  const float* delta = (*iter & 1) ? delta_odd : delta_even;
   const double m = dsum ? *dsum / (double)n : 0.0;  // mean of delta, removed
   const size_t t0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
   if (aligned16(u) && aligned16(delta) && aligned16(u32) && (n & 1) == 0) {
@@ -292,6 +293,17 @@ __global__ void k_accumulate_f64(double* u, const float* delta, float* u32, size
       u[i] = v;
       u32[i] = (float)v;
     }
+  }
+}
+
+// a = b = c = 0 (the handle's own fields, a multiple of 4 values).
+__global__ void k_zero_f32(float* a, float* b, float* c, size_t n, const int* skip) {
+  if (*skip) return;
+  const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n / 4; i += (size_t)gridDim.x * blockDim.x) {
+    reinterpret_cast<float4*>(a)[i] = z;
+    if (b != nullptr) reinterpret_cast<float4*>(b)[i] = z;
+    if (c != nullptr) reinterpret_cast<float4*>(c)[i] = z;
   }
 }
 
@@ -652,9 +664,13 @@ cudaError_t launch_round_f32(float* out, const double* in, size_t n, cudaStream_
   k_round_f32<<<grid1d(n), 256, 0, st>>>(out, in, n);
   return cudaGetLastError();
 }
-cudaError_t launch_accumulate_f64(double* u, const float* delta, float* u32, size_t n, const double* dsum,
-                                  cudaStream_t st, const int* skip) {
-  k_accumulate_f64<<<grid1d(n), 256, 0, st>>>(u, delta, u32, n, dsum, skip);
+cudaError_t launch_accumulate_f64(double* u, const float* delta, const float* delta_odd, const int* iter, float* u32,
+                                  size_t n, const double* dsum, cudaStream_t st, const int* skip) {
+  k_accumulate_f64<<<grid1d(n / 2), 256, 0, st>>>(u, delta, delta_odd, iter, u32, n, dsum, skip);
+  return cudaGetLastError();
+}
+cudaError_t launch_zero_f32(float* a, float* b, float* c, size_t n, const int* skip, cudaStream_t st) {
+  k_zero_f32<<<grid1d(n / 4), 256, 0, st>>>(a, b, c, n, skip);
   return cudaGetLastError();
 }
 

@@ -39,10 +39,11 @@ cudaError_t launch_dht_cols(T* data, const KParams& kp, int ax, T scale, const i
                             const AxisTables<T>& tb, cudaStream_t st);
 
 // (FP64 passes: block fixed point, see fx_line.cuh; their scale is a power of
-// two.)  The x pass from an FP32 field.  skip (device, may be null): the pass
+// two.)  The x pass from an FP32 field: src where *iter is even, else src_odd.  skip (device, may be null): the pass
 // returns at once when *skip != 0.
-cudaError_t launch_dht_rows_from_f32(const float* src, double* dst, int nx, int nrows, const AxisTables<double>& tb,
-                                     cudaStream_t st, const int* skip = nullptr);
+cudaError_t launch_dht_rows_from_f32(const float* src, const float* src_odd, const int* iter, double* dst, int nx,
+                                     int nrows, const AxisTables<double>& tb, cudaStream_t st,
+                                     const int* skip = nullptr);
 // The last FP64 pass (z in 3D, y in 2D) with a fused epilogue: out32 ==
 // nullptr: theta += DHT(data) / mu, and (dc != null) *dc = the zero-frequency
 // coefficient (the sum of the transformed field); else out32 = (float)(DHT(data)
@@ -102,6 +103,8 @@ struct ResArgs {
   int update_iter; // 1: this call advances the iteration count
   int fixed;       // FP64 plain, p = 4, 2D or 3D column kernel: take the fixed-point variant with the
                    // scales in ctrl (fx_s, fx_g) unless they say not to
+  float* r32;      // FP64 plain: receives r rounded to FP32, twice (null: none; then r may be null)
+  float* r32b;
 };
 
 // r = f - N_h^{loc}[u_in + alpha d] (plain) or
@@ -154,9 +157,10 @@ long long residual_grid_blocks(const KParams& kp, bool fp32);
 // Loop while !c->done and the body count stays below guard_max (the guard
 // trips PSD_ERR_NOCONV).
 cudaError_t launch_loop_cond(cudaGraphConditionalHandle h, Ctrl* c, int guard_max, cudaStream_t st);
-// Set the condition to 1 just before a WHILE node (it keeps the value of the
-// previous exit when an enclosing loop body runs the node again).
-cudaError_t launch_cond_arm(cudaGraphConditionalHandle h, cudaStream_t st);
+// Set the condition just before a WHILE node (it keeps the value of the previous
+// exit when an enclosing loop body runs the node again): 1, or 0 when run (may be
+// null) is done.
+cudaError_t launch_cond_arm(cudaGraphConditionalHandle h, const Ctrl* run, cudaStream_t st);
 // General-p line search: another Newton pass while the bracket has not
 // converged (c->c3 == 0), the run is not done, and fewer than max_passes ran.
 cudaError_t launch_ls_cond(cudaGraphConditionalHandle h, Ctrl* c, int max_passes, cudaStream_t st);
@@ -167,7 +171,7 @@ cudaError_t launch_copy_if_odd(T* dst, const T* src, const Ctrl* c, size_t n, cu
 // decide convergence / failure into c3, and either stop the inner solve
 // (c->done = 1) or initialise it from the template tmpl with max_iter =
 // min(max_iter - inner_total, inner_cap).  cond: the outer WHILE handle.
-cudaError_t launch_mixed_check(Ctrl* c3, const Ctrl* c2, Ctrl* c, const Ctrl* tmpl, double tol, int max_iter,
+cudaError_t launch_mixed_check(Ctrl* c3, Ctrl* c2, Ctrl* c, const Ctrl* tmpl, double tol, int max_iter,
                                int max_outer, int inner_cap, int order6, cudaStream_t st);
 // Mixed solve, after the inner solve: inner_total += c->iter, last alpha,
 // non-finite inner residual -> c3 failed (done).
@@ -203,9 +207,11 @@ cudaError_t launch_norms(const double* x, size_t n, double hd, Ctrl* c, double* 
 cudaError_t launch_mean_project(double* u, const double* g, size_t n, Ctrl* c, double* partials, cudaStream_t st);
 cudaError_t launch_round_f32(float* out, const double* in, size_t n, cudaStream_t st);
 // u += delta - mean(delta) (dsum: device pointer to sum(delta), or null for
-// no mean removal), u32 = (float) u.
-cudaError_t launch_accumulate_f64(double* u, const float* delta, float* u32, size_t n, const double* dsum,
-                                  cudaStream_t st, const int* skip = nullptr);
+// no mean removal), u32 = (float) u; delta where *iter is even, else delta_odd.
+cudaError_t launch_accumulate_f64(double* u, const float* delta, const float* delta_odd, const int* iter, float* u32,
+                                  size_t n, const double* dsum, cudaStream_t st, const int* skip = nullptr);
+// a = b = c = 0 (n values each, b and c may be null) unless *skip != 0.
+cudaError_t launch_zero_f32(float* a, float* b, float* c, size_t n, const int* skip, cudaStream_t st);
 
 void init_dht_attributes();
 

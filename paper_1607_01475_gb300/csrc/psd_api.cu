@@ -398,16 +398,16 @@ psd_status full_dht(psd_context* c, T* x, T scale, const AxisTables<T>& tb) {
 }
 
 // theta += DHT(v) / mu (order 6, mixed): v is src64 (FP64, transformed in
-// place) or src32 (FP32, transformed into D); theta lives in Z.  skip
-// (device, may be null): the passes return at once when *skip != 0.
-psd_status dht_theta(psd_context* c, const double* src64, const float* src32, double* dc = nullptr,
-                        const int* skip = nullptr) {
+// place), or (null) the inner solve's correction delta, in da or db by the parity
+// of its iterations (transformed into D); theta lives in Z.  skip (device, may be
+// null): the passes return at once when *skip != 0.
+psd_status dht_theta(psd_context* c, const double* src64, double* dc = nullptr, const int* skip = nullptr) {
   const KParams& kp = c->kp;
   const int nrows = kp.ny * kp.nz;
   double* x = c->D;
-  if (src32) {
+  if (!src64) {
     ProfScope p_(c, PSD_PROF_DHT_ROWS_FF);
-    CK(psd::launch_dht_rows_from_f32(src32, x, kp.nx, nrows, c->tb64, c->st, skip));
+    CK(psd::launch_dht_rows_from_f32(c->da, c->db, &c->ctrl->iter, x, kp.nx, nrows, c->tb64, c->st, skip));
   } else {
     ProfScope p_(c, PSD_PROF_DHT_ROWS_FF);
     CK(psd::launch_dht_rows<double>(src64, x, kp.nx, nrows, 1.0, skip, c->tb64, c->st));
@@ -449,10 +449,11 @@ psd_status cap_stream(psd_context* c, int d, cudaStream_t* out) {
 // Insert a WHILE conditional node at the current position of the capture on
 // c->st and capture its body: body(handle) enqueues on c->st (a stream of the
 // next depth) and must end with a kernel that sets the condition.  A kernel
-// just before the node sets the condition to 1, so the body runs at least
-// once every time the node is reached.
+// just before the node sets the condition to 1, or to 0 when the run `run` (may be
+// null) is already done: then the body, whose kernels would all return at once, is
+// not entered.
 template <typename Body>
-psd_status capture_while(psd_context* c, Body&& body) {
+psd_status capture_while(psd_context* c, const Ctrl* run, Body&& body) {
   cudaStream_t s = c->st, s2 = nullptr;
   TRY(cap_stream(c, c->cap_depth + 1, &s2));
   cudaStreamCaptureStatus cs;
@@ -465,7 +466,7 @@ psd_status capture_while(psd_context* c, Body&& body) {
   CK(cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault));
   // a node nested in another loop's body is reached again with the value of
   // its last exit: arm it first
-  CK(psd::launch_cond_arm(h, s));
+  CK(psd::launch_cond_arm(h, run, s));
   CK(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, &deps, nullptr, &nd));
   cudaGraphNodeParams cp = {};
   cp.type = cudaGraphNodeTypeConditional;
@@ -527,7 +528,7 @@ psd_status linesearch(psd_context* c, const T* u, const T* ubase, const T* D, Ct
     return PSD_OK;
   }
   if (c->capturing) {
-    return capture_while(c, [&](cudaGraphConditionalHandle h) -> psd_status {
+    return capture_while(c, ctrl, [&](cudaGraphConditionalHandle h) -> psd_status {
       CK(psd::launch_linesearch<T>(u, ubase, D, c->pk, c->kp, ctrl, c->partials, c->st));
       CK(psd::launch_ls_cond(h, ctrl, kLsPassesGen, c->st));
       return PSD_OK;
@@ -579,13 +580,11 @@ psd_status fx_scan(psd_context* c, const double* u, const float* u32, Ctrl* ctrl
 
 // FP64 residual r = f - N_h[u] into r (order 6: P0[...] including T_h[u - g]),
 // norms into ctrl2 (res_l2, res_linf), all enqueued (ctrl2 reset on device).
-// u32: the FP32 copy of u where there is one (its scan reads half the bytes).
 // Uses W, Z as scratch (order 6).
-psd_status residual64(psd_context* c, const double* u, const double* f, const double* g, double* r,
-                      const float* u32 = nullptr) {
+psd_status residual64(psd_context* c, const double* u, const double* f, const double* g, double* r) {
   const KParams& kp = c->kp;
   CK(psd::launch_ctrl_reset(c->ctrl2, c->st));
-  TRY(fx_scan(c, u, u32, c->ctrl2));
+  TRY(fx_scan(c, u, nullptr, c->ctrl2));
   ResArgs<double> a{u, nullptr, nullptr, f, nullptr, r, kp.order == 4 ? 1 : 0, 0, 1};
   { ProfScope p_(c, PSD_PROF_RESIDUAL_FP64); CK(psd::launch_residual<double>(a, psd::RM_PLAIN, c->pk, kp, c->ctrl2, c->partials, c->st)); }
   if (kp.order == 6) {
@@ -600,14 +599,24 @@ psd_status residual64(psd_context* c, const double* u, const double* f, const do
   return PSD_OK;
 }
 
+// Fourth-order outer residual (mixed precision): f - N_h[u] rounded to FP32 into
+// R32, and into W32, which is the inner solve's first residual (delta = 0); norms
+// into ctrl2, which the caller has reset (enqueued).  The scan reads the FP32 copy of u.
+psd_status outer_residual4(psd_context* c, const double* u, const double* f) {
+  TRY(fx_scan(c, u, c->u32, c->ctrl2));
+  ResArgs<double> a{u, nullptr, nullptr, f, nullptr, nullptr, 1, 0, 1, c->R32, c->W32};
+  ProfScope p_(c, PSD_PROF_RESIDUAL_FP64);
+  CK(psd::launch_residual<double>(a, psd::RM_PLAIN, c->pk, c->kp, c->ctrl2, c->partials, c->st));
+  return PSD_OK;
+}
+
 // Sixth-order outer residual in the transform domain (mixed precision):
 // R32 <- (float) DHT(P0[f - N_h^{loc}[u]] - T_h[u - g]) = DHT(r_loc) - theta
 // with theta = DHT(T_h[u - g]) in Z (the subtraction, the rounding and the
 // Parseval norm fused into the last transform pass); ||R||_2 into
-// ctrl2->res_l2 (enqueued).
+// ctrl2->res_l2 (enqueued; the caller has reset ctrl2).
 psd_status outer_residual6_spec(psd_context* c, const double* u, const double* f) {
   const KParams& kp = c->kp;
-  CK(psd::launch_ctrl_reset(c->ctrl2, c->st));
   TRY(fx_scan(c, u, c->u32, c->ctrl2));
   ResArgs<double> a{u, nullptr, nullptr, f, nullptr, c->W, 0, 0, 1};
   { ProfScope p_(c, PSD_PROF_RESIDUAL_FP64); CK(psd::launch_residual<double>(a, psd::RM_PLAIN, c->pk, kp, c->ctrl2, c->partials, c->st)); }
@@ -657,7 +666,7 @@ psd_status fp64_iterations(psd_context* c, const double* f, double* u, int count
 psd_status fp64_graph_body(psd_context* c, const double* f, const double* g, double* u) {
   TRY(fp64_start(c, f, g, u));
   const int guard = c->prm.max_iter / kBody + 3;
-  TRY(capture_while(c, [&](cudaGraphConditionalHandle h) -> psd_status {
+  TRY(capture_while(c, c->ctrl, [&](cudaGraphConditionalHandle h) -> psd_status {
     TRY(fp64_iterations(c, f, u, kBody));
     CK(psd::launch_loop_cond(h, c->ctrl, guard, c->st));
     return PSD_OK;
@@ -775,17 +784,14 @@ psd_status inner_iterations(psd_context* c, int count) {
   return PSD_OK;
 }
 
-// The start of an inner solve: delta = 0, the direction spectrum 0 (order
-// 6), and the inner residual at delta = 0.
+// The start of an inner solve (skipped once c->ctrl is done): delta = 0 and, order
+// 6, the direction spectrum 0.  At delta = 0 the inner residual is the outer one: order 4
+// has it in W32, and order 6, whose outer residual enters in the middle pass as the
+// initial xi (R32 holds its spectrum and is advanced in place), starts from W32 = 0.
 psd_status inner_start(psd_context* c) {
-  const KParams& kp = c->kp;
-  const bool six = kp.order == 6;
-  CK(cudaMemsetAsync(c->da, 0, c->N * sizeof(float), c->st));
-  if (six) CK(cudaMemsetAsync(c->Dsp32, 0, c->N * sizeof(float), c->st));
-  // order 6: the outer residual enters in the middle pass as the initial xi
-  // (R32 holds its spectrum and is advanced in place by the inner solve)
-  ResArgs<float> a{c->da, nullptr, nullptr, six ? nullptr : c->R32, c->u32, c->W32, six ? 0 : 1, 0};
-  { ProfScope p_(c, PSD_PROF_RESIDUAL_FP32); CK(psd::launch_residual<float>(a, psd::RM_INNER, c->pk, kp, c->ctrl, c->partials, c->st)); }
+  const bool six = c->kp.order == 6;
+  ProfScope p_(c, PSD_PROF_OTHER);
+  CK(psd::launch_zero_f32(c->da, six ? c->Dsp32 : nullptr, six ? c->W32 : nullptr, c->N, &c->ctrl->done, c->st));
   return PSD_OK;
 }
 
@@ -810,7 +816,7 @@ psd_status mixed_project_mean(psd_context* c, const double* g, double* u) {
   return PSD_OK;
 }
 
-// The device part of the mixed solve's start: u32 = fl32(u); order 6:
+// The device part of the mixed solve's start: u32 = fl32(u), ctrl2 reset; order 6:
 // theta = DHT(T_h[u0 - g]) (advanced with DHT(T_h delta) after every
 // correction).
 psd_status mixed_start(psd_context* c, const double* g, double* u) {
@@ -818,8 +824,9 @@ psd_status mixed_start(psd_context* c, const double* g, double* u) {
   if (c->kp.order == 6) {
     CK(cudaMemsetAsync(c->Z, 0, c->N * sizeof(double), c->st));
     { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_axpby<double>(c->D, u, g, 1.0, -1.0, 0.0, c->N, c->st)); }
-    TRY(dht_theta(c, c->D, nullptr));
+    TRY(dht_theta(c, c->D));
   }
+  CK(psd::launch_ctrl_reset(c->ctrl2, c->st));
   return PSD_OK;
 }
 
@@ -833,29 +840,27 @@ psd_status mixed_graph_body(psd_context* c, const double* f, const double* g, do
   const int guard_outer = std::max(c->prm.max_outer, 1) + 3;
   const int inner_cap = std::min(std::max(c->prm.max_iter, 1), kInnerMaxIter);
   const int guard_inner = inner_cap / kBody + 3;
-  return capture_while(c, [&](cudaGraphConditionalHandle ho) -> psd_status {
+  return capture_while(c, nullptr, [&](cudaGraphConditionalHandle ho) -> psd_status {
     if (six) {
       TRY(outer_residual6_spec(c, u, f));
     } else {
-      TRY(residual64(c, u, f, g, c->W, c->u32));
-      { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_round_f32(c->R32, c->W, c->N, c->st)); }
+      TRY(outer_residual4(c, u, f));
     }
     CK(psd::launch_mixed_check(c->ctrl3, c->ctrl2, c->ctrl, c->ctrl_tmpl, c->prm.tol, c->prm.max_iter,
                                c->prm.max_outer, kInnerMaxIter, six ? 1 : 0, c->st));
     TRY(inner_start(c));
-    TRY(capture_while(c, [&](cudaGraphConditionalHandle hi) -> psd_status {
+    TRY(capture_while(c, c->ctrl, [&](cudaGraphConditionalHandle hi) -> psd_status {
       TRY(inner_iterations(c, kBody));
       CK(psd::launch_loop_cond(hi, c->ctrl, guard_inner, c->st));
       return PSD_OK;
     }));
-    CK(psd::launch_copy_if_odd<float>(c->da, c->db, c->ctrl, c->N, c->st));
     CK(psd::launch_mixed_after(c->ctrl3, c->ctrl, c->st));
     // order 6: theta += DHT(T_h delta) with sum(delta) recorded; u += delta
     // (mean removed for order 6), u32 = fl32(u) -- skipped once the outer
     // loop is done
     double* dsum = six ? &c->ctrl2->c3 : nullptr;
-    if (six) TRY(dht_theta(c, nullptr, c->da, dsum, &c->ctrl3->done));
-    { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_accumulate_f64(u, c->da, c->u32, c->N, dsum, c->st, &c->ctrl3->done)); }
+    if (six) TRY(dht_theta(c, nullptr, dsum, &c->ctrl3->done));
+    { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_accumulate_f64(u, c->da, c->db, &c->ctrl->iter, c->u32, c->N, dsum, c->st, &c->ctrl3->done)); }
     CK(psd::launch_loop_cond(ho, c->ctrl3, guard_outer, c->st));
     (void)inner_cap;
     return PSD_OK;
@@ -904,22 +909,22 @@ psd_status solve_mixed(psd_context* c, const double* f, const double* g, double*
       // removes the mean of delta, which is zero only up to FP32 rounding,
       // so that mean(u) = mean(g) holds throughout
       double* dsum = six ? &c->ctrl2->c3 : nullptr;
-      if (six) TRY(dht_theta(c, nullptr, c->da, dsum));
-      { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_accumulate_f64(u, c->da, c->u32, c->N, dsum, c->st)); }
+      if (six) TRY(dht_theta(c, nullptr, dsum));
+      { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_accumulate_f64(u, c->da, c->db, &c->ctrl->iter, c->u32, c->N, dsum, c->st)); }
     }
     if (six) {
       // the outer residual stays in the transform domain; the inner solve adds
       // it to its own transformed residual in the middle pass
       TRY(outer_residual6_spec(c, u, f));
     } else {
-      TRY(residual64(c, u, f, g, c->W, c->u32));
+      TRY(outer_residual4(c, u, f));
     }
     Ctrl h2;
     TRY(read_ctrl(c, c->ctrl2, h2));
+    CK(psd::launch_ctrl_reset(c->ctrl2, c->st));  // for the next outer residual
     res = h2.res_l2;
     resinf = six ? -1.0 : h2.res_linf;
     ++outer;
-    if (!six) { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_round_f32(c->R32, c->W, c->N, c->st)); }
     if (!std::isfinite(res)) {
       status = PSD_ERR_NONFINITE;
       break;
@@ -951,7 +956,6 @@ psd_status solve_mixed(psd_context* c, const double* f, const double* g, double*
       status = PSD_ERR_NONFINITE;
       break;
     }
-    if (hc.iter % 2 == 1) CK(cudaMemcpyAsync(c->da, c->db, c->N * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
     have_delta = hc.iter > 0;
   }
   CK(cudaEventRecord(c->ev1, c->st));

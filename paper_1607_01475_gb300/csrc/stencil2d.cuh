@@ -235,7 +235,11 @@ __device__ __forceinline__ void res2d_march(const ResArgs<T>& a, const KParams& 
             accm = fmax(accm, fabs(r[v]));
           }
         }
-        if (out) store_row(a.r + (size_t)(k - 2) * nx + gx, r);
+        if constexpr (V == 1) {
+          if (out) store_r<MODE>(a, (size_t)(k - 2) * nx + gx, r[0]);
+        } else {
+          if (out) store_row(a.r + (size_t)(k - 2) * nx + gx, r);
+        }
       }
     }
 #pragma unroll

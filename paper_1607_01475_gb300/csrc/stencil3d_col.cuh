@@ -393,7 +393,7 @@ __device__ __forceinline__ void res3d_col(const ResArgs<T>& a, const KParams& kp
         r = (cu * uc + cbih * bih) - cdiv * div;
       else
         r = (fcur - cuq * uc) + (cdivq * div - cbihq * bih);
-      a.r[(size_t)(z & (nz - 1)) * plane + gown] = r;
+      store_r<MODE>(a, (size_t)(z & (nz - 1)) * plane + gown, r);
       acc2 += HVP ? uc * r : r * r;
       accm = fmax(accm, fabs(r));
       Lm = L0;

@@ -107,6 +107,20 @@ __device__ __forceinline__ void flux_lin(const T (&a)[3], const T (&e)[3], T bet
   }
 }
 
+// Store a residual value (FP64 plain: or, for the mixed solver, its FP32 rounding
+// twice).
+template <int MODE, typename T>
+__device__ __forceinline__ void store_r(const ResArgs<T>& a, size_t i, T r) {
+  if constexpr (sizeof(T) == 8 && MODE == RM_PLAIN) {
+    if (a.r32 != nullptr) {
+      a.r32[i] = (float)r;
+      a.r32b[i] = (float)r;
+      return;
+    }
+  }
+  a.r[i] = r;
+}
+
 // Last-block bookkeeping of the residual kernel.
 __device__ void residual_epilogue(Ctrl* ctrl, const KParams& kp, double sum2, double maxabs, int norm,
                                   int update_iter, bool hvp = false) {
@@ -279,7 +293,7 @@ __global__ void __launch_bounds__(NT)
         r = (cu * uc + se2 * bih) - s * div;
       else
         r = (a.f ? a.f[g] : T(0)) - cu * uc + s * div - se2 * bih;
-      a.r[g] = r;
+      store_r<MODE>(a, g, r);
       acc2 += (MODE == RM_HVP) ? uc * r : r * r;
       accm = fmax(accm, fabs(r));
     }
