@@ -372,11 +372,14 @@ __global__ void __launch_bounds__(kFxThreads, 3)
 }
 
 // ------------------------------------------------------------- middle pass
-// FP64 form of k_mid (dht_kernels.cuh): one tile of 2 * pairs x-columns at
-// one outer index per CTA, lines along the last axis.  The symbol division
-// and the Parseval sums are FP64; both transforms are fixed point, each with
-// its own line exponents.
-template <int N, int RM, int ORDER>
+// FP64 form of k_mid (dht_kernels.cuh), lines along the last axis.  The symbol
+// division and the Parseval sums are FP64; both transforms are fixed point, each with
+// its own line exponents.  MIRROR (3D): the two lines of a thread's pair mirror each
+// other in y (y and ny - y; lines 0 and ny / 2, which mirror themselves, make one
+// pair), so that mu and the reciprocal of the symbol are formed once for two modes:
+// the FP64 pipe, with 10 (order 4) and 15 (order 6) operations a mode at 1.74 per
+// clock and SM, was 50 to 80% of the pass.  Otherwise they are x and x + 1.
+template <int N, int RM, int ORDER, bool MIRROR>
 __global__ void __launch_bounds__(kFxThreads, 2)
     k_mid_fx(double* data, unsigned line_stride, unsigned outer_stride, int ntx, KParams kp, Ctrl* ctrl,
              double* partials, double* xi_, double* dspec, const double* __restrict__ symx,
@@ -398,21 +401,35 @@ __global__ void __launch_bounds__(kFxThreads, 2)
   // order 6: xi and dspec of the tile, copied while the transform runs
   double2* pre_x = reinterpret_cast<double2*>(smem_raw + (size_t)pairs * 2 * LS * sizeof(fx));
   double2* pre_d = pre_x + (size_t)N * pairs;
-  const int xb = (int)blockIdx.x % ntx, yo = (int)blockIdx.x / ntx;
-  const int x = xb * 2 * pairs + 2 * p;
-  const unsigned base = (unsigned)yo * outer_stride + (unsigned)x;  // every grid has fewer than 2^32 cells
+  const int x = ((int)blockIdx.x % ntx * pairs + p) * (MIRROR ? 1 : 2), yo = (int)blockIdx.x / ntx;
+  const int y1 = !MIRROR ? yo : (yo == 0 ? kp.ny >> 1 : kp.ny - yo);  // of the second line
+  const bool self = !MIRROR || yo == 0;                               // each line has its own mu
+  const unsigned base0 = (unsigned)yo * outer_stride + (unsigned)x;   // every grid has fewer than 2^32 cells
+  const unsigned base1 = (unsigned)y1 * outer_stride + (unsigned)x;   // MIRROR
   double xr[R], xi[R];
 #pragma unroll
   for (int q = 0; q < R; ++q) {
-    const unsigned idx = base + (unsigned)(j + q * TS) * line_stride;
-    const double2 v = *reinterpret_cast<const double2*>(data + idx);
+    const unsigned off = (unsigned)(j + q * TS) * line_stride;
     if (ORDER == 6) {
       const unsigned e = (unsigned)(q * TS + j) * pairs + p;
-      cp_async_16(pre_x + e, xi_ + idx);
-      cp_async_16(pre_d + e, dspec + idx);
+      if (MIRROR) {
+        cp_async_8(&pre_x[e].x, xi_ + base0 + off);
+        cp_async_8(&pre_x[e].y, xi_ + base1 + off);
+        cp_async_8(&pre_d[e].x, dspec + base0 + off);
+        cp_async_8(&pre_d[e].y, dspec + base1 + off);
+      } else {
+        cp_async_16(pre_x + e, xi_ + base0 + off);
+        cp_async_16(pre_d + e, dspec + base0 + off);
+      }
     }
-    xr[q] = v.x;
-    xi[q] = v.y;
+    if (MIRROR) {
+      xr[q] = data[base0 + off];
+      xi[q] = data[base1 + off];
+    } else {
+      const double2 v = *reinterpret_cast<const double2*>(data + base0 + off);
+      xr[q] = v.x;
+      xi[q] = v.y;
+    }
   }
   FxLine ln = fx_cols_transform<N, RM>(xr, xi, p, j, pairs, sr, si, scr, tab);
   if (ORDER == 6) cp_async_wait_all();
@@ -420,21 +437,32 @@ __global__ void __launch_bounds__(kFxThreads, 2)
   const double s = C.s, se2 = C.se2, sl = C.sl;
   const double alpha_prev = ORDER == 6 ? ctrl->alpha : 0.0;
   const double mo = symo != nullptr ? symo[yo] : 0.0;
-  const double mxa = symx[x] + mo, mxb = symx[x + 1] + mo;
+  const double mxa = symx[x] + mo, mxb = MIRROR ? symx[x] + symo[y1] : symx[x + 1] + mo;
   double acc[mid_nsums<double, ORDER>()] = {};
+  auto put = [&](double* f, unsigned off, double a, double b) {
+    if (MIRROR) {
+      f[base0 + off] = a;
+      f[base1 + off] = b;
+    } else {
+      *reinterpret_cast<double2*>(f + base0 + off) = make_double2(a, b);
+    }
+  };
 #pragma unroll
   for (int q = 0; q < R; ++q) {
     const int kk = j + q * TS;
     fx w[2];
     dht_split(sr, si, kk, N, w[0], w[1]);
     const double ml = syml[kk];
-    double dv[2];
+    double mu = 0.0, ip = 0.0, dv[2];
     if (ORDER == 4) {
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const double h = fx_leave<N, RM>(w[c], ln, 0);
-        const double mu = (c ? mxb : mxa) + ml;
-        const double d = h * recip_pos(fma(mu, fma(se2, mu, s), 1.0));
+        if (c == 0 || self) {
+          mu = (c ? mxb : mxa) + ml;
+          ip = recip_pos(fma(mu, fma(se2, mu, s), 1.0));
+        }
+        const double d = h * ip;
         const double m = mu * d;
         dv[c] = d;
         acc[0] = fma(h, d, acc[0]);
@@ -444,19 +472,33 @@ __global__ void __launch_bounds__(kFxThreads, 2)
       // xi advances with the previous step and is added to the transformed
       // local residual; d = mu rt / P and T_h d = rt / P, P = 1 + mu (lam s +
       // mu (s + s eps^2 mu)) (see k_mid)
-      const unsigned idx = base + (unsigned)kk * line_stride, e = (unsigned)(q * TS + j) * pairs + p;
+      const unsigned off = (unsigned)kk * line_stride, e = (unsigned)(q * TS + j) * pairs + p;
       const double2 xv = pre_x[e], dp = pre_d[e];
       const double xs[2] = {xv.x, xv.y}, ds[2] = {dp.x, dp.y};
       double xn[2], tn[2];
+      double mus[2], ips[2];
+      if (MIRROR) {  // both before the conversions: 187 us for a solve of L_h at 128^3, else 191
+        mus[0] = mxa + ml;
+        mus[1] = self ? mxb + ml : mus[0];
+        ips[0] = recip_pos(fma(mus[0], fma(mus[0], fma(se2, mus[0], s), sl), 1.0));
+        ips[1] = ips[0];
+        if (self) ips[1] = recip_pos(fma(mus[1], fma(mus[1], fma(se2, mus[1], s), sl), 1.0));
+      }
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const double h = fx_leave<N, RM>(w[c], ln, 0);
-        const double mu = (c ? mxb : mxa) + ml;
         double rt = 0.0, d = 0.0, xc = 0.0, td = 0.0;
-        if (!(x + c == 0 && yo == 0 && kk == 0)) {  // mu > 0: every mode but the zero one
+        if (MIRROR) {
+          mu = mus[c];
+          ip = ips[c];
+        } else {
+          mu = (c ? mxb : mxa) + ml;
+          ip = recip_pos(fma(mu, fma(mu, fma(se2, mu, s), sl), 1.0));
+        }
+        if (!(c == 0 && yo == 0 && x == 0 && kk == 0)) {  // mu > 0: every mode but the zero one
           xc = fma(-alpha_prev, ds[c], xs[c]);
           rt = h + xc;
-          td = rt * recip_pos(fma(mu, fma(mu, fma(se2, mu, s), sl), 1.0));
+          td = rt * ip;
           d = mu * td;
         }
         const double m = mu * d;
@@ -467,8 +509,8 @@ __global__ void __launch_bounds__(kFxThreads, 2)
         acc[1] = fma(m, d, acc[1]);
         acc[mid_nsums<double, ORDER>() - 1] = fma(rt, rt, acc[mid_nsums<double, ORDER>() - 1]);
       }
-      *reinterpret_cast<double2*>(xi_ + idx) = make_double2(xn[0], xn[1]);
-      *reinterpret_cast<double2*>(dspec + idx) = make_double2(tn[0], tn[1]);
+      put(xi_, off, xn[0], xn[1]);
+      put(dspec, off, tn[0], tn[1]);
     }
     xr[q] = dv[0];
     xi[q] = dv[1];
@@ -481,8 +523,7 @@ __global__ void __launch_bounds__(kFxThreads, 2)
     const int kk = j + q * TS;
     fx h1, h2;
     dht_split(sr, si, kk, N, h1, h2);
-    *reinterpret_cast<double2*>(data + (base + (unsigned)kk * line_stride)) =
-        make_double2(fx_leave<N, RM>(h1, ln, scale_e), fx_leave<N, RM>(h2, ln, scale_e));
+    put(data, (unsigned)kk * line_stride, fx_leave_hw<N, RM>(h1, ln, scale_e), fx_leave_hw<N, RM>(h2, ln, scale_e));
   }
   mid_finish<double, ORDER>(acc, sred, partials, ctrl, kp, &sflag);
 }
@@ -552,26 +593,39 @@ inline LastAxis last_axis(const KParams& kp) {
   return {(size_t)kp.nx * kp.ny, (size_t)kp.nx, kp.ny, 2};
 }
 
-template <int N, int RM>
-cudaError_t mid_fx_impl(double* data, const KParams& kp, Ctrl* ctrl, double* partials, double* xi, double* dspec,
-                        const AxisTables<double>& tb, cudaStream_t st) {
+template <int N, int RM, bool MIRROR>
+cudaError_t mid_fx_launch(double* data, const KParams& kp, Ctrl* ctrl, double* partials, double* xi, double* dspec,
+                          const AxisTables<double>& tb, cudaStream_t st) {
   constexpr int TS = LineFFT<fx, N, RM>::TS;
   const LastAxis a = last_axis(kp);
   int se;
   if (!fx_scale_exp(kp.inv_ntot, &se)) return cudaErrorInvalidValue;
-  const int pairs = fx_pairs<N, RM, false>((long long)(kp.nx / 2) * a.nouter, kp.nx / 2, tb.nsm);
-  const int ntx = kp.nx / (2 * pairs);
+  const int cols = MIRROR ? kp.nx : kp.nx / 2, nout = MIRROR ? kp.ny / 2 : a.nouter;
+  const int pairs = fx_pairs<N, RM, false>((long long)cols * nout, cols, tb.nsm);
+  const int ntx = cols / pairs;
   const double* symo = kp.dim == 2 ? nullptr : tb.sym[1];
   const size_t sm = pairs * fx_pair_smem<N, RM, false>() + (kp.order == 6 ? 2 : 0) * (size_t)N * pairs * sizeof(double2);
   if (kp.order == 4)
-    k_mid_fx<N, RM, 4><<<ntx * a.nouter, pairs * TS, sm, st>>>(data, (unsigned)a.line_stride, (unsigned)a.outer_stride, ntx,
-                                                          kp, ctrl, partials, xi, dspec, tb.sym[0], symo, tb.sym[a.ax],
-                                                          tb.fxtw[a.ax], se);
+    k_mid_fx<N, RM, 4, MIRROR><<<ntx * nout, pairs * TS, sm, st>>>(
+        data, (unsigned)a.line_stride, (unsigned)a.outer_stride, ntx, kp, ctrl, partials, xi, dspec, tb.sym[0], symo,
+         tb.sym[a.ax], tb.fxtw[a.ax], se);
   else
-    k_mid_fx<N, RM, 6><<<ntx * a.nouter, pairs * TS, sm, st>>>(data, (unsigned)a.line_stride, (unsigned)a.outer_stride, ntx,
-                                                          kp, ctrl, partials, xi, dspec, tb.sym[0], symo, tb.sym[a.ax],
-                                                          tb.fxtw[a.ax], se);
+    k_mid_fx<N, RM, 6, MIRROR><<<ntx * nout, pairs * TS, sm, st>>>(
+        data, (unsigned)a.line_stride, (unsigned)a.outer_stride, ntx, kp, ctrl, partials, xi, dspec, tb.sym[0], symo,
+         tb.sym[a.ax], tb.fxtw[a.ax], se);
   return cudaGetLastError();
+}
+// Mirrored pairs of lines where a block reads whole 32-byte sectors of a row (four
+// columns; shorter blocks are those of 1024-point lines and of the smallest grids).
+// Solve of L_h at 256x128x64, order 4: 150 -> 137 us; middle pass of order 6 at 256^3: 627 -> 599 us.
+// In 2D, where x is the axis to mirror, it loses: the rows' sectors are split between
+// blocks (1024^2, order 6, whole solve of L_h: 107 us adjacent, 127 us mirrored).
+template <int N, int RM>
+cudaError_t mid_fx_impl(double* data, const KParams& kp, Ctrl* ctrl, double* partials, double* xi, double* dspec,
+                        const AxisTables<double>& tb, cudaStream_t st) {
+  if (kp.dim == 3 && fx_pairs<N, RM, false>((long long)kp.nx * (kp.ny / 2), kp.nx, tb.nsm) >= 4)
+    return mid_fx_launch<N, RM, true>(data, kp, ctrl, partials, xi, dspec, tb, st);
+  return mid_fx_launch<N, RM, false>(data, kp, ctrl, partials, xi, dspec, tb, st);
 }
 
 template <int N, int RM>

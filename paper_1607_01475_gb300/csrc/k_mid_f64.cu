@@ -28,8 +28,10 @@ void set_attrs_mid_fx() {
   constexpr size_t np = kFxThreads / LineFFT<fx, N, RM>::TS;
   constexpr int line = (int)(np * fx_pair_smem<N, RM, false>()), stage = (int)(np * N * sizeof(double2));
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaFuncSetAttribute(k_mid_fx<N, RM, 4>, attr, line);
-  cudaFuncSetAttribute(k_mid_fx<N, RM, 6>, attr, line + 2 * stage);
+  cudaFuncSetAttribute(k_mid_fx<N, RM, 4, true>, attr, line);
+  cudaFuncSetAttribute(k_mid_fx<N, RM, 6, true>, attr, line + 2 * stage);
+  cudaFuncSetAttribute(k_mid_fx<N, RM, 4, false>, attr, line);
+  cudaFuncSetAttribute(k_mid_fx<N, RM, 6, false>, attr, line + 2 * stage);
   cudaFuncSetAttribute(k_last_fx<N, RM, EPI_THETA>, attr, line + stage);
   cudaFuncSetAttribute(k_last_fx<N, RM, EPI_RESID>, attr, line + stage);
 }
