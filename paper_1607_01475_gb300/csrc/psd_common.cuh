@@ -211,6 +211,14 @@ __device__ __forceinline__ double fx_sqrt_above(unsigned hi) {
 
 // ------------------------------------------------------------------ reductions
 
+// fmax(m, |x|) for m >= 0 (a NaN leaves m).  FP64 as integers: the bits of
+// non-negative values are ordered, and an FP64 comparison takes the slot of an addition.
+__device__ __forceinline__ float max_abs(float m, float x) { return fmaxf(m, fabsf(x)); }
+__device__ __forceinline__ double max_abs(double m, double x) {
+  const long long b = __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFLL;
+  return b > __double_as_longlong(m) && b <= 0x7FF0000000000000LL ? __longlong_as_double(b) : m;
+}
+
 // Block maxima of two values, for every thread (one-dimensional blocks of
 // whole warps); sh: two words of shared memory.
 __device__ __forceinline__ void block_max2(unsigned& a, unsigned& b, unsigned* sh) {

@@ -229,10 +229,11 @@ __device__ __forceinline__ void res2d_march(const ResArgs<T>& a, const KParams& 
           else if (HVP)
             r[v] = (cu * uc + cbih * bih) - cdiv * div;
           else
-            r[v] = (fc[v] - cuq * uc) + (cdivq * div - cbihq * bih);
+            r[v] = FX ? fma(cdivq, div, fma(-cbihq, bih, fma(-cuq, uc, fc[v])))
+                      : (fc[v] - cuq * uc) + (cdivq * div - cbihq * bih);
           if (out) {
             acc2 += HVP ? uc * r[v] : r[v] * r[v];
-            accm = fmax(accm, fabs(r[v]));
+            accm = max_abs(accm, r[v]);
           }
         }
         if constexpr (V == 1) {

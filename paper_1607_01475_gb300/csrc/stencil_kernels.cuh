@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(NT)
         r = (a.f ? a.f[g] : T(0)) - cu * uc + s * div - se2 * bih;
       store_r<MODE>(a, g, r);
       acc2 += (MODE == RM_HVP) ? uc * r : r * r;
-      accm = fmax(accm, fabs(r));
+      accm = max_abs(accm, r);
     }
   };
 

@@ -39,6 +39,14 @@ def test_precond_every_length(oracle, shape, order):
     assert np.max(np.abs(d.cpu().numpy() - ref)) <= 1e-12 * np.max(np.abs(ref))
 
 
+# Middle passes on mirrored pairs of lines with several outer pairs per block row,
+# at radix 4 and 8 and at 512-point lines of four columns per block.
+@pytest.mark.parametrize("shape", [(512, 64, 32), (256, 32, 64), (16, 256, 256), (64, 8, 8)])
+@pytest.mark.parametrize("order", [4, 6])
+def test_precond_mirrored_lines(oracle, shape, order):
+    test_precond_every_length(oracle, shape, order)
+
+
 def test_precond_zero_scaled_and_nonfinite_lines():
     shape = (16, 32, 64)
     S = Solver(4, shape, 0.1, 4.0, 0.05, 0.1)
