@@ -1,4 +1,6 @@
-// Double-word ("float-float") arithmetic: a value is the unevaluated sum
+// Conversions between FP64, 64-bit integers and their bits, and double-word
+// ("float-float") arithmetic, which no kernel uses any more (the transforms are block
+// fixed point, fx_line.cuh); its host check stays.  A double-word value is the unevaluated sum
 // hi + lo of two FP32 numbers with |lo| <= ulp(hi)/2, about 48 significant
 // bits.  On GB300 the FP32 pipes issue 64 times as many operations per
 // clock as the FP64 pipe, so a transform done in float-float costs a small

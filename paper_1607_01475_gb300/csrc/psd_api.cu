@@ -216,46 +216,47 @@ psd_status validate(const psd_params* p, std::string& why) {
 psd_status build_tables(psd_context* c) {
   const int dim = c->prm.dim;
   int n[3] = {c->prm.n[0], c->prm.n[1], dim == 3 ? c->prm.n[2] : 1};
-  size_t tot = 0;
-  for (int a = 0; a < 3; ++a) tot += 3 * (size_t)n[a];
-  std::vector<double> h64(tot);
-  std::vector<float> h32(tot);
-  size_t off = 0;
+  const size_t nfx = (size_t)n[0] + n[1] + n[2], tot = 3 * nfx;
+  // one image of all tables: Q62 twiddles of the fixed-point transforms (16-byte
+  // entries first), then cosines, sines and symbols in FP64 and in FP32
+  const size_t bytes = nfx * sizeof(psd::fx_tw) + tot * (sizeof(double) + sizeof(float));
+  std::vector<psd::fx_tw> image((bytes + sizeof(psd::fx_tw) - 1) / sizeof(psd::fx_tw));
+  psd::fx_tw* hfx = image.data();
+  double* h64 = (double*)(hfx + nfx);
+  float* h32 = (float*)(h64 + tot);
   size_t offs[3][3];
+  const size_t ofx[3] = {0, (size_t)n[0], (size_t)n[0] + n[1]};
   const long double pi = 3.141592653589793238462643383279502884L;
   const long double h = c->prm.h;
   for (int a = 0; a < 3; ++a) {
-    offs[a][0] = off;
-    for (int t = 0; t < n[a]; ++t) h64[off + t] = (double)cosl(2.0L * pi * t / n[a]);
-    off += n[a];
-    offs[a][1] = off;
-    for (int t = 0; t < n[a]; ++t) h64[off + t] = (double)sinl(2.0L * pi * t / n[a]);
-    off += n[a];
-    offs[a][2] = off;
-    for (int k = 0; k < n[a]; ++k) {
-      const long double sn = (n[a] > 1) ? sinl(pi * k / n[a]) : 0.0L;
-      h64[off + k] = (double)(4.0L / (h * h) * sn * sn);
+    for (int k = 0; k < 3; ++k) offs[a][k] = 3 * ofx[a] + (size_t)k * n[a];
+    // the quad-precision functions cost about a microsecond each on Arm hosts:
+    // once per angle, and not again for an axis of the same length
+    const int same = a > 0 && n[a] == n[0] ? 0 : (a > 1 && n[a] == n[1] ? 1 : a);
+    if (same < a) {
+      memcpy(hfx + ofx[a], hfx + ofx[same], n[a] * sizeof(psd::fx_tw));
+      memcpy(h64 + offs[a][0], h64 + offs[same][0], 3 * (size_t)n[a] * sizeof(double));
+      continue;
     }
-    off += n[a];
+    for (int t = 0; t < n[a]; ++t) {
+      const long double cs = cosl(2.0L * pi * t / n[a]), sn = sinl(2.0L * pi * t / n[a]);
+      hfx[ofx[a] + t] = psd::fx_make_tw(cs, sn);
+      h64[offs[a][0] + t] = (double)cs;
+      h64[offs[a][1] + t] = (double)sn;
+      const long double sh = (n[a] > 1) ? sinl(pi * t / n[a]) : 0.0L;
+      h64[offs[a][2] + t] = (double)(4.0L / (h * h) * sh * sh);
+    }
   }
   for (size_t i = 0; i < tot; ++i) h32[i] = (float)h64[i];
-  // Q62 twiddles of the fixed-point transforms
-  std::vector<psd::fx_tw> hfx((size_t)n[0] + n[1] + n[2]);
-  size_t ofx[3] = {0, (size_t)n[0], (size_t)n[0] + n[1]};
-  for (int a = 0; a < 3; ++a)
-    for (int t = 0; t < n[a]; ++t)
-      hfx[ofx[a] + t] = psd::fx_make_tw(cosl(2.0L * pi * t / n[a]), sinl(2.0L * pi * t / n[a]));
   {
     unsigned char* t = nullptr;
-    TRY(alloc(c, &t, tot * (sizeof(double) + sizeof(float)) + hfx.size() * sizeof(psd::fx_tw)));
+    TRY(alloc(c, &t, bytes));
     c->tables = t;
   }
-  psd::fx_tw* dfx = (psd::fx_tw*)c->tables;  // 16-byte entries first
-  double* d64 = (double*)(dfx + hfx.size());
+  CK(cudaMemcpy(c->tables, image.data(), bytes, cudaMemcpyHostToDevice));
+  psd::fx_tw* dfx = (psd::fx_tw*)c->tables;
+  double* d64 = (double*)(dfx + nfx);
   float* d32 = (float*)(d64 + tot);
-  CK(cudaMemcpy(d64, h64.data(), tot * sizeof(double), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(dfx, hfx.data(), hfx.size() * sizeof(psd::fx_tw), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d32, h32.data(), tot * sizeof(float), cudaMemcpyHostToDevice));
   for (int a = 0; a < 3; ++a) {
     c->tb64.twc[a] = d64 + offs[a][0];
     c->tb64.tws[a] = d64 + offs[a][1];
