@@ -579,12 +579,13 @@ cudaError_t mid_impl(T* data, const KParams& kp, Ctrl* ctrl, double* partials, T
 }
 
 template <typename T, int N>
-void set_attrs_T() {
+cudaError_t set_attrs_T() {
   constexpr int RP = kRadixPass, RD = kRadixMid;
   cudaFuncSetAttribute(k_dht_rows<T, N, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
   cudaFuncSetAttribute(k_dht_cols<T, N, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
   cudaFuncSetAttribute(k_mid<T, N, 4, RD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemPre);
   cudaFuncSetAttribute(k_mid<T, N, 6, RD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemPre);
+  return cudaSuccess;
 }
 
 #define PSD_DISPATCH_N(n, CALL)      \

@@ -30,15 +30,6 @@ cudaError_t launch_mid<float>(float* data, const KParams& kp, Ctrl* ctrl, double
   PSD_DISPATCH_N(n, (mid_impl<float, NN>(data, kp, ctrl, partials, xi, dspec, tb, st)));
 }
 
-void init_dht_attributes_f32() {
-  set_attrs_T<float, 8>();
-  set_attrs_T<float, 16>();
-  set_attrs_T<float, 32>();
-  set_attrs_T<float, 64>();
-  set_attrs_T<float, 128>();
-  set_attrs_T<float, 256>();
-  set_attrs_T<float, 512>();
-  set_attrs_T<float, 1024>();
-}
+cudaError_t init_dht_attributes_f32(int n) { PSD_DISPATCH_N(n, (set_attrs_T<float, NN>())); }
 
 }  // namespace psd

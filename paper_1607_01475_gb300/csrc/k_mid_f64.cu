@@ -24,7 +24,7 @@ cudaError_t launch_dht_last(const double* data, double* theta, float* out32, con
 
 namespace {
 template <int N, int RM>
-void set_attrs_mid_fx() {
+void set_attrs_mid_fx_radix() {
   constexpr size_t np = kFxThreads / LineFFT<fx, N, RM>::TS;
   constexpr int line = (int)(np * fx_pair_smem<N, RM, false>()), stage = (int)(np * N * sizeof(double2));
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
@@ -35,26 +35,20 @@ void set_attrs_mid_fx() {
   cudaFuncSetAttribute(k_last_fx<N, RM, EPI_THETA>, attr, line + stage);
   cudaFuncSetAttribute(k_last_fx<N, RM, EPI_RESID>, attr, line + stage);
 }
+template <int N>
+cudaError_t set_attrs_mid_fx() {
+  set_attrs_mid_fx_radix<N, 8>();
+  if constexpr (kFxShort<N> != 8) set_attrs_mid_fx_radix<N, kFxShort<N>>();
+  return cudaSuccess;
+}
 }  // namespace
 
-void init_dht_attributes_f32();
+cudaError_t init_dht_attributes_f32(int n);
 
-void init_dht_attributes() {
-  init_dht_attributes_f32();
-  set_attrs_mid_fx<8, 4>();
-  set_attrs_mid_fx<8, 8>();
-  set_attrs_mid_fx<16, 4>();
-  set_attrs_mid_fx<16, 8>();
-  set_attrs_mid_fx<32, 4>();
-  set_attrs_mid_fx<32, 8>();
-  set_attrs_mid_fx<64, 4>();
-  set_attrs_mid_fx<64, 8>();
-  set_attrs_mid_fx<128, 4>();
-  set_attrs_mid_fx<128, 8>();
-  set_attrs_mid_fx<256, 4>();
-  set_attrs_mid_fx<256, 8>();
-  set_attrs_mid_fx<512, 8>();
-  set_attrs_mid_fx<1024, 8>();
+cudaError_t init_dht_attributes(int n) {
+  const cudaError_t e = init_dht_attributes_f32(n);
+  if (e != cudaSuccess) return e;
+  PSD_DISPATCH_N(n, (set_attrs_mid_fx<NN>()));
 }
 
 }  // namespace psd

@@ -213,6 +213,7 @@ cudaError_t launch_accumulate_f64(double* u, const float* delta, const float* de
 // a = b = c = 0 (n values each, b and c may be null) unless *skip != 0.
 cudaError_t launch_zero_f32(float* a, float* b, float* c, size_t n, const int* skip, cudaStream_t st);
 
-void init_dht_attributes();
+// Shared-memory limits of the passes over lines of n points (loads those kernels).
+cudaError_t init_dht_attributes(int n);
 
 }  // namespace psd

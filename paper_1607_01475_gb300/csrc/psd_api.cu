@@ -1247,8 +1247,14 @@ psd_status psd_create(const psd_params* params, psd_handle* out) {
   kp.inv_ntot = 1.0 / (double)c->N;
   psd::finish_kparams(kp);
   c->pk = psd::pkind_of(params->p);
-  static const bool attrs = (psd::init_dht_attributes(), true);  // once, thread-safe
-  (void)attrs;
+  // once per length, thread-safe: the first handle of a process does not load the
+  // kernels of lengths it has no use for
+  static std::once_flag attrs[11];
+  for (int a = 0; a < params->dim; ++a) {
+    int k = 0;
+    while ((1 << k) < params->n[a]) ++k;
+    std::call_once(attrs[k], [&]() { (void)psd::init_dht_attributes(params->n[a]); });
+  }
 
   auto bail = [&](psd_status st) {
     g_create_error = c->err;
