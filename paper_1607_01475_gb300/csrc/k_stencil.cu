@@ -11,9 +11,8 @@
 namespace psd {
 namespace {
 
-// Four consecutive values of a row (16-byte aligned, FP64 32-byte) as FP32,
-// rounded or truncated to 20 bits; FP64 values outside the FP32 range give 0 or
-// infinity.
+// Values of u as FP32 for the gradient estimate of k_fx_scan, FP64 ones truncated to
+// 20 bits (0 or infinity outside the FP32 range).
 __device__ __forceinline__ float scan_f32(float v) { return v; }
 __device__ __forceinline__ float scan_f32(double v) {
   const unsigned h = (unsigned)__double2hiint(v);
@@ -21,23 +20,47 @@ __device__ __forceinline__ float scan_f32(double v) {
   const unsigned b = e <= 0 ? 0u : (e >= 255 ? 0x7F800000u : ((unsigned)e << 23) | ((h & 0xFFFFFu) << 3));
   return __uint_as_float(b | (h & 0x80000000u));
 }
-__device__ __forceinline__ void scan_load(const float* p, float (&v)[5]) {
+// The magnitude of a value as an integer that is ordered like it and is 0 for zeros
+// only (FP64: the high word, its last bit set where the low word is not zero).
+__device__ __forceinline__ unsigned scan_bits(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
+__device__ __forceinline__ unsigned scan_bits(double v) {
+  return ((unsigned)__double2hiint(v) & 0x7FFFFFFFu) | (__double2loint(v) != 0 ? 1u : 0u);
+}
+// An upper bound of |u| from the largest of those; FP32: of the FP64 field that it
+// rounds, which may have rounded to zero (|u| <= 2^-150 there).
+template <typename T>
+__device__ __forceinline__ double scan_bound(unsigned bits) {
+  if (sizeof(T) == 8) return bits == 0u ? 0.0 : __hiloint2double((int)bits, -1);
+  return (double)__uint_as_float(bits) * (1.0 + 0x1p-19) + 0x1p-140;
+}
+// Four consecutive values of a row (FP32: 16-byte aligned), and the largest of
+// their bits.
+__device__ __forceinline__ unsigned scan_load(const float* p, float (&v)[5]) {
   const float4 a = *reinterpret_cast<const float4*>(p);
   v[0] = a.x;
   v[1] = a.y;
   v[2] = a.z;
   v[3] = a.w;
+  return max(max(scan_bits(a.x), scan_bits(a.y)), max(scan_bits(a.z), scan_bits(a.w)));
 }
-__device__ __forceinline__ void scan_load(const double* p, float (&v)[5]) {
+__device__ __forceinline__ unsigned scan_load(const double* p, float (&v)[5]) {
+  unsigned m = 0u;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) v[k] = scan_f32(p[k]);
+  for (int k = 0; k < 4; ++k) {
+    const double x = p[k];
+    v[k] = scan_f32(x);
+    m = max(m, scan_bits(x));
+  }
+  return m;
 }
 
 // Bounds on |u| and on the modulus of the vertex gradient sums G (G from the 8
-// surrounding cells) into ctrl->umax, gmax (infinity if a value is not finite),
-// and the scales of a fixed-point residual at u into ctrl->fx_s, fx_g.  The
-// maxima are taken in FP32 on values within 2^-20 of u, so G is within 2^-17
-// max|u| of the estimate.  Each thread takes four consecutive vertices of a row.
+// surrounding cells) into ctrl->umax (0: every u is zero), gmax (not finite if a
+// value is not), and the scales of a fixed-point residual at u into ctrl->fx_s,
+// fx_g.  |u| comes from the bits of u.  G is estimated in FP32 on values within
+// 2^-20 of u: within 2^-15 max|u|, while its squares stay in the FP32 range (max|u| in
+// [2^-40, 2^60]); outside it is taken as 8 sqrt(3) max|u|, which bounds any
+// field.  Each thread takes four consecutive vertices of a row.
 template <typename T>
 __global__ void __launch_bounds__(NT) k_fx_scan(const T* __restrict__ u, KParams kp, double tol, int forced,
                                                 Ctrl* ctrl) {
@@ -46,7 +69,8 @@ __global__ void __launch_bounds__(NT) k_fx_scan(const T* __restrict__ u, KParams
   const int nx = kp.nx, ny = kp.ny, nz = kp.nz;
   const int lq = __ffs(nx / 4) - 1, lqy = lq + __ffs(ny) - 1;  // sizes are powers of two
   const size_t plane = (size_t)nx * ny, nq = plane * nz / 4;
-  float m = 0.0f, um = 0.0f;
+  float m = 0.0f;
+  unsigned ub = 0u;
   for (size_t i = blockIdx.x * (size_t)NT + threadIdx.x; i < nq; i += (size_t)gridDim.x * NT) {
     const int x = 4 * (int)(i & (nx / 4 - 1)), y = (int)((i >> lq) & (ny - 1)), z = (int)(i >> lqy);
     const int x4 = (x + 4) & (nx - 1), y1 = (y + 1) & (ny - 1), z1 = (z + 1) & (nz - 1);
@@ -55,7 +79,7 @@ __global__ void __launch_bounds__(NT) k_fx_scan(const T* __restrict__ u, KParams
     const T* r10 = u + (size_t)z1 * plane + (size_t)y * nx;
     const T* r11 = u + (size_t)z1 * plane + (size_t)y1 * nx;
     float av[5], bv[5], cv[5], dv[5];
-    scan_load(r00 + x, av);
+    ub = max(ub, scan_load(r00 + x, av));
     scan_load(r01 + x, bv);
     if (kp.dim == 2) {  // G_x = D(y) + D(y+1), G_y = A(y+1) - A(y)
       av[4] = scan_f32(r00[x4]);
@@ -64,8 +88,6 @@ __global__ void __launch_bounds__(NT) k_fx_scan(const T* __restrict__ u, KParams
       for (int k = 0; k < 4; ++k) {
         const float g0 = (av[k + 1] - av[k]) + (bv[k + 1] - bv[k]), g1 = (bv[k] - av[k]) + (bv[k + 1] - av[k + 1]);
         m = fmaxf(m, sqrtf(g0 * g0 + g1 * g1));
-        const float au = fabsf(av[k]);
-        um = (au <= FLT_MAX) ? fmaxf(um, au) : INFINITY;
       }
       continue;
     }
@@ -82,11 +104,9 @@ __global__ void __launch_bounds__(NT) k_fx_scan(const T* __restrict__ u, KParams
       const float g1 = ((bv[k] - av[k]) + (bv[k + 1] - av[k + 1])) + ((dv[k] - cv[k]) + (dv[k + 1] - cv[k + 1]));
       const float g2 = ((cv[k] - av[k]) + (cv[k + 1] - av[k + 1])) + ((dv[k] - bv[k]) + (dv[k + 1] - bv[k + 1]));
       m = fmaxf(m, sqrtf(g0 * g0 + g1 * g1 + g2 * g2));
-      const float au = fabsf(av[k]);
-      um = (au <= FLT_MAX) ? fmaxf(um, au) : INFINITY;  // NaN or infinity: infinity
     }
   }
-  unsigned mb = __float_as_uint(m), ub = __float_as_uint(um);  // of non-negative floats: ordered as integers
+  unsigned mb = __float_as_uint(m);  // of a non-negative float: ordered as an integer
   block_max2(mb, ub, smax);
   if (threadIdx.x == 0) {
     atomicMax(&ctrl->gmax2_hi, mb);
@@ -95,9 +115,9 @@ __global__ void __launch_bounds__(NT) k_fx_scan(const T* __restrict__ u, KParams
     sflag = atomicAdd(&ctrl->counter[CS_MISC], 1u) == gridDim.x - 1;
     if (sflag) {
       const double g = (double)__uint_as_float(atomicExch(&ctrl->gmax2_hi, 0u));
-      const double um2 = (double)__uint_as_float(atomicExch(&ctrl->umax_hi, 0u)) * (1.0 + 0x1p-19);
-      ctrl->umax = um2;
-      ctrl->gmax = g * (1.0 + 0x1p-18) + 0x1p-16 * um2;
+      const double um = scan_bound<T>(atomicExch(&ctrl->umax_hi, 0u));
+      ctrl->umax = um;
+      ctrl->gmax = um >= 0x1p-40 && um <= 0x1p60 ? g * (1.0 + 0x1p-18) + 0x1p-15 * um : 14.0 * um;
       ctrl->counter[CS_MISC] = 0;
       fx_decide(ctrl, kp, ctrl->umax, ctrl->gmax, forced ? INFINITY : tol);
     }

@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kWarps2D * 32)
     }
     if (!fixed) res2d_march<T, PK, MODE, V, false>(a, kp, ctrl, m, 0, 0, acc2, accm, um, gm);
   }
-  if constexpr (TRACK) track_publish(um, gm, fxs, fxg, ctrl, smax);
+  if constexpr (TRACK) track_publish(um, gm, fxs, fxg, fxs != kFxOff && a.d == nullptr, ctrl, smax);
   T v[2] = {acc2, accm};
   block_reduce<T, 2, true>(v, sred);
   if (publish_and_check_last<T>(v, 2, reinterpret_cast<T*>(partials), &ctrl->counter[CS_RES], &sflag)) {

@@ -407,7 +407,7 @@ __device__ __forceinline__ void res3d_col(const ResArgs<T>& a, const KParams& kp
   }
 
   if constexpr (TRACK) {
-    track_publish(um, gm, FX ? fxs : kFxOff, fxg, ctrl, sm.smax);
+    track_publish(um, gm, FX ? fxs : kFxOff, fxg, FX && a.d == nullptr, ctrl, sm.smax);
   }
   T v[2] = {acc2, accm};
   block_reduce<T, 2, true>(v, sm.sred);

@@ -333,11 +333,15 @@ __global__ void __launch_bounds__(NT)
 // The fixed-point variants' bookkeeping (see fx_decide).  track_publish: the
 // block's bounds on |u| and |G|^2 (um, gm: largest high words, of integers in
 // units of 2^-fxs and of the flux's |G|^2 when fxs is a scale, of FP64 values
-// otherwise) into the running maxima of ctrl; track_collect, in the last block:
-// the maxima become the iterate's bounds.
-__device__ __forceinline__ void track_publish(unsigned um, unsigned gm, int fxs, int fxg, Ctrl* ctrl, unsigned* smax) {
+// otherwise) into the running maxima of ctrl; scanned: ctrl->umax is the bound of this
+// very iterate, from its scan, and 0 there leaves both at 0 (the integers' unit would
+// bound it by 2^-23, and the next scales would be too coarse for a solution much
+// smaller than that).  track_collect, in the last block: the maxima become the
+// iterate's bounds.
+__device__ __forceinline__ void track_publish(unsigned um, unsigned gm, int fxs, int fxg, bool scanned, Ctrl* ctrl,
+                                              unsigned* smax) {
   block_max2(um, gm, smax);
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && !(scanned && ctrl->umax == 0.0)) {
     const bool fx = fxs != kFxOff;
     const double ub = fx ? ((double)um + 1.0) * fx_unit(fxs - 32) : __hiloint2double((int)um, -1);
     const double g2 = fx ? ((double)gm + 1.0) * fx_unit(2 * (fxs + fxg) - 96) : __hiloint2double((int)gm, -1);
