@@ -453,36 +453,42 @@ __global__ void __launch_bounds__(kFxThreads, 2)
     fx w[2];
     dht_split(sr, si, kk, N, w[0], w[1]);
     const double ml = syml[kk];
-    double mu = 0.0, ip = 0.0, dv[2];
+    double mu = 0.0, ip = 0.0, wl = 0.0, dv[2];  // wl: the symbol without its s mu (order 6: s mu^2) term
     if (ORDER == 4) {
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const double h = fx_leave<N, RM>(w[c], ln, 0);
         if (c == 0 || self) {
           mu = (c ? mxb : mxa) + ml;
-          ip = recip_pos(fma(mu, fma(se2, mu, s), 1.0));
+          wl = fma(se2 * mu, mu, 1.0);
+          ip = recip_pos(fma(s, mu, wl));
         }
         const double d = h * ip;
-        const double m = mu * d;
         dv[c] = d;
         acc[0] = fma(h, d, acc[0]);
-        acc[1] = fma(m, d, acc[1]);
+        acc[1] = fma(wl * d, d, acc[1]);
       }
     } else {
       // xi advances with the previous step and is added to the transformed
       // local residual; d = mu rt / P and T_h d = rt / P, P = 1 + mu (lam s +
-      // mu (s + s eps^2 mu)) (see k_mid)
+      // mu (s + s eps^2 mu)) (see k_mid), formed as wl + s mu^2
       const unsigned off = (unsigned)kk * line_stride, e = (unsigned)(q * TS + j) * pairs + p;
       const double2 xv = pre_x[e], dp = pre_d[e];
       const double xs[2] = {xv.x, xv.y}, ds[2] = {dp.x, dp.y};
       double xn[2], tn[2];
-      double mus[2], ips[2];
+      double mus[2], ips[2], wls[2];
+      auto symbol = [&](double m, double& w) {
+        const double m2 = m * m;
+        w = fma(fma(se2, m2, sl), m, 1.0);
+        return recip_pos(fma(s, m2, w));
+      };
       if (MIRROR) {  // both before the conversions: 187 us for a solve of L_h at 128^3, else 191
         mus[0] = mxa + ml;
         mus[1] = self ? mxb + ml : mus[0];
-        ips[0] = recip_pos(fma(mus[0], fma(mus[0], fma(se2, mus[0], s), sl), 1.0));
+        ips[0] = symbol(mus[0], wls[0]);
         ips[1] = ips[0];
-        if (self) ips[1] = recip_pos(fma(mus[1], fma(mus[1], fma(se2, mus[1], s), sl), 1.0));
+        wls[1] = wls[0];
+        if (self) ips[1] = symbol(mus[1], wls[1]);
       }
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
@@ -491,9 +497,10 @@ __global__ void __launch_bounds__(kFxThreads, 2)
         if (MIRROR) {
           mu = mus[c];
           ip = ips[c];
+          wl = wls[c];
         } else {
           mu = (c ? mxb : mxa) + ml;
-          ip = recip_pos(fma(mu, fma(mu, fma(se2, mu, s), sl), 1.0));
+          ip = symbol(mu, wl);
         }
         if (!(c == 0 && yo == 0 && x == 0 && kk == 0)) {  // mu > 0: every mode but the zero one
           xc = fma(-alpha_prev, ds[c], xs[c]);
@@ -501,12 +508,11 @@ __global__ void __launch_bounds__(kFxThreads, 2)
           td = rt * ip;
           d = mu * td;
         }
-        const double m = mu * d;
         xn[c] = xc;
         tn[c] = td;
         dv[c] = d;
         acc[0] = fma(rt, d, acc[0]);
-        acc[1] = fma(m, d, acc[1]);
+        acc[1] = fma(wl * td, d, acc[1]);
         acc[mid_nsums<double, ORDER>() - 1] = fma(rt, rt, acc[mid_nsums<double, ORDER>() - 1]);
       }
       put(xi_, off, xn[0], xn[1]);
