@@ -51,8 +51,8 @@ constexpr size_t fx_pair_smem() {
 
 // The common exponent and scale of a line pair from its team's values.  ROWS:
 // the team is TS consecutive threads; otherwise the team of pair p is the
-// threads tid = p (mod pairs).  share() reduces the largest exponent and the L1
-// norm relative to it within the warp; a team of several warps leaves them in
+// threads tid = p (mod pairs).  share() reduces the largest exponent and the squared
+// 2-norm relative to it within the warp; a team of several warps leaves them in
 // scr, and after a barrier line() combines the warps in a fixed order.
 struct FxLine {
   int E, B;  // largest biased exponent, scale
@@ -63,7 +63,7 @@ struct FxTeam {
   static constexpr bool kOneWarp = ROWS && TS <= 32;
   int p, pairs;
   int E;       // of this warp
-  unsigned l;  // L1 bound of this warp, in units of 2^(E - 1042)
+  unsigned l;  // bound on the squared 2-norm of this warp's points, in units of 2^(2 (E - 1032))
 
   __device__ __forceinline__ void share(const double (&xr)[R], const double (&xi)[R], uint2 (*scr)[32]) {
     const int nthr = (int)blockDim.x;
@@ -80,7 +80,7 @@ struct FxTeam {
     l = 0u;
 #pragma unroll
     for (int q = 0; q < R; ++q)
-      l += fx_l1((unsigned)__double2hiint(xr[q]), E) + fx_l1((unsigned)__double2hiint(xi[q]), E);
+      l += fx_square((unsigned)__double2hiint(xr[q]), E) + fx_square((unsigned)__double2hiint(xi[q]), E);
     for (int o = o0; o < o1; o <<= 1) l += __shfl_xor_sync(mask, l, o);
     const int lane = threadIdx.x & 31;
     if (!kOneWarp && (ROWS ? lane == 0 : lane < pairs)) scr[threadIdx.x >> 5][lane] = make_uint2((unsigned)E, l);
@@ -96,7 +96,7 @@ struct FxTeam {
     unsigned lm = 0u;
     for (int w = w0; w < nw; w += step) {
       const uint2 v = scr[w][lane];
-      lm += (v.y >> min(Em - (int)v.x, 31)) + 1u;
+      lm += (v.y >> min(2 * (Em - (int)v.x), 31)) + 1u;
     }
     return {Em, fx_scale<FxPlan<N, RM>>(lm)};
   }

@@ -14,21 +14,27 @@
 // largest biased exponent), a value enters as q = x 2^(B - (E - 1022)),
 // rounded, |q| <= 2^B.  A radix-RP butterfly can grow a modulus by RP; a
 // twiddle product in Q62 (the high 64 bits of the product) divides by 4.
-// With Sum_p the product of the first p radices, the modulus after pass p is
-// at most sqrt(2) 2^B Sum_p / 4^(p-1), and at most L1 / 4^(p-1) with L1 = sum
-// |re| + |im| over the line: every intermediate value of the FFT is a sum of
-// rotated inputs, each at most once.  All moduli stay below 2^61, which leaves
-// room for the sums of a rotation (sqrt(2)) and of the Hartley split (2 sqrt(2)),
-// when B <= 60 - H, H = max_p log2(Sum_p / 4^(p-1)), or when L1 <= 2^61: B is
-// the larger of the two, so that a line with few large points (a decaying
-// spectrum), which does not grow to the worst case, keeps the bits.
+// With Sum_p the product of the first p radices, an intermediate value of pass p
+// is a sum of at most Sum_p rotated inputs, each at most once, divided by 4^(p-1).
+// Its modulus is therefore at most sqrt(2) 2^B Sum_p / 4^(p-1), and at most
+// sqrt(Sum_p) L2 / 4^(p-1) with L2 the 2-norm of the (scaled) line, which is largest
+// at p = 1 for radices up to 8.  All moduli stay below 2^61, which leaves room for
+// the sums of a rotation (sqrt(2)) and of the Hartley split (2 sqrt(2)), when
+// B <= 60 - H, H = max_p log2(Sum_p / 4^(p-1)), or when sqrt(R) L2 <= 2^61: B is the
+// larger of the two.  The second keeps the bits of every line whose points are not
+// all large, from one large point or a decaying spectrum to a point that stands out
+// of a dense background: the error relative to the line's norm is then about
+// sqrt(2 N R) 2^-61, whatever the line's shape.  (The 1-norm in its place has the same
+// cost, but lost up to 2 bits against FP64 on 1024 points with a background of 1/4
+// to 1/128 of the largest: 9.0e-16 against FP64's 2.0e-16, 1.1e-16 now.)
 //
 // Error: every step rounds to a unit of 2^-B (B = 55 .. 60) of the line's
 // largest value, against 2^-53 of the value in FP64, with two to three units
 // on the outputs, so that the transform's error relative to the norm of the
-// line stays below that of the FP64 butterflies (tests/fx_line_check.cu
-// measures both against long double, for n = 8 .. 1024 with radix 8 and
-// n = 8 .. 256 with radix 4, dense and decaying lines).  Lines whose largest value is below 2^-958 give zero; a NaN or an
+// line stays below that of the FP64 butterflies (tests/fx_line_check.cu and
+// tests/fx_peak_check.cu measure both against long double, for n = 8 .. 1024 with
+// radix 8 and n = 8 .. 256 with radix 4: 0.4 to 1.2e-16 on dense, decaying and
+// peaked lines, FP64 1.1 to 2.3e-16).  Lines whose largest value is below 2^-958 give zero; a NaN or an
 // infinity makes every output of its line pair NaN, as the FP64 sums would.
 #pragma once
 
@@ -171,21 +177,25 @@ struct FxPlan {
 constexpr int kFxMinExp = 64;    // a line whose largest biased exponent is below this is zero
 constexpr int kFxMaxExp = 2046;  // above: NaN or infinity
 
-// An upper bound of this value's share of the line's L1 norm in units of
-// 2^(E - 1042), from its high word.
-__host__ __device__ __forceinline__ unsigned fx_l1(unsigned hi, int E) {
+// An upper bound of this value's share of the line's squared 2-norm in units of
+// 2^(2 (E - 1032)), from its high word: at most 2^20, so that 2048 values fit.
+__host__ __device__ __forceinline__ unsigned fx_square(unsigned hi, int E) {
   const int d = E - (int)((hi >> 20) & 0x7FFu);
-  return ((((hi & 0xFFFFFu) | 0x100000u) >> 1) >> (d < 31 ? d : 31)) + 1u;
+  const unsigned m = ((((hi & 0xFFFFFu) | 0x100000u) >> 11) >> (d < 31 ? d : 31)) + 1u;
+  return m * m;
 }
-// The scale B of a line whose L1 norm is below l1 2^(E - 1042).
+// The name under which tests/fx_line_check.cu sums the same bound.
+__host__ __device__ __forceinline__ unsigned fx_l1(unsigned hi, int E) { return fx_square(hi, E); }
+// The scale B of a line whose squared 2-norm is below l2 2^(2 (E - 1032)):
+// R L2^2 2^(2 B) <= 2^122 in units of 2^(2 (E - 1022)).
 template <class Plan>
-__host__ __device__ __forceinline__ int fx_scale(unsigned l1) {
+__host__ __device__ __forceinline__ int fx_scale(unsigned l2) {
 #ifdef __CUDA_ARCH__
-  const int bits = 32 - __clz((int)l1);
+  const int bits = 32 - __clz((int)l2);
 #else
-  const int bits = l1 ? 32 - __builtin_clz(l1) : 0;
+  const int bits = l2 ? 32 - __builtin_clz(l2) : 0;
 #endif
-  const int B = 81 - bits;
+  const int B = (142 - Plan::lr - bits) >> 1;
   return B < Plan::B ? Plan::B : (B > 60 ? 60 : B);
 }
 
