@@ -123,7 +123,7 @@ cudaError_t launch_linesearch(const T* u, const T* ubase, const T* d, int pk, co
 
 // Bounds on |u| and on the unscaled vertex gradient sums |G| (g = q G) of u into
 // ctrl->umax, gmax, and the scales of a fixed-point residual at u (fx_decide;
-// forced: without its error rule) into ctrl->fx_s, fx_g.  T: FP64, or FP32 for
+// forced: without its error rule; tol: see there) into ctrl->fx_s, fx_g.  T: FP64, or FP32 for
 // the FP64 field that u rounds.
 template <typename T>
 cudaError_t launch_fx_scan(const T* u, const KParams& kp, double tol, bool forced, Ctrl* ctrl, cudaStream_t st);

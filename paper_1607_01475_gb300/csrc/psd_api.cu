@@ -569,13 +569,16 @@ psd_status ensure_fp32(psd_context* c) {
 // large enough for the FP64 variant to cost more.
 bool fx_scan_pays(const psd_context* c) { return psd::fx_stencils(c->kp, c->pk) && c->N >= kFxScanCells; }
 // Scales of the fixed-point residual at u into ctrl (without a scan: the FP64 variant).
+// u32: u rounded, for an outer residual of a mixed solve, whose correction absorbs errors
+// far below its tolerance (3D, as fx_decide says); every other residual is as
+// exact as FP64 whatever the handle's tolerance.
 psd_status fx_scan(psd_context* c, const double* u, const float* u32, Ctrl* ctrl) {
   if (!fx_scan_pays(c)) return PSD_OK;
   ProfScope p_(c, PSD_PROF_OTHER);
   if (u32)
-    CK(psd::launch_fx_scan<float>(u32, c->kp, c->prm.tol, false, ctrl, c->st));
+    CK(psd::launch_fx_scan<float>(u32, c->kp, c->kp.dim == 3 ? c->prm.tol : 0.0, false, ctrl, c->st));
   else
-    CK(psd::launch_fx_scan<double>(u, c->kp, c->prm.tol, false, ctrl, c->st));
+    CK(psd::launch_fx_scan<double>(u, c->kp, 0.0, false, ctrl, c->st));
   return PSD_OK;
 }
 
@@ -1429,7 +1432,7 @@ psd_status psd_residual_fixed(psd_handle c, const double* u, const double* f, do
   init_ctrl(h, -1.0, 1 << 30);
   TRY(upload_ctrl(c, c->ctrl2, h));
   { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_norms(u, c->N, kp.hd, c->ctrl2, c->partials, c->st)); }
-  { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_fx_scan<double>(u, kp, c->prm.tol, true, c->ctrl2, c->st)); }
+  { ProfScope p_(c, PSD_PROF_OTHER); CK(psd::launch_fx_scan<double>(u, kp, 0.0, true, c->ctrl2, c->st)); }
   Ctrl h2;
   TRY(read_ctrl(c, c->ctrl2, h2));
   const double umax = h2.res_linf;

@@ -180,9 +180,9 @@ __device__ __forceinline__ bool fx_scale_of(double vmax, int* S) {
 // max|u|, so g >= 2).  With 2^ge = 2^(61-S-g) >= |G|, the flux error is at most cdiv
 // 2^-51 2^(3 ge) per cell (24 fluxes of a few units of 2^-58 of the cube of 2^ge);
 // the variant runs when that is below the FP64 rounding of the Laplacian sums,
-// about 64 units 2^-53 of cbih max|u|, or, in the 2-norm, below tol / 20.
-// Otherwise (gradients steeper than any smooth field on the grid) the FP64
-// variant runs.
+// about 64 units 2^-53 of cbih max|u|.  Otherwise (gradients steeper than any smooth
+// field on the grid) the FP64 variant runs.  tol > 0, for the outer residuals of 3D
+// mixed solves only: also when the error is below tol / 20 in the 2-norm.
 template <class C, class K>
 __device__ __forceinline__ void fx_decide(C* c, const K& kp, double umax, double gmax, double tol) {
   int S = kFxOff, g = 60;

@@ -387,9 +387,8 @@ __global__ void __launch_bounds__(kWarps2D * 32)
     }
     if (!fixed) ls2d_march<T, PK, INNER, V, false>(u, ubase, d, kp, trial, m, 0, 0, acc, sbb, gm);
   }
-  const double tol = TRACK ? ctrl->tol : -1.0;
   if constexpr (TRACK) ls_track(acc, sbb, gm, fixed, Su, Sd, ctrl, smax);
-  ls_finish<T, PK>(acc, sred, partials, ctrl, kp, &sflag, tol);
+  ls_finish<T, PK>(acc, sred, partials, ctrl, kp, &sflag, TRACK);
 }
 
 }  // namespace

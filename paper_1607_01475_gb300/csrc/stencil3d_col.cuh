@@ -457,7 +457,7 @@ struct LsColSmem {
 template <typename T, int PK, bool INNER, bool FX>
 __device__ __forceinline__ void ls3d_col(const T* __restrict__ u, const T* __restrict__ ubase,
                                          const T* __restrict__ d, const KParams& kp, Ctrl* ctrl, double* partials,
-                                         double tol, LsColSmem<T>& sm, T* sred, int Su, int Sd) {
+                                         LsColSmem<T>& sm, T* sred, int Su, int Sd) {
   constexpr bool TRACK = sizeof(T) == 8 && PK == PK_4 && !INNER;
   static_assert(!FX || TRACK, "FX: FP64 p = 4 without a base only");
   using LT = typename std::conditional<FX, long long, T>::type;
@@ -564,7 +564,7 @@ __device__ __forceinline__ void ls3d_col(const T* __restrict__ u, const T* __res
   if constexpr (TRACK) {
     ls_track(acc, sbb, gm, FX, Su, Sd, ctrl, sm.smax);
   }
-  ls_finish<T, PK>(acc, sred, partials, ctrl, kp, &sm.sflag, TRACK ? tol : -1.0);
+  ls_finish<T, PK>(acc, sred, partials, ctrl, kp, &sm.sflag, TRACK);
 }
 
 template <typename T, int PK, bool INNER>
@@ -578,11 +578,11 @@ __global__ void __launch_bounds__(256, 3)
   if constexpr (sizeof(T) == 8 && PK == PK_4 && !INNER) {
     int Su, Sd;
     if (ls_scales(ctrl, &Su, &Sd)) {
-      ls3d_col<T, PK, INNER, true>(u, ubase, d, kp, ctrl, partials, ctrl->tol, sm, sred, Su, Sd);
+      ls3d_col<T, PK, INNER, true>(u, ubase, d, kp, ctrl, partials, sm, sred, Su, Sd);
       return;
     }
   }
-  ls3d_col<T, PK, INNER, false>(u, ubase, d, kp, ctrl, partials, ctrl->tol, sm, sred, 0, 0);
+  ls3d_col<T, PK, INNER, false>(u, ubase, d, kp, ctrl, partials, sm, sred, 0, 0);
 }
 
 }  // namespace

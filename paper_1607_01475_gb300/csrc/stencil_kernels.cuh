@@ -661,11 +661,11 @@ __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double 
 }
 
 // Block and grid reduction of a line-search pass (fixed order; the last
-// block runs the epilogue).  fx_tol >= 0: the scales of the residual that
+// block runs the epilogue).  track: the scales of the residual that
 // follows are chosen from the bounds in ctrl (fx_decide).  sred: 32 * ls_nsums<PK>() shared elements.
 template <typename T, int PK>
 __device__ __forceinline__ void ls_finish(T (&acc)[ls_nsums<PK>()], T* sred, double* partials, Ctrl* ctrl,
-                                          const KParams& kp, int* sflag, double fx_tol = -1.0) {
+                                          const KParams& kp, int* sflag, bool track = false) {
   constexpr int M = ls_nsums<PK>();
   block_reduce<T, M, false>(acc, sred);
   if (publish_and_check_last<T>(acc, M, reinterpret_cast<T*>(partials), &ctrl->counter[CS_LS], sflag)) {
@@ -677,10 +677,10 @@ __device__ __forceinline__ void ls_finish(T (&acc)[ls_nsums<PK>()], T* sred, dou
 #pragma unroll
       for (int m = 0; m < M; ++m) tot[m] = (double)tt[m];
       linesearch_epilogue<PK>(ctrl, kp, tot, sizeof(T) == 4);
-      if (fx_tol >= 0.0) {
+      if (track) {
         // the next iterate u + alpha d: |u| and |G| are at most these
         const double al = fabs(ctrl->alpha), gd = fx_sqrt_above(atomicExch(&ctrl->gmax2_hi, 0u));
-        fx_decide(ctrl, kp, ctrl->umax + al * __hiloint2double((int)ctrl->dmax_hi, 0), ctrl->gmax + al * gd, fx_tol);
+        fx_decide(ctrl, kp, ctrl->umax + al * __hiloint2double((int)ctrl->dmax_hi, 0), ctrl->gmax + al * gd, 0.0);
       }
     }
   }
