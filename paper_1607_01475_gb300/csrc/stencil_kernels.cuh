@@ -488,6 +488,13 @@ __host__ __device__ constexpr int ls_nsums() {
   return PK == PK_6 ? 5 : (PK == PK_4 ? 3 : 2);
 }
 
+// Whether 2 x < y for x, y >= 0 (FP64: from the high words, an FP64 comparison takes
+// the slot of an addition).
+__device__ __forceinline__ bool below_half(float x, float y) { return 2.0f * x < y; }
+__device__ __forceinline__ bool below_half(double x, double y) {
+  return __double2hiint(x) + 0x100000 < __double2hiint(y);
+}
+
 // Vertex sums for one vertex with a = grad u (+ grad ubase), b = grad d.
 // With A = |a|^2, B = a.b, C = |b|^2, the vertex term of P(alpha) =
 // sum_v |a + alpha b|^{p-2} (a + alpha b).b is (A + 2 alpha B + alpha^2 C)^k
@@ -530,7 +537,10 @@ __device__ __forceinline__ void ls_accumulate(const T (&av)[3], const T (&bv)[3]
       w = fc > T(0) ? T(1) / fc : T(0);
     } else {
       fc = pow(c2, beta);
-      dfac = A > T(0) ? pow(A, beta) * expm1(beta * log1p(fmax(dl / A, T(-1)))) : fc;
+      // from dl where |c| is close to |a|; where it is much smaller, dl / A + 1 has lost it,
+      // and with it |c|^{p-2}, up to eps^{(p-2)/2} |a|^{p-2}
+      const T fa = pow(A, beta);
+      dfac = below_half(c2, A) ? fc - fa : (A > T(0) ? fa * expm1(beta * log1p(fmax(dl / A, T(-1)))) : fc);
       w = c2 > T(0) ? pm2 * fc / c2 : T(0);
     }
     acc[0] += fc * trial * C + dfac * B;
