@@ -246,6 +246,7 @@ __device__ __forceinline__ void mid_finish(T (&acc)[mid_nsums<T, ORDER>()], T* s
       ctrl->c2 = -1.0;
       ctrl->c3 = 0.0;
       ctrl->trial = ctrl->alpha;
+      ctrl->ls_step = 0.0;
       ctrl->alpha = 0.0;
       ctrl->ls_pass = 0;
       ctrl->dmax_hi = 0u;

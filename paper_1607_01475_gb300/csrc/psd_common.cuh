@@ -71,6 +71,7 @@ struct Ctrl {
   int hist_cap;
   double* hist_alpha;  // device arrays of length hist_cap (or null)
   double* hist_res;
+  double ls_step;  // general p: how far the last Newton pass moved trial (0: first pass of the iteration)
 };
 
 // Problem scalars passed by value to the kernels.

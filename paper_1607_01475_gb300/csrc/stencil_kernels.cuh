@@ -613,6 +613,25 @@ __device__ __forceinline__ void ls_track(T (&acc)[M], T sbb, unsigned gm, bool f
   }
 }
 
+// Whether the Newton step `step` from `trial` (both moduli) is the general-p line
+// search's last: what it leaves has to be below rounding.  For p >= 3, q' is
+// Lipschitz and the step after one of length e is M e^2, M = step / prev^2 from the last
+// two (prev: the move before, 0 on the first pass, where trial stands for it), so
+// step^3 / prev^2 is left.  For 2 < p < 3, q' is only Hoelder continuous: where the
+// gradients vanish at the root, Newton contracts by up to (p - 2) / (p - 1) a pass,
+// and step^2 / prev bounds what is left at every rate.  A limit on the step alone
+// (5e-9) left alpha 1e-10 off there.  Steps that stop contracting are rounding.  FP32
+// sums give an alpha that is used rounded to FP32.
+__device__ __forceinline__ bool newton_settled(double step, double trial, double prev, bool smooth, bool f32) {
+  if (!(step <= (f32 ? 1e-4 : 5e-9) * trial)) return false;
+  if (step <= (f32 ? 2e-7 : 4e-16) * trial) return true;
+  if (prev > 0.0 && step >= 0.7 * prev) return true;
+  const double left = (f32 ? 1e-8 : 1e-16) * trial;
+  if (!smooth) return step * step <= left * prev;
+  const double e = prev > 0.0 ? prev : trial;
+  return step * step * step <= left * (e * e);
+}
+
 // Last-block logic of the line search (f32: the sums are FP32's).
 template <int PK>
 __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double (&tot)[ls_nsums<PK>()], bool f32) {
@@ -633,9 +652,7 @@ __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double 
     }
   } else {
     // one safeguarded Newton step per launch; state in c1 (lo), c2 (hi), c3 (done
-    // flag); the first trial is the previous iteration's step size.  A step below
-    // 1e-4 of alpha (FP32 sums, whose alpha is used rounded to FP32) or 5e-9 (FP64)
-    // is the last: what it leaves is of the order of its square.
+    // flag); the first trial is the previous iteration's step size.
     const double trial = f32 ? (double)(float)ctrl->trial : ctrl->trial;
     const double qv = -ctrl->rd + trial * lin + kp.cdiv * kp.hd * tot[0];
     const double dqv = lin + kp.cdiv * kp.hd * tot[1];
@@ -646,7 +663,7 @@ __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double 
       hi = trial;
     const double step = (dqv > 0.0) ? qv * recip_pos(dqv) : 0.0;
     double nw = (dqv > 0.0) ? trial - step : 0.5 * (lo + hi);
-    const bool tiny = (dqv > 0.0) && fabs(step) <= (f32 ? 1e-4 : 5e-9) * fabs(trial);
+    const bool tiny = (dqv > 0.0) && newton_settled(fabs(step), fabs(trial), ctrl->ls_step, kp.p >= 3.0, f32);
     if (!tiny) {
       if (hi > 0.0) {
         if (!(lo < nw && nw < hi)) nw = 0.5 * (lo + hi);
@@ -660,6 +677,7 @@ __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double 
     }
     ctrl->c1 = lo;
     ctrl->c2 = hi;
+    ctrl->ls_step = fabs(nw - trial);
     ctrl->alpha = nw;
     ctrl->trial = nw;
     if (!isfinite(nw) || !isfinite(qv)) {

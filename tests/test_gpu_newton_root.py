@@ -1,4 +1,5 @@
-"""The general-p line search at a root where the vertex gradients vanish.  f is chosen so that the first
+"""The general-p line search at a root where Newton's method is slow: for 2 < p < 3
+q' is not Lipschitz where vertex gradients vanish.  f is chosen so that the first
 direction is d = -u0 / a with a = (L_h u0, u0) / (N_h[u0], u0): then the root of
 q(alpha) = (N_h[u0 + alpha d] - f, d) is a, where u0 + a d = 0 and every gradient
 vanishes.
@@ -20,7 +21,7 @@ from paper_1607_01475_gb300 import Solver, synthetic  # noqa: E402
 
 
 @pytest.mark.parametrize("shape", [(64, 64), (16, 16, 32)])
-@pytest.mark.parametrize("p", [3.0, 3.5, 4.5, 5.0])
+@pytest.mark.parametrize("p", [2.1, 2.2, 2.5, 3.0, 3.5, 5.0])
 @pytest.mark.parametrize("s,eps", [(10.0, 0.01), (100.0, 0.1)])
 def test_root_at_vanishing_gradients(oracle, shape, p, s, eps):
     h = 2 * np.pi / shape[-1]
