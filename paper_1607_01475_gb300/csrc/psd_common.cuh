@@ -427,11 +427,13 @@ __device__ __forceinline__ float recip_ge1(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return fmaf(r, fmaf(-x, r, 1.0f), r);
 }
-// 1/x for finite x > 0 in FP64 (the symbols): the hardware estimate (relative error
-// below 2^-20) with one cubic step r (1 + e + e^2), e = 1 - x r: within an
-// ulp of 1/x in three FP64 operations.
+// 1/x for x >= 0 in FP64 (the symbols, the line search's slopes): the hardware estimate
+// (rcp.approx.ftz.f64, about 20 bits) with one step of the third-order Newton-Householder
+// iteration for the reciprocal, r (1 + e + e^2), e = 1 - x r, which leaves e^3: within an
+// ulp of 1/x (tests/recip64_check.cu) in three FP64 operations.  The estimate flushes
+// subnormal arguments and results: those, 0, infinity and NaN take the quotient.
 __device__ __forceinline__ double recip_pos(double x) {
-  if ((unsigned)__double2hiint(x) >= 0x7FE00000u) return 1.0 / x;  // 2^1023 and above, infinity, NaN
+  if ((unsigned)__double2hiint(x) - 0x00100000u >= 0x7FC00000u) return 1.0 / x;  // outside [2^-1022, 2^1022)
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   const double e = fma(-x, r, 1.0);
