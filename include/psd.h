@@ -30,6 +30,9 @@
  *  - Every call returns a psd_status; nothing aborts.  After an error,
  *    psd_last_error() returns a one-line description.
  *  - A handle is not thread safe: one host thread at a time.
+ *  - FP64 transforms (in every call that solves L_h or applies T_h) take values
+ *    below 2^-1022 for zero in their results; a NaN or an infinity in a grid
+ *    makes its whole transform NaN.
  */
 #ifndef PSD_H
 #define PSD_H

@@ -34,8 +34,10 @@
 // line stays below that of the FP64 butterflies (tests/fx_line_check.cu and
 // tests/fx_peak_check.cu measure both against long double, for n = 8 .. 1024 with
 // radix 8 and n = 8 .. 256 with radix 4: 0.4 to 1.2e-16 on dense, decaying and
-// peaked lines, FP64 1.1 to 2.3e-16).  Lines whose largest value is below 2^-958 give zero; a NaN or an
-// infinity makes every output of its line pair NaN, as the FP64 sums would.
+// peaked lines, FP64 1.1 to 2.3e-16).  The passes scale lines
+// whose largest value is below 2^-958 up first (fx_enter), and subnormal outputs are
+// 0; a NaN or an infinity makes every output of its line pair NaN, as the FP64 sums
+// would.
 #pragma once
 
 #include "fft_line.cuh"
@@ -174,7 +176,7 @@ struct FxPlan {
   static constexpr int kOut = -1022 + 2 * (P - 1) - 1;
 };
 
-constexpr int kFxMinExp = 64;    // a line whose largest biased exponent is below this is zero
+constexpr int kFxMinExp = 64;    // lines whose largest biased exponent is below this are scaled up first
 constexpr int kFxMaxExp = 2046;  // above: NaN or infinity
 
 // An upper bound of this value's share of the line's squared 2-norm in units of
