@@ -13,8 +13,8 @@ struct fx_tw;  // Q62 twiddle of the block fixed-point transforms (fx_line.cuh)
 // Per-axis tables owned by a context, in FP64 and FP32.
 template <typename T>
 struct AxisTables {
-  const T* twc[3];  // cos(2 pi t / n_a), t < n_a
-  const T* tws[3];  // sin(2 pi t / n_a)
+  const T* twc[3];  // cos(2 pi t / n_a), t < n_a (FP32)
+  const T* tws[3];  // sin(2 pi t / n_a) (FP32)
   const T* sym[3];  // (4/h^2) sin^2(pi k / n_a), k < n_a
   // tile widths chosen by the autotuner: at most this many line pairs per
   // block in the row, strided and middle passes (0: as many as fill 256

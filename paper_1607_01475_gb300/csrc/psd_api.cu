@@ -216,14 +216,14 @@ psd_status validate(const psd_params* p, std::string& why) {
 psd_status build_tables(psd_context* c) {
   const int dim = c->prm.dim;
   int n[3] = {c->prm.n[0], c->prm.n[1], dim == 3 ? c->prm.n[2] : 1};
-  const size_t nfx = (size_t)n[0] + n[1] + n[2], tot = 3 * nfx;
+  const size_t nfx = (size_t)n[0] + n[1] + n[2];
   // one image of all tables: Q62 twiddles of the fixed-point transforms (16-byte
-  // entries first), then cosines, sines and symbols in FP64 and in FP32
-  const size_t bytes = nfx * sizeof(psd::fx_tw) + tot * (sizeof(double) + sizeof(float));
+  // entries first), the symbols in FP64, and cosines, sines and symbols in FP32
+  const size_t bytes = nfx * (sizeof(psd::fx_tw) + sizeof(double) + 3 * sizeof(float));
   std::vector<psd::fx_tw> image((bytes + sizeof(psd::fx_tw) - 1) / sizeof(psd::fx_tw));
   psd::fx_tw* hfx = image.data();
-  double* h64 = (double*)(hfx + nfx);
-  float* h32 = (float*)(h64 + tot);
+  double* hsym = (double*)(hfx + nfx);
+  float* h32 = (float*)(hsym + nfx);
   size_t offs[3][3];
   const size_t ofx[3] = {0, (size_t)n[0], (size_t)n[0] + n[1]};
   const long double pi = 3.141592653589793238462643383279502884L;
@@ -235,19 +235,20 @@ psd_status build_tables(psd_context* c) {
     const int same = a > 0 && n[a] == n[0] ? 0 : (a > 1 && n[a] == n[1] ? 1 : a);
     if (same < a) {
       memcpy(hfx + ofx[a], hfx + ofx[same], n[a] * sizeof(psd::fx_tw));
-      memcpy(h64 + offs[a][0], h64 + offs[same][0], 3 * (size_t)n[a] * sizeof(double));
+      memcpy(hsym + ofx[a], hsym + ofx[same], n[a] * sizeof(double));
+      memcpy(h32 + offs[a][0], h32 + offs[same][0], 3 * (size_t)n[a] * sizeof(float));
       continue;
     }
     for (int t = 0; t < n[a]; ++t) {
       const long double cs = cosl(2.0L * pi * t / n[a]), sn = sinl(2.0L * pi * t / n[a]);
       hfx[ofx[a] + t] = psd::fx_make_tw(cs, sn);
-      h64[offs[a][0] + t] = (double)cs;
-      h64[offs[a][1] + t] = (double)sn;
       const long double sh = (n[a] > 1) ? sinl(pi * t / n[a]) : 0.0L;
-      h64[offs[a][2] + t] = (double)(4.0L / (h * h) * sh * sh);
+      hsym[ofx[a] + t] = (double)(4.0L / (h * h) * sh * sh);
+      h32[offs[a][0] + t] = (float)(double)cs;
+      h32[offs[a][1] + t] = (float)(double)sn;
+      h32[offs[a][2] + t] = (float)hsym[ofx[a] + t];
     }
   }
-  for (size_t i = 0; i < tot; ++i) h32[i] = (float)h64[i];
   {
     unsigned char* t = nullptr;
     TRY(alloc(c, &t, bytes));
@@ -255,12 +256,10 @@ psd_status build_tables(psd_context* c) {
   }
   CK(cudaMemcpy(c->tables, image.data(), bytes, cudaMemcpyHostToDevice));
   psd::fx_tw* dfx = (psd::fx_tw*)c->tables;
-  double* d64 = (double*)(dfx + nfx);
-  float* d32 = (float*)(d64 + tot);
+  double* dsym = (double*)(dfx + nfx);
+  float* d32 = (float*)(dsym + nfx);
   for (int a = 0; a < 3; ++a) {
-    c->tb64.twc[a] = d64 + offs[a][0];
-    c->tb64.tws[a] = d64 + offs[a][1];
-    c->tb64.sym[a] = d64 + offs[a][2];
+    c->tb64.sym[a] = dsym + ofx[a];
     c->tb32.twc[a] = d32 + offs[a][0];
     c->tb32.tws[a] = d32 + offs[a][1];
     c->tb32.sym[a] = d32 + offs[a][2];
