@@ -216,7 +216,8 @@ psd_status validate(const psd_params* p, std::string& why) {
 psd_status build_tables(psd_context* c) {
   const int dim = c->prm.dim;
   int n[3] = {c->prm.n[0], c->prm.n[1], dim == 3 ? c->prm.n[2] : 1};
-  const size_t nfx = (size_t)n[0] + n[1] + n[2];
+  // entries per table kind, padded (n[2] = 1 in 2D would leave all that follows odd)
+  const size_t nfx = ((size_t)n[0] + n[1] + n[2] + 31) / 32 * 32;
   // one image of all tables: Q62 twiddles of the fixed-point transforms (16-byte
   // entries first), the symbols in FP64, and cosines, sines and symbols in FP32
   const size_t bytes = nfx * (sizeof(psd::fx_tw) + sizeof(double) + 3 * sizeof(float));

@@ -32,7 +32,7 @@
 
 namespace {
 
-constexpr int kMaxBlocks = 2048;  // residual blocks: every valid grid needs at most 2048 on up to 1024 SMs
+constexpr int kMaxBlocks = 2048;  // residual blocks: every valid grid needs at most 2048 on up to 512 SMs
 constexpr size_t kCtrlBytes = (sizeof(psd::Ctrl) + 255) / 256 * 256;
 constexpr size_t kScratchBytes = kCtrlBytes + (size_t)kMaxBlocks * 2 * sizeof(double);
 constexpr int kMaxDevices = 64;

@@ -690,7 +690,8 @@ __device__ void linesearch_epilogue(Ctrl* ctrl, const KParams& kp, const double 
 
 // Block and grid reduction of a line-search pass (fixed order; the last
 // block runs the epilogue).  track: the scales of the residual that
-// follows are chosen from the bounds in ctrl (fx_decide).  sred: 32 * ls_nsums<PK>() shared elements.
+// follows are chosen from the bounds in ctrl (fx_decide).  sred:
+// red_size<T>(ls_nsums<PK>()) shared elements.
 template <typename T, int PK>
 __device__ __forceinline__ void ls_finish(T (&acc)[ls_nsums<PK>()], T* sred, double* partials, Ctrl* ctrl,
                                           const KParams& kp, int* sflag, bool track = false) {
