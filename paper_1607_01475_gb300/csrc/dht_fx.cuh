@@ -3,11 +3,11 @@
 // the preconditioner and the last pass of the mixed solver's outer loop.
 // Data in memory is FP64 before and after every pass.
 //
-// At 256^3 a pass moves 268 MB (40 us at the measured copy rate) and takes 92
+// At 256^3 a pass moves 268 MB (40 us at the measured copy rate) and takes 88
 // us (rows, columns), bound by integer issue; with FP64 butterflies it took 547
-// us.  The sixth-order middle pass takes 628 us instead of 1711, bound by the
-// 15 FP64 operations per element of the symbol division and the Parseval sums
-// (480 us at 1.74 per clock and SM).
+// us.  The sixth-order middle pass takes 535 us instead of 1711, bound by the
+// 13 FP64 operations per element of the symbol division, the Parseval sums and the
+// output conversions (about 410 us at 1.74 per clock and SM) and by integer issue.
 #pragma once
 
 #include <algorithm>
@@ -158,7 +158,7 @@ __device__ __forceinline__ double fx_leave(fx w, const FxLine& ln, int scale_e) 
 }
 // The same by the hardware conversion and an addition to the exponent, for the
 // passes whose FP64 pipe is otherwise idle (one FP64-rate operation instead of
-// about 20 integer ones; 256^3 row pass 107 -> 94 us, event-timed).  Lines whose outputs
+// about 20 integer ones; 256^3 row pass 107 -> 94 us when it was taken).  Lines whose outputs
 // could leave the normal range take fx_leave.
 template <int N, int RM>
 __device__ __forceinline__ double fx_leave_hw(fx w, const FxLine& ln, int scale_e) {
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(kFxThreads, 3)
 // its own line exponents.  MIRROR (3D): the two lines of a thread's pair mirror each
 // other in y (y and ny - y; lines 0 and ny / 2, which mirror themselves, make one
 // pair), so that mu and the reciprocal of the symbol are formed once for two modes:
-// the FP64 pipe, with 10 (order 4) and 15 (order 6) operations a mode at 1.74 per
+// the FP64 pipe, with 11 (order 4) and 16 (order 6) operations a mode at 1.74 per
 // clock and SM, was 50 to 80% of the pass.  Otherwise they are x and x + 1.
 template <int N, int RM, int ORDER, bool MIRROR>
 __global__ void __launch_bounds__(kFxThreads, 2)
@@ -552,8 +552,8 @@ __global__ void __launch_bounds__(kFxThreads, 2)
 // would leave SMs without a block (down to one warp; strided passes keep two
 // pairs, whole 32-byte sectors).  total: line pairs of the pass.  On a 64^2 grid
 // (eight blocks of one warp instead of one of 256 threads, on one SM) a row pass
-// takes 8.6 us instead of 21 and the middle pass 26 instead of 59, fixed point
-// and narrowing together.
+// takes 7.6 us instead of 21 and the middle pass 15.5 instead of 59, fixed point,
+// narrowing and radix 4 together.
 template <int N, int RM, bool ROWS>
 int fx_pairs(long long total, int avail, int nsm) {
   constexpr int TS = LineFFT<fx, N, RM>::TS;
@@ -636,7 +636,8 @@ cudaError_t mid_fx_launch(double* data, const KParams& kp, Ctrl* ctrl, double* p
 }
 // Mirrored pairs of lines where a block reads whole 32-byte sectors of a row (four
 // columns; shorter blocks are those of 1024-point lines and of the smallest grids).
-// Solve of L_h at 256x128x64, order 4: 150 -> 137 us; middle pass of order 6 at 256^3: 627 -> 599 us.
+// Solve of L_h at 64x256x128, order 4: 156 -> 142 us; middle pass of order 6 at 256^3: 582 -> 534 us,
+// of order 4 at 128^3: 92 -> 76.5 us.
 // In 2D, where x is the axis to mirror, it loses: the rows' sectors are split between
 // blocks (1024^2, order 6, whole solve of L_h: 107 us adjacent, 127 us mirrored).
 template <int N, int RM>

@@ -40,7 +40,11 @@ constexpr int kChunk = 8;          // iterations enqueued between host checks (d
 constexpr int kBody = 2;           // iterations per WHILE-loop body of a captured solve
 static_assert(kBody % 2 == 0, "a loop body must start and end on the same ping-pong parity");
 constexpr int kCapDepth = 3;       // nesting of WHILE loops: outer, inner, general-p line search
-constexpr size_t kFxScanCells = 1 << 18;  // grids from here on scan u for the fixed-point residual's scales
+// Grids from here on scan u for the scales of a fixed-point residual.  Residual calls with the
+// scan and without (FP64 variant), smooth fields: 2D 128^2 35 and 31 us, 256^2 38 and 42, 2^17
+// cells 44.5 and 45.5, 512^2 45 and 55; 3D 32^3 57 and 72, 64^3 57 and 73.  A rough field pays the
+// scan for nothing (512^2 2 us, 128^3 15 us).  3D grids of 2^15 cells would gain as well.
+constexpr size_t kFxScanCells = 1 << 18;
 constexpr int kSolveGraphs = 4;    // solve graphs cached per handle (by pointer set)
 static_assert(kChunk % 2 == 0, "a chunk must start and end on the same ping-pong parity");
 constexpr int kLsPassesGen = 16;   // Newton passes of the general-p line search

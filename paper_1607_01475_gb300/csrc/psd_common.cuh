@@ -60,7 +60,7 @@ struct Ctrl {
   int cfg_pad_;
   double last_alpha;
   unsigned int counter[CS_COUNT];
-  // FP64 p = 4 stencils in 3D (fixed-point variants): bounds on |u| and on the
+  // FP64 p = 4 stencils (fixed-point variants): bounds on |u| and on the
   // vertex gradient sums |G| of the last residual's iterate (umax < 0: none),
   // the high word of a bound on |d| (the x pass that ends the preconditioner),
   // the scales of the next residual (fx_s = kFxOff: the FP64 variant), and

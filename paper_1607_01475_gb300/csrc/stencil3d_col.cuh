@@ -65,7 +65,7 @@ struct ResColSmem {
 // of the FP64 Laplacian sums it replaces; the variant runs when the flux part's
 // worst-case error is below those roundings too (fx_decide).  FP64 issues at
 // 1/64 of the FP32 rate: at 256^3 the all-FP64 kernel takes 1.88 ms, this one
-// 0.51 ms (0.57 with the maximum as an FP64 comparison and four operations in r).
+// 0.53 ms (0.57 with the maximum as an FP64 comparison and four operations in r).
 //
 // TRACK (both variants of that case): the largest |u| and |G| of the new
 // iterate go to ctrl for the next scales.

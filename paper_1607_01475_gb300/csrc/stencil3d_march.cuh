@@ -20,9 +20,9 @@
 // The kernels are bound by instruction issue (about 190 instructions per cell in
 // the residual, with 20% of the lanes outside the grid at nx = 256).  Grids with at
 // least 2 x 152 tiles of 32 x 32 x 16 cells take the shared-memory kernels of
-// stencil3d_rb.cuh, whose tiles waste no lanes (256^3 residual: 142 us there, 160
-// here); on smaller grids these replace the 32 x 8 column tiles and the general
-// tiles (128^3, event-timed: residual 46 -> 31 us, line search 27 -> 20 us).  One
+// stencil3d_rb.cuh, whose tiles waste no lanes (256^3 residual: 132 us there, 156
+// here; line search 65.5 and 67); on smaller grids these replace the 32 x 8 column tiles and the general
+// tiles (128^3, traced launches: residual 46 -> 27.5 us, line search 27 -> 19 us).  One
 // wave of CTAs takes equal shares of the (column, plane) pairs, a column being a
 // strip of the CTA's warps, four rows each, one below the other, which share
 // their halo rows in L1.
